@@ -1,5 +1,7 @@
 // Layout conversions between the C-ABI's lexicographic complex128 arrays and the
 // internal line layout, gauge ingest, and the per-line wrap-around matrices Lambda.
+#include <algorithm>
+
 #include "wf_internal.h"
 
 namespace wf {
@@ -21,162 +23,373 @@ __device__ __forceinline__ void site_coords(const Geom& g, size_t site, int& x, 
   t = (int)(r / g.L);
 }
 
-// gamma_5 = -[[0, 1], [1, 0]] in the Dirac-Pauli basis: spin s <- -(spin s +- 2).
-// Optional colour rotation per site (axial frame): import psi' = g psi, export psi = g^dag psi'.
-// g (if not null) is given per parity as [l][9][tp] in FP64.
-__device__ __forceinline__ void rotate3(const Cx<double>* __restrict__ gl, int tp, int sl, bool dag, Cx<double> (&v)[3]) {
-  Mat3<double> G;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) G.e[k] = gl[k * tp + sl];
-  Vec3<double> x;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) x.c[k] = v[k];
-  Vec3<double> y = dag ? matvec_dag(G, x) : matvec(G, x);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) v[k] = y.c[k];
+// ----------------------------------------------------------------------------
+// Spinor import / export: between the caller's complex128 arrays, [rhs][t][z][y][x][12] (both
+// parities) or [rhs][t][l][12] (one parity, "compact"), and the line layout [rhs][l][12][slot] in
+// precision R, with the axial frame's colour rotation per site (import psi' = g psi, export
+// psi = g^dag psi') and optionally gamma_5 = -[[0, 1], [1, 0]] (spin s <- -(spin s +- 2)).
+//
+// A caller's site is 192 contiguous bytes, a layout run is consecutive slots of one component, so
+// each side wants another thread order. A CTA therefore takes a tile of `tl` lines x `J` lane
+// groups (n J consecutive times) x all 12 components through shared memory: the caller's side
+// moves as 16-byte pieces, 12 consecutive threads to a site; on the layout's side one thread holds
+// one site and consecutive threads consecutive slots (runs of J elements). The rotation of a site
+// stays in registers for all sources the CTA loops over. Shared-memory rows of 13 elements keep
+// both orders free of bank conflicts.
+//
+// The rotation's 144 multiply-adds per site bound the FP64 form (GB300: two FP64 FMAs per clock and
+// SM; 0.10 ms of an 0.08 ms floor for a full field of 12^3 x 48 x 4 sources). FP32 fields take
+// rotate3_split instead, whose products are exact FP32 ones (below). Spins one after another and six
+// CTAs per SM: the loads of one CTA overlap the arithmetic of the others (unrolled, at 4 CTAs per SM,
+// 1.4 times slower). Measured, one odd field of 24^3 x 128 x 12 sources to and from FP32 (3.1 GB,
+// 0.45 ms at the copy bandwidth): import 0.96 ms, export 0.99 ms; 6.39 and 4.34 ms with one thread
+// per spin, its scattered elements and the rotation in FP64. One source of 16^3 x 128: 43 and 37 us,
+// from 88 and 86.
+// ----------------------------------------------------------------------------
+constexpr int kTileThreads = 128;
+constexpr int kTileMinBlocks = 6;      // resident CTAs per SM
+constexpr int kTileRow = NSPIN_C + 1;  // shared-memory elements per site
+
+// Tile of an import / export launch (host: tile_of)
+struct SpinorTile {
+  int J;      // lane groups per tile (a divisor of lpl)
+  int nJ;     // times per tile, n J
+  int tl;     // lines per tile (1, 2, 4 or 8)
+  int nch;    // time chunks per line, lpl / J
+  int ntl;    // line tiles per parity
+  int rper;   // sources per CTA
+};
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+               "l"(__cvta_generic_to_global(src))
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// ---- FP32 rotation with exact products.
+// d = f + lo for a double of magnitude in [2^-80, 2^100) or zero, by integer operations (the
+// conversions between FP64 and FP32 run at the FP64 rate): f its sign, exponent and leading 20
+// fraction bits, lo the next 23. Returns false (f, lo unset) outside that range.
+__device__ __forceinline__ bool split_double(double d, float& f, float& lo) {
+  const unsigned hw = (unsigned)__double2hiint(d), lw = (unsigned)__double2loint(d);
+  const unsigned a = hw & 0x7fffffffu, sg = hw & 0x80000000u;
+  const bool zero = (a | lw) == 0;
+  if (!zero && a - (943u << 20) >= (180u << 20)) return false;
+  const float sc = __uint_as_float(sg | (((a >> 20) - 939u) << 23));
+  f = zero ? 0.f : __uint_as_float(sg | ((a - 0x38000000u) << 3));
+  lo = zero ? 0.f : (__uint_as_float(0x4b000000u | (lw >> 9)) - 8388608.f) * sc;
+  return true;
+}
+// exact FP64 value of a finite float by integer operations; subnormal values give zero
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), a = b & 0x7fffffffu;
+  const bool z = a < 0x00800000u;
+  return __hiloint2double(z ? 0 : (int)((b & 0x80000000u) | ((a >> 3) + 0x38000000u)), z ? 0 : (int)(b << 29));
 }
 
-// One thread per (rhs, parity, line, slot): all four spins of the site, so that the stores (import)
-// and loads (export) of the line layout are coalesced over the slots, the rotation g is loaded
-// once per site, and the lexicographic side moves each site's 192 contiguous bytes. Padding
-// slots (t >= T) are written as zero on import.
-__device__ __forceinline__ int slot_time(const Geom& g, int sl) { return (sl % g.lpl) * g.n + sl / g.lpl; }
+// A rotation matrix split as h + l, h a multiple of 2^-10 (|g| <= 1: 11 bits)
+struct SplitMat {
+  Cx<float> h[9], l[9];
+};
+__device__ __forceinline__ void split_unit(double g, float& h, float& l) {
+  float f, lo;
+  if (!split_double(g, f, lo)) f = lo = 0.f;  // below 2^-80
+  h = (f + 12288.f) - 12288.f;
+  l = (f - h) + lo;
+}
+__device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl, int tp, int sl, SplitMat& G) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const Cx<double> e = gl[(size_t)k * tp + sl];
+    split_unit(e.re, G.h[k].re, G.l[k].re);
+    split_unit(e.im, G.h[k].im, G.l[k].im);
+  }
+}
+__device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl, int tp, int sl, Mat3<double>& G) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) G.e[k] = gl[(size_t)k * tp + sl];
+}
 
-template <typename R>
-__global__ void k_import_spinor(const Geom g, const Cx<double>* __restrict__ lex, Cx<R>* even, Cx<R>* odd, int nrhs,
-                                int g5, const Cx<double>* g_e, const Cx<double>* g_o) {
-  const size_t V = (size_t)g.L * g.L * g.L * g.T;
-  const size_t per_p = (size_t)g.Nl * g.tp;
-  const size_t total = (size_t)nrhs * 2 * per_p;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int sl = (int)(i % g.tp);
-    const int l = (int)((i / g.tp) % g.Nl);
-    const int p = (int)((i / per_p) % 2);
-    const int rhs = (int)(i / (2 * per_p));
-    Cx<R>* dst = p ? odd : even;
-    if (!dst) continue;
-    Cx<R>* out = dst + (size_t)(rhs * g.Nl + l) * NSPIN_C * g.tp + sl;
-    const int t = slot_time(g, sl);
-    if (t >= g.T) {
+// s + c = g v (DAG: g^dag v) for a vector v = f + lo (lo of relative size 2^-20 at most, or zero):
+// f is split again at 2^-10 of the vector's largest exponent, so that each h-h product is an
+// integer multiple of one power of two that fits FP32 and their sums are exact; the other
+// products, 2^-10 of those, are summed in FP32. The error is about 2^-34 of |v|, against
+// 2^-25 for the rounding of an FP32 result.
+template <bool DAG>
+__device__ __forceinline__ void rotate3_split(const SplitMat& G, const float (&f)[6], const float (&lo)[6],
+                                              float (&s)[6], float (&c)[6]) {
+  unsigned e = 0;
 #pragma unroll
-      for (int k = 0; k < NSPIN_C; ++k) out[(size_t)k * g.tp] = mk<R>(R(0), R(0));
-      continue;
+  for (int i = 0; i < 6; ++i) e = max(e, __float_as_uint(f[i]) & 0x7f800000u);
+  const float M = e ? __uint_as_float(e + (13u << 23) + 0x00400000u) : 0.f;  // 1.5 x 2^(E + 13)
+  float vh[6], vl[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    vh[i] = __fadd_rn(__fadd_rn(f[i], M), -M);
+    vl[i] = (f[i] - vh[i]) + lo[i];
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float sr = 0.f, si = 0.f, cr = 0.f, ci = 0.f;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const Cx<float> H = DAG ? G.h[3 * b + a] : G.h[3 * a + b], L = DAG ? G.l[3 * b + a] : G.l[3 * a + b];
+      const float hi = DAG ? -H.im : H.im, li = DAG ? -L.im : L.im;
+      sr = fmaf(H.re, vh[2 * b], sr);
+      sr = fmaf(-hi, vh[2 * b + 1], sr);
+      si = fmaf(H.re, vh[2 * b + 1], si);
+      si = fmaf(hi, vh[2 * b], si);
+      const float xr = vh[2 * b] + vl[2 * b], xi = vh[2 * b + 1] + vl[2 * b + 1];
+      cr = fmaf(H.re, vl[2 * b], cr);
+      cr = fmaf(-hi, vl[2 * b + 1], cr);
+      cr = fmaf(L.re, xr, cr);
+      cr = fmaf(-li, xi, cr);
+      ci = fmaf(H.re, vl[2 * b + 1], ci);
+      ci = fmaf(hi, vl[2 * b], ci);
+      ci = fmaf(L.re, xi, ci);
+      ci = fmaf(li, xr, ci);
     }
-    int x, y, z;
-    line_coords(g, p, l, x, y, z);
-    const size_t site = (size_t)x + g.L * ((size_t)y + g.L * ((size_t)z + (size_t)g.L * t));
-    const Cx<double>* src = lex + ((size_t)rhs * V + site) * NSPIN_C;
-    const Cx<double>* gr = p ? g_o : g_e;
-    Mat3<double> G;
-    if (gr) {
+    s[2 * a] = sr;
+    s[2 * a + 1] = si;
+    c[2 * a] = cr;
+    c[2 * a + 1] = ci;
+  }
+}
+
+// One spin of a site on import: in (shared memory, 3 FP64 elements, negated for gamma_5) rotated by G
+// into out (components tp elements apart)
+__device__ __forceinline__ void import_spin(const Mat3<double>& G, const Cx<double>*, int, const Cx<double>* in, bool neg,
+                                            Cx<double>* out, int tp) {
+  Vec3<double> v;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) G.e[k] = gr[((size_t)l * 9 + k) * g.tp + sl];
-    }
+  for (int c = 0; c < 3; ++c) v.c[c] = neg ? mk<double>(-in[c].re, -in[c].im) : in[c];
+  const Vec3<double> w = matvec(G, v);
 #pragma unroll
-    for (int sp = 0; sp < 4; ++sp) {
-      const int ssrc = g5 ? (sp + 2) % 4 : sp;
-      Vec3<double> v;
+  for (int c = 0; c < 3; ++c) out[(size_t)c * tp] = w.c[c];
+}
+// the same in FP64 for FP32 fields: extreme magnitudes, infinities, NaN (rare, kept out of line)
+__device__ __noinline__ void import_spin_wide(const Cx<double>* gl, const Cx<double>* in, bool neg, Cx<float>* out,
+                                              int tp) {
+  for (int a = 0; a < 3; ++a) {
+    Cx<double> w = czero<double>();
+    for (int b = 0; b < 3; ++b) w = cfma(w, gl[(size_t)(3 * a + b) * tp], neg ? mk<double>(-in[b].re, -in[b].im) : in[b]);
+    out[(size_t)a * tp] = mk<float>((float)w.re, (float)w.im);
+  }
+}
+__device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>* gl, int sl, const Cx<double>* in,
+                                            bool neg, Cx<float>* out, int tp) {
+  float f[6], lo[6];
+  bool ok = true;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) v.c[c] = g5 ? mk<double>(-src[ssrc * 3 + c].re, -src[ssrc * 3 + c].im) : src[ssrc * 3 + c];
-      if (gr) v = matvec(G, v);
+  for (int k = 0; k < 3; ++k) {
+    const Cx<double> v = in[k];
+    ok &= split_double(neg ? -v.re : v.re, f[2 * k], lo[2 * k]);
+    ok &= split_double(neg ? -v.im : v.im, f[2 * k + 1], lo[2 * k + 1]);
+  }
+  if (!ok) {
+    import_spin_wide(gl + sl, in, neg, out, tp);
+    return;
+  }
+  float s[6], c[6];
+  rotate3_split<false>(G, f, lo, s, c);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) out[(size_t)(sp * 3 + c) * g.tp] = mk<R>((R)v.c[c].re, (R)v.c[c].im);
-    }
+  for (int k = 0; k < 3; ++k) out[(size_t)k * tp] = mk<float>(s[2 * k] + c[2 * k], s[2 * k + 1] + c[2 * k + 1]);
+}
+// One spin of a site on export: v rotated by G^dag into out (shared memory, 3 FP64 elements)
+__device__ __forceinline__ void export_spin(const Mat3<double>& G, const Cx<double>*, int, int, const Vec3<double>& v,
+                                            bool neg, Cx<double>* out) {
+  const Vec3<double> w = matvec_dag(G, v);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[c] = neg ? mk<double>(-w.c[c].re, -w.c[c].im) : w.c[c];
+}
+__device__ __noinline__ void export_spin_wide(const Cx<double>* gl, int tp, Vec3<float> v, bool neg, Cx<double>* out) {
+  for (int a = 0; a < 3; ++a) {
+    Cx<double> w = czero<double>();
+    for (int b = 0; b < 3; ++b)
+      w = cfmaconj(w, gl[(size_t)(3 * b + a) * tp], mk<double>((double)v.c[b].re, (double)v.c[b].im));
+    out[a] = neg ? mk<double>(-w.re, -w.im) : w;
+  }
+}
+__device__ __forceinline__ void export_spin(const SplitMat& G, const Cx<double>* gl, int tp, int sl,
+                                            const Vec3<float>& v, bool neg, Cx<double>* out) {
+  float f[6];
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    f[k] = k & 1 ? v.c[k >> 1].im : v.c[k >> 1].re;
+    const unsigned a = __float_as_uint(f[k]) & 0x7fffffffu;
+    ok &= a == 0 || (a >= (47u << 23) && a < (227u << 23));  // [2^-80, 2^100)
+  }
+  if (!ok) {
+    export_spin_wide(gl + sl, tp, v, neg, out);
+    return;
+  }
+  const float lo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  float s[6], c[6];
+  rotate3_split<true>(G, f, lo, s, c);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const double w = widen(neg ? -s[k] : s[k]) + widen(neg ? -c[k] : c[k]);
+    if (k & 1)
+      out[k >> 1].im = w;
+    else
+      out[k >> 1].re = w;
   }
 }
 
 template <typename R>
-__global__ void k_export_spinor(const Geom g, const Cx<R>* even, const Cx<R>* odd, Cx<double>* __restrict__ lex,
-                                int nrhs, int g5, const Cx<double>* g_e, const Cx<double>* g_o) {
-  const size_t V = (size_t)g.L * g.L * g.L * g.T;
-  const size_t per_p = (size_t)g.Nl * g.tp;
-  const size_t total = (size_t)nrhs * 2 * per_p;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int sl = (int)(i % g.tp);
-    const int l = (int)((i / g.tp) % g.Nl);
-    const int p = (int)((i / per_p) % 2);
-    const int rhs = (int)(i / (2 * per_p));
-    const int t = slot_time(g, sl);
-    if (t >= g.T) continue;
-    int x, y, z;
-    line_coords(g, p, l, x, y, z);
-    const size_t site = (size_t)x + g.L * ((size_t)y + g.L * ((size_t)z + (size_t)g.L * t));
-    Cx<double>* dst = lex + ((size_t)rhs * V + site) * NSPIN_C;
-    const Cx<R>* src = p ? odd : even;
-    if (!src) {
-#pragma unroll
-      for (int k = 0; k < NSPIN_C; ++k) dst[k] = mk<double>(0.0, 0.0);
-      continue;
-    }
-    const Cx<R>* in = src + (size_t)(rhs * g.Nl + l) * NSPIN_C * g.tp + sl;
-    const Cx<double>* gr = p ? g_o : g_e;
-    Mat3<double> G;
-    if (gr) {
-#pragma unroll
-      for (int k = 0; k < 9; ++k) G.e[k] = gr[((size_t)l * 9 + k) * g.tp + sl];
-    }
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp) {
-      const int ss = g5 ? (sp + 2) % 4 : sp;
-      Vec3<double> v;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const Cx<R> w = in[(size_t)(ss * 3 + c) * g.tp];
-        v.c[c] = mk<double>((double)w.re, (double)w.im);
+struct RotationOf {
+  typedef SplitMat type;
+};
+template <>
+struct RotationOf<double> {
+  typedef Mat3<double> type;
+};
+
+// Block and thread of a tile launch -> parity, lines and times. Caller's side: thread q < 96 moves
+// component q % 12 of the tile's sites s = q / 12, s + 8, ..., site s = tt tl + li; layout's side:
+// thread k + (128 / SPL) h holds spins h, h + SPL, .. of row k: line li = k / nJ, slot m lpl + j0 + jj with
+// (m, jj) = (k % nJ) / J, % J. SPL = 1 (a thread holds the site), or 4 where the lattice is so small
+// that the rotation's serial chain, not the memory, is what a launch waits for.
+struct TileAt {
+  int p, l0, j0, r0, r1;
+  __device__ __forceinline__ TileAt(const Geom& g, const SpinorTile& t, int npar, int nrhs) {
+    int b = blockIdx.x;
+    p = npar == 2 ? b & 1 : 0;
+    b /= npar;
+    l0 = (b % t.ntl) * t.tl;
+    j0 = (b / t.ntl) * t.J;
+    r0 = blockIdx.y * t.rper;
+    r1 = min(nrhs, r0 + t.rper);
+  }
+};
+// element offset of line l's site at t = 0 in the caller's array (add t * stride)
+__device__ __forceinline__ size_t caller_site(const Geom& g, int compact, int p, int l) {
+  if (compact) return (size_t)l;
+  int x, y, z;
+  line_coords(g, p, l, x, y, z);
+  return (size_t)x + g.L * ((size_t)y + (size_t)g.L * z);
+}
+
+template <typename R, int SPL>
+__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_import_spinor(const Geom g, const SpinorTile t, int compact,
+                                                                const Cx<double>* __restrict__ lex, Cx<R>* even,
+                                                                Cx<R>* odd, int nrhs, int g5, const Cx<double>* g_e,
+                                                                const Cx<double>* g_o) {
+  __shared__ __align__(16) Cx<double> buf[kTileThreads / SPL * kTileRow];
+  const TileAt at(g, t, compact ? 1 : 2, nrhs);
+  Cx<R>* dst = at.p ? odd : even;
+  if (!dst) return;
+  const Cx<double>* gr = at.p ? g_o : g_e;
+  const int q = threadIdx.x;
+  const size_t ts = compact ? (size_t)g.Nl : (size_t)g.L * g.L * g.L;  // sites per time slice of the caller's array
+  // layout's side
+  const int row = q % (kTileThreads / SPL), sp0 = q / (kTileThreads / SPL);
+  const int li = row / t.nJ, mj = row - li * t.nJ, m = mj / t.J, jj = mj - m * t.J;
+  const int l = at.l0 + li, sl = m * g.lpl + at.j0 + jj;
+  const bool mine = li < t.tl && l < g.Nl;
+  const bool valid = mine && (at.j0 + jj) * g.n + m < g.T;
+  typename RotationOf<R>::type G;
+  const Cx<double>* gl = gr ? gr + (size_t)l * 9 * g.tp : nullptr;
+  if (valid && gr) load_rotation(gl, g.tp, sl, G);
+  // caller's side
+  const int cc = q % 12, cs = q / 12, cli = cs & (t.tl - 1), step = 8 / t.tl;
+  const bool mover = q < 96 && at.l0 + cli < g.Nl;
+  const size_t csite = mover ? caller_site(g, compact, at.p, at.l0 + cli) : 0;
+
+  for (int rhs = at.r0; rhs < at.r1; ++rhs) {
+    if (mover) {
+      const Cx<double>* src = lex + ((size_t)rhs * g.T * ts + csite) * NSPIN_C + cc;
+      for (int tt = cs / t.tl; tt < t.nJ; tt += step) {
+        const int time = at.j0 * g.n + tt;
+        if (time >= g.T) break;
+        const int j = tt / g.n;
+        const int to = (cli * g.n + (tt - j * g.n)) * t.J + j;  // its row
+        cp_async16(&buf[to * kTileRow + cc], src + (size_t)time * ts * NSPIN_C);
       }
-      if (gr) v = matvec_dag(G, v);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) dst[sp * 3 + c] = g5 ? mk<double>(-v.c[c].re, -v.c[c].im) : v.c[c];
     }
+    cp_async_wait_all();
+    __syncthreads();
+    if (mine) {
+      Cx<R>* out = dst + ((size_t)rhs * g.Nl + l) * NSPIN_C * g.tp + sl;
+#pragma unroll 1
+      for (int i = 0; i < 4 / SPL; ++i) {
+        const int sp = sp0 + i * SPL;
+        Cx<R>* o = out + (size_t)sp * 3 * g.tp;
+        const Cx<double>* in = buf + row * kTileRow + (g5 ? (sp + 2) % 4 : sp) * 3;
+        if (valid && gr) {
+          import_spin(G, gl, sl, in, g5 != 0, o, g.tp);
+        } else {  // the caller's gauge, or padding slots: zero
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const Cx<double> v = valid ? in[c] : czero<double>();
+            o[(size_t)c * g.tp] = g5 ? mk<R>((R)-v.re, (R)-v.im) : mk<R>((R)v.re, (R)v.im);
+          }
+        }
+      }
+    }
+    __syncthreads();
   }
 }
 
-// compact half-lattice array of one parity: [rhs][t][l][12] (sites in lexicographic order)
-template <typename R>
-__global__ void k_import_compact(const Geom g, const Cx<double>* __restrict__ cmp, Cx<R>* half, int nrhs, int g5,
-                                 const Cx<double>* gr) {
-  const size_t total = (size_t)nrhs * g.T * g.Nl * 4;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int sp = (int)(i % 4);
-    const size_t k = i / 4;
-    const int l = (int)(k % g.Nl);
-    const int t = (int)((k / g.Nl) % g.T);
-    const int rhs = (int)(k / ((size_t)g.Nl * g.T));
-    const int ssrc = g5 ? (sp + 2) % 4 : sp;
-    const Cx<double>* src = cmp + k * NSPIN_C + ssrc * 3;
-    Cx<double> v[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) v[c] = g5 ? mk<double>(-src[c].re, -src[c].im) : src[c];
-    const int sl = slot_of(g, t);
-    if (gr) rotate3(gr + (size_t)l * 9 * g.tp, g.tp, sl, false, v);
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-      half[((size_t)(rhs * g.Nl + l) * NSPIN_C + sp * 3 + c) * g.tp + sl] = mk<R>((R)v[c].re, (R)v[c].im);
-  }
-}
+template <typename R, int SPL>
+__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_export_spinor(const Geom g, const SpinorTile t, int compact,
+                                                                const Cx<R>* even, const Cx<R>* odd,
+                                                                Cx<double>* __restrict__ lex, int nrhs, int g5,
+                                                                const Cx<double>* g_e, const Cx<double>* g_o) {
+  __shared__ __align__(16) Cx<double> buf[kTileThreads / SPL * kTileRow];
+  const TileAt at(g, t, compact ? 1 : 2, nrhs);
+  const Cx<R>* src = at.p ? odd : even;  // null: that parity's sites are zero
+  const Cx<double>* gr = at.p ? g_o : g_e;
+  const int q = threadIdx.x;
+  const size_t ts = compact ? (size_t)g.Nl : (size_t)g.L * g.L * g.L;
+  const int row = q % (kTileThreads / SPL), sp0 = q / (kTileThreads / SPL);
+  const int li = row / t.nJ, mj = row - li * t.nJ, m = mj / t.J, jj = mj - m * t.J;
+  const int l = at.l0 + li, sl = m * g.lpl + at.j0 + jj;
+  const bool valid = li < t.tl && l < g.Nl && (at.j0 + jj) * g.n + m < g.T;
+  typename RotationOf<R>::type G;
+  const Cx<double>* gl = gr ? gr + (size_t)l * 9 * g.tp : nullptr;
+  if (valid && gr && src) load_rotation(gl, g.tp, sl, G);
+  const int cc = q % 12, cs = q / 12, cli = cs & (t.tl - 1), step = 8 / t.tl;
+  const bool mover = q < 96 && at.l0 + cli < g.Nl;
+  const size_t csite = mover ? caller_site(g, compact, at.p, at.l0 + cli) : 0;
 
-template <typename R>
-__global__ void k_export_compact(const Geom g, const Cx<R>* half, Cx<double>* __restrict__ cmp, int nrhs, int g5,
-                                 const Cx<double>* gr) {
-  const size_t total = (size_t)nrhs * g.T * g.Nl * 4;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int sp = (int)(i % 4);
-    const size_t k = i / 4;
-    const int l = (int)(k % g.Nl);
-    const int t = (int)((k / g.Nl) % g.T);
-    const int rhs = (int)(k / ((size_t)g.Nl * g.T));
-    const int ss = g5 ? (sp + 2) % 4 : sp;
-    const int sl = slot_of(g, t);
-    Cx<double> v[3];
+  for (int rhs = at.r0; rhs < at.r1; ++rhs) {
+    if (valid) {
+      const Cx<R>* in = src ? src + ((size_t)rhs * g.Nl + l) * NSPIN_C * g.tp + sl : nullptr;
+#pragma unroll 1
+      for (int i = 0; i < 4 / SPL; ++i) {
+        const int sp = sp0 + i * SPL, ss = g5 ? (sp + 2) % 4 : sp;
+        Cx<double>* out = buf + row * kTileRow + sp * 3;
+        Vec3<R> v = {};
+        if (src) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      Cx<R> w = half[((size_t)(rhs * g.Nl + l) * NSPIN_C + ss * 3 + c) * g.tp + sl];
-      v[c] = mk<double>((double)w.re, (double)w.im);
+          for (int c = 0; c < 3; ++c) v.c[c] = in[(size_t)(ss * 3 + c) * g.tp];
+        }
+        if (src && gr) {
+          export_spin(G, gl, g.tp, sl, v, g5 != 0, out);
+        } else {
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const Cx<double> w = mk<double>((double)v.c[c].re, (double)v.c[c].im);
+            out[c] = g5 ? mk<double>(-w.re, -w.im) : w;
+          }
+        }
+      }
     }
-    if (gr) rotate3(gr + (size_t)l * 9 * g.tp, g.tp, sl, true, v);
-    Cx<double>* dst = cmp + k * NSPIN_C + sp * 3;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) dst[c] = g5 ? mk<double>(-v[c].re, -v[c].im) : v[c];
+    __syncthreads();
+    if (mover) {
+      Cx<double>* dst = lex + ((size_t)rhs * g.T * ts + csite) * NSPIN_C + cc;
+      for (int tt = cs / t.tl; tt < t.nJ; tt += step) {
+        const int time = at.j0 * g.n + tt;
+        if (time >= g.T) break;
+        const int j = tt / g.n;
+        const int from = (cli * g.n + (tt - j * g.n)) * t.J + j;
+        dst[(size_t)time * ts * NSPIN_C] = buf[from * kTileRow + cc];
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -329,33 +542,75 @@ static int grid_for(size_t n) {
   return b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b);
 }
 
+// Tile of an import / export over npar parities: about 32 times (runs of 4 to 32 slots) of up to 8
+// lines, 128 sites at most; 32 sites with four threads each where that leaves fewer than two CTAs per
+// SM (then as few as one line), and all sources of a tile in one CTA (its rotation is then read
+// once) only where the tiles alone fill the chip
+static SpinorTile tile_of(const Geom& g, int npar, int nrhs, dim3& grid, bool& split) {
+  SpinorTile t;
+  t.J = g.n == 1 ? 32 : g.n == 2 ? 16 : g.n <= 4 ? 8 : 4;
+  if (t.J > g.lpl) t.J = g.lpl;
+  t.nJ = g.n * t.J;
+  t.nch = g.lpl / t.J;
+  auto lines = [&](int sites) {
+    t.tl = 8;
+    while (t.tl > 1 && t.tl * t.nJ > sites) t.tl >>= 1;
+    t.ntl = (g.Nl + t.tl - 1) / t.tl;
+    return (long long)npar * t.ntl * t.nch;
+  };
+  long long blocks = lines(kTileThreads);
+  split = blocks * nrhs < 2 * 152;
+  if (split) blocks = lines(kTileThreads / 4);
+  long long rgroups = std::min<long long>(nrhs, (8 * 152 + blocks - 1) / blocks);
+  t.rper = (int)((nrhs + rgroups - 1) / rgroups);
+  grid = dim3((unsigned)blocks, (unsigned)((nrhs + t.rper - 1) / t.rper));
+  return t;
+}
+
+template <typename R>
+static void launch_import_tiles(const Geom& g, int compact, const Cx<double>* in, Cx<R>* even, Cx<R>* odd, int nrhs,
+                                int g5, const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
+  dim3 grid;
+  bool split;
+  const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, grid, split);
+  if (split)
+    k_import_spinor<R, 4><<<grid, kTileThreads, 0, s>>>(g, t, compact, in, even, odd, nrhs, g5, g_e, g_o);
+  else
+    k_import_spinor<R, 1><<<grid, kTileThreads, 0, s>>>(g, t, compact, in, even, odd, nrhs, g5, g_e, g_o);
+  WF_CUDA(cudaGetLastError());
+}
+template <typename R>
+static void launch_export_tiles(const Geom& g, int compact, const Cx<R>* even, const Cx<R>* odd, Cx<double>* out,
+                                int nrhs, int g5, const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
+  dim3 grid;
+  bool split;
+  const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, grid, split);
+  if (split)
+    k_export_spinor<R, 4><<<grid, kTileThreads, 0, s>>>(g, t, compact, even, odd, out, nrhs, g5, g_e, g_o);
+  else
+    k_export_spinor<R, 1><<<grid, kTileThreads, 0, s>>>(g, t, compact, even, odd, out, nrhs, g5, g_e, g_o);
+  WF_CUDA(cudaGetLastError());
+}
+
 template <typename R>
 void launch_import_spinor(const Geom& g, const Cx<double>* lex, Cx<R>* even, Cx<R>* odd, int nrhs, int g5,
                           const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
-  const size_t n = (size_t)nrhs * 2 * g.Nl * g.tp;
-  k_import_spinor<R><<<grid_for(n), kThreads, 0, s>>>(g, lex, even, odd, nrhs, g5, g_e, g_o);
-  WF_CUDA(cudaGetLastError());
+  launch_import_tiles<R>(g, 0, lex, even, odd, nrhs, g5, g_e, g_o, s);
 }
 template <typename R>
 void launch_export_spinor(const Geom& g, const Cx<R>* even, const Cx<R>* odd, Cx<double>* lex, int nrhs, int g5,
                           const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
-  const size_t n = (size_t)nrhs * 2 * g.Nl * g.tp;
-  k_export_spinor<R><<<grid_for(n), kThreads, 0, s>>>(g, even, odd, lex, nrhs, g5, g_e, g_o);
-  WF_CUDA(cudaGetLastError());
+  launch_export_tiles<R>(g, 0, even, odd, lex, nrhs, g5, g_e, g_o, s);
 }
 template <typename R>
 void launch_import_compact(const Geom& g, const Cx<double>* cmp, Cx<R>* half, int nrhs, int g5,
                            const Cx<double>* gr, cudaStream_t s) {
-  size_t n = (size_t)nrhs * g.T * g.Nl * 4;
-  k_import_compact<R><<<grid_for(n), kThreads, 0, s>>>(g, cmp, half, nrhs, g5, gr);
-  WF_CUDA(cudaGetLastError());
+  launch_import_tiles<R>(g, 1, cmp, half, nullptr, nrhs, g5, gr, nullptr, s);
 }
 template <typename R>
 void launch_export_compact(const Geom& g, const Cx<R>* half, Cx<double>* cmp, int nrhs, int g5,
                            const Cx<double>* gr, cudaStream_t s) {
-  size_t n = (size_t)nrhs * g.T * g.Nl * 4;
-  k_export_compact<R><<<grid_for(n), kThreads, 0, s>>>(g, half, cmp, nrhs, g5, gr);
-  WF_CUDA(cudaGetLastError());
+  launch_export_tiles<R>(g, 1, half, nullptr, cmp, nrhs, g5, gr, nullptr, s);
 }
 #define WF_INST(R)                                                                                          \
   template void launch_import_spinor<R>(const Geom&, const Cx<double>*, Cx<R>*, Cx<R>*, int, int,             \
