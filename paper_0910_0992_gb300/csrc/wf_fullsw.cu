@@ -35,14 +35,14 @@
 // with partial pivoting in shared memory, then the twelve columns of T_0^-1 V by the sweeps (one
 // 16-lane group per column, the forward sweep's z in a global scratch array), kept as Z, then
 // Lambda.
-// k_qinv_apply: one 16-lane group per (line, right-hand side), lane r < 12 holding component
-// r (= 3 spin + colour) of the current 12-vector; a sweep step is a 12x12 (6x12 in the forward
-// sweep) product whose vector the group exchanges through shared memory; the correction chi - Z c
-// has no serial chain. Lane r only ever needs
-// row r of a block, so it streams its rows (and b_t) into a per-group ring in shared memory with
-// cp.async several steps ahead of their use: the sweeps' serial chains then wait on shared memory
-// and arithmetic, not on DRAM. Blocks are stored row-major per time slice, [line][t][r][k], so that
-// a lane copies its row as 16-byte pieces.
+// k_qinv_line: one warp per (line, right-hand side). The recurrences act on one spin half each, so the
+// sweeps are written as
+//   forward   c_t = Sigma_t^-1 z_t, z_t = b_t + [P_+ (x) W_{t-1}^dag] c_{t-1}    (all of c_t; its P_+ half carries on),
+//   backward  y_t = c_t + Sigma_t^-1 [P_- (x) W_t] y_{t+1}                     (the six P_- columns only),
+// and the correction chi - Z c has no serial chain. The line's 12-vectors stay in shared memory from
+// the load to the store; the block entries stream through a ring there. Sigma_t^-1 is stored as its
+// P_+ and its P_- columns, [line][2][t][12][6], so that the backward sweep streams the latter alone;
+// Z_t row-major, [line][t][12][12].
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -64,18 +64,21 @@ constexpr size_t kScratchBytes = 256u << 20;   // bound of the setup's sweep scr
 template <typename R>
 __device__ __forceinline__ Cx<R> cconj(Cx<R> a) { return mk<R>(a.re, -a.im); }
 
-// row r of the 12x12 block B (element (r, k) at B[12 r + k]) times the group's vector v
+// element (r, k) of Sigma_t^-1 in a line's array [column half][t][row][6]
+__host__ __device__ __forceinline__ size_t s_at(int T, int t, int r, int k) {
+  return ((size_t)(k >= 6 ? T : 0) + t) * 72 + 6 * r + (k >= 6 ? k - 6 : k);
+}
 template <typename R>
-__device__ __forceinline__ Cx<R> row_times(const Cx<R>* __restrict__ B, int r, const Cx<R>* v) {
+__device__ __forceinline__ Cx<R> s_row_times(const Cx<R>* __restrict__ S, int T, int t, int r, const Cx<R>* v) {
   Cx<R> acc = czero<R>();
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc = cfma(acc, B[12 * r + k], v[k]);
+  for (int k = 0; k < 12; ++k) acc = cfma(acc, S[s_at(T, t, r, k)], v[k]);
   return acc;
 }
 
 // One solve T_0 y = b on one line by a 16-lane group, as the setup runs it for the columns of V
 // (the apply kernel has its own sweeps, fed ahead through shared memory): lane r < 12 holds
-// component r, lanes 12-15 only join the group's barriers (mask). S: the line's Sigma_t^-1 blocks [T][144]; ut: the line's
+// component r, lanes 12-15 only join the group's barriers (mask). S: the line's Sigma_t^-1 blocks (s_at); ut: the line's
 // U_t [9][tp] (general frame; unused in the axial frame, where W_t = 1). rhs(t): component r of
 // b_t; zst / zld: store / load component r of the forward sweep's z_t; out(t, y): component r of
 // y_t, produced for t = N_t - 1 down to 0. sh: the group's 16-element exchange vector.
@@ -90,7 +93,7 @@ __device__ __forceinline__ void t0_solve(const Cx<R>* __restrict__ S, const Cx<R
   for (int t = 1; t < T; ++t) {
     if (act) sh[r] = z;
     __syncwarp(mask);
-    const Cx<R> w = r < 6 ? row_times(S + (size_t)(t - 1) * kBlk, r, sh) : czero<R>();
+    const Cx<R> w = r < 6 ? s_row_times(S, T, t - 1, r, sh) : czero<R>();
     __syncwarp(mask);
     if (r < 6) sh[r] = w;
     __syncwarp(mask);
@@ -109,7 +112,7 @@ __device__ __forceinline__ void t0_solve(const Cx<R>* __restrict__ S, const Cx<R
   }
   if (act) sh[r] = z;
   __syncwarp(mask);
-  Cx<R> y = act ? row_times(S + (size_t)(T - 1) * kBlk, r, sh) : czero<R>();
+  Cx<R> y = act ? s_row_times(S, T, T - 1, r, sh) : czero<R>();
   if (act) out(T - 1, y);
   for (int t = T - 2; t >= 0; --t) {
     __syncwarp(mask);
@@ -128,7 +131,7 @@ __device__ __forceinline__ void t0_solve(const Cx<R>* __restrict__ S, const Cx<R
     __syncwarp(mask);
     if (act) sh[r] = v;
     __syncwarp(mask);
-    y = act ? row_times(S + (size_t)t * kBlk, r, sh) : czero<R>();
+    y = act ? s_row_times(S, T, t, r, sh) : czero<R>();
     if (act) out(t, y);
   }
   __syncwarp(mask);
@@ -188,7 +191,7 @@ struct SetupArgs {
   const Cx<R>* ut;      // general frame: U_t of the parity [Nl][9][tp]
   const Cx<R>* pl;      // axial frame: the boundary link P of every line [Nl][9]
   R s;                  // boundary sign
-  Cx<R>* sinv;          // out: Sigma_t^-1 [Nl][T][144], row-major per block
+  Cx<R>* sinv;          // out: Sigma_t^-1 [Nl][column half][T][12][6]
   Cx<R>* lam;           // out: Lambda [Nl][144], row-major
   Cx<R>* zv;            // out: Z = T_0^-1 V [Nl][T][144], row-major per time slice
   Cx<R>* scratch;       // [lines of this launch][12][T][12]: forward sweeps of the columns of V
@@ -253,7 +256,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_qinv_setup(const SetupArgs<R>
       const int r = tid / 12, k = tid - 12 * (tid / 12);
       const Cx<R> v = aug[r][k + 12];
       prev[12 * k + r] = v;
-      S[(size_t)t * kBlk + 12 * r + k] = v;
+      S[s_at(T, t, r, k)] = v;
     }
     __syncthreads();
   }
@@ -308,7 +311,7 @@ struct QinvArgs {
   const Cx<R>* xpost;  // null: out = Q^-1 in
   R apost;
   int swap_in;         // read in with the spin halves exchanged
-  const Cx<R>* sinv;   // [Nl][T][144]
+  const Cx<R>* sinv;   // [Nl][2][T][72]
   const Cx<R>* lam;    // [Nl][144]
   const Cx<R>* zv;     // Z = T_0^-1 V [Nl][T][144]
   const Cx<R>* ut;     // general frame: U_t [Nl][9][tp]
@@ -316,410 +319,336 @@ struct QinvArgs {
   R s;                 // boundary sign
 };
 
-// per-lane asynchronous global -> shared copies (completion tracked per thread in commit groups)
-template <typename R>
-__device__ __forceinline__ void cp_async(Cx<R>* dst, const Cx<R>* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
-               "l"(__cvta_generic_to_global(src)), "n"((int)sizeof(Cx<R>))
-               : "memory");
-}
-// 16 bytes: two FP32 or one FP64 complex element (both addresses 16-byte aligned), cached in L1
-// so that the sources of one line on an SM share the rows
+// 16- and 8-byte asynchronous global -> shared copies (addresses aligned to their size; completion
+// tracked per thread in commit groups)
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
                "l"(__cvta_generic_to_global(src))
                : "memory");
 }
-// elements k and k + 1 of a 16-byte aligned row in shared memory
-__device__ __forceinline__ void ld_pair(const Cx<float>* p, Cx<float>& a, Cx<float>& b) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
-  a = mk<float>(v.x, v.y);
-  b = mk<float>(v.z, v.w);
-}
-__device__ __forceinline__ void ld_pair(const Cx<double>* p, Cx<double>& a, Cx<double>& b) {
-  a = p[0];
-  b = p[1];
-}
-// lane row of 12 block elements from global src (16-byte aligned) to shared dst
-template <typename R>
-__device__ __forceinline__ void cp_row(Cx<R>* dst, const Cx<R>* src) {
-  constexpr int per = 16 / (int)sizeof(Cx<R>);
-#pragma unroll
-  for (int i = 0; i < 12; i += per) cp_async16(dst + i, src + i);
-}
-// row . v over 12 elements, two accumulators
-template <typename R>
-__device__ __forceinline__ Cx<R> row_dot(const Cx<R>* row, const Cx<R>* v) {
-  Cx<R> a0 = czero<R>(), a1 = czero<R>();
-#pragma unroll
-  for (int k = 0; k < 12; k += 2) {
-    Cx<R> m0, m1, v0, v1;
-    ld_pair(row + k, m0, m1);
-    ld_pair(v + k, v0, v1);
-    a0 = cfma(a0, m0, v0);
-    a1 = cfma(a1, m1, v1);
-  }
-  return a0 + a1;
-}
-// row . v with v in registers
-template <typename R>
-__device__ __forceinline__ Cx<R> row_dot_reg(const Cx<R>* row, const Cx<R> (&v)[12]) {
-  Cx<R> a0 = czero<R>(), a1 = czero<R>();
-#pragma unroll
-  for (int k = 0; k < 12; k += 2) {
-    Cx<R> m0, m1;
-    ld_pair(row + k, m0, m1);
-    a0 = cfma(a0, m0, v[k]);
-    a1 = cfma(a1, m1, v[k + 1]);
-  }
-  return a0 + a1;
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+               "l"(__cvta_generic_to_global(src))
+               : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-constexpr int kQGroups = 4;  // 16-lane groups per CTA of k_qinv_apply
-
-// Ring of k_qinv_apply: depth (the steps whose operands are in flight; a shallower ring with more
-// CTAs per SM measured slower) and elements per lane row (12 of a block, the step's other operand,
-// and padding that keeps rows 16-byte aligned and 16-byte row reads free of bank conflicts)
+// N consecutive elements of a row in shared memory; N even and 16-byte aligned: pairs
+template <int N>
+__device__ __forceinline__ void ld_row(const Cx<float>* p, Cx<float> (&v)[N]) {
+  if constexpr (N % 2 == 0) {
+#pragma unroll
+    for (int k = 0; k < N; k += 2) {
+      const float4 q = *reinterpret_cast<const float4*>(p + k);
+      v[k] = mk<float>(q.x, q.y);
+      v[k + 1] = mk<float>(q.z, q.w);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = p[k];
+  }
+}
+template <int N>
+__device__ __forceinline__ void ld_row(const Cx<double>* p, Cx<double> (&v)[N]) {
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k] = p[k];
+}
+// s + a . v; FP32 in two accumulators (its chain is what a step waits for), FP64 in one (bound by
+// the number of FP64 operations)
+template <typename R, int N>
+__device__ __forceinline__ Cx<R> dot(Cx<R> s, const Cx<R> (&a)[N], const Cx<R> (&v)[N]) {
+  if constexpr (sizeof(R) == 8) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) s = cfma(s, a[k], v[k]);
+    return s;
+  } else {
+    Cx<R> s1 = cmul(a[1], v[1]);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      if (k == 1) continue;
+      if (k & 1)
+        s1 = cfma(s1, a[k], v[k]);
+      else
+        s = cfma(s, a[k], v[k]);
+    }
+    return s + s1;
+  }
+}
+// the sum over a pair of lanes (2r, 2r + 1)
 template <typename R>
-struct QRing {
-  static constexpr int depth = sizeof(R) == 8 ? 4 : 6;
-  static constexpr int row = sizeof(R) == 8 ? 13 : 14;
-};
-constexpr int kTMax = 256;  // longest time line
-
-// Q^-1 per (line, right-hand side), one 16-lane group each: chi = T_0^-1 b by the two sweeps,
-// then Q^-1 b = chi - Z c with c = Lambda W^dag chi, a pass with no serial chain. Every step takes
-// lane r's row of a 12x12 block and one more operand (b_t, or the post-axpy operand) from a
-// per-group ring of D steps in shared memory that the lane fills D - 1 steps ahead with cp.async;
-// a lane reads only what it copied itself, so the ring needs no barrier. z_t and chi_t go through
-// out and come back two steps ahead of their use.
-template <typename R, bool AX>
-__global__ void __launch_bounds__(kQGroups * kGrp) k_qinv_apply(const QinvArgs<R> A) {
-  constexpr int D = QRing<R>::depth, RW = QRing<R>::row;
-  __shared__ __align__(16) Cx<R> ring[kQGroups][D][12][RW];
-  __shared__ __align__(16) Cx<R> gsh[kQGroups][kGrp];
-  __shared__ int stab[kTMax];  // slot of every time
-  const Geom& g = A.g;
-  for (int i = threadIdx.x; i < g.tp; i += blockDim.x) stab[i] = slot_of(g, i);
-  __syncthreads();
-  const int q = threadIdx.x, r = q % kGrp, gi = q / kGrp;
-  const unsigned mask = 0xFFFFu << (q & 16);
-  const size_t grp = (size_t)blockIdx.x * kQGroups + gi;
-  if (grp >= (size_t)A.nrhs * g.Nl) return;  // the group's 16 lanes leave together
-  const int l = (int)(grp / A.nrhs), k = (int)(grp % A.nrhs);
-  const int T = g.T, tp = g.tp;
-  const bool act = r < 12;
-  const int rc = act ? r : 0;  // lanes 12-15 address component 0 but never load or store
-  const int sr = rc / 3, cr = rc - 3 * (rc / 3);
-  const size_t base = ((size_t)k * g.Nl + l) * NSPIN_C * tp;
-  const Cx<R>* in = A.in + base + (size_t)(A.swap_in ? (rc + 6) % 12 : rc) * tp;
-  Cx<R>* out = A.out + base + (size_t)rc * tp;
-  const Cx<R>* xp = A.xpost ? A.xpost + base + (size_t)rc * tp : nullptr;
-  const Cx<R>* S = A.sinv + (size_t)l * T * kBlk + 12 * rc;  // lane rc's row: S[t * 144 + k]
-  const Cx<R>* Zl = A.zv + (size_t)l * T * kBlk + 12 * rc;
-  const Cx<R>* ut = AX ? nullptr : A.ut + (size_t)l * 9 * tp;
-  Cx<R>(*rg)[12][RW] = ring[gi];
-  Cx<R>* sh = gsh[gi];
-
-  // forward sweep: z_t to out
-  Cx<R> z = czero<R>();
-  {
-    auto issue = [&](int t) {  // step t: b_t, and for lanes 0-5 row rc of Sigma_{t-1}^-1
-      if (t < T && act) {
-        Cx<R>* d = rg[t % D][rc];
-        cp_async<R>(d + 12, in + stab[t]);
-        if (t >= 1 && r < 6) cp_row<R>(d, S + (size_t)(t - 1) * kBlk);
-      }
-      cp_commit();
-    };
-    for (int t = 0; t < D - 1; ++t) issue(t);
-    for (int t = 0; t < T; ++t) {
-      issue(t + D - 1);
-      cp_wait<D - 1>();
-      const Cx<R>* d = rg[t % D][rc];
-      Cx<R> b = act ? d[12] : czero<R>();
-      if (t > 0) {
-        if (act) sh[rc] = z;
-        __syncwarp(mask);
-        const Cx<R> w = r < 6 ? row_dot(d, sh) : czero<R>();
-        __syncwarp(mask);
-        if (r < 6) sh[rc] = w;
-        __syncwarp(mask);
-        if (r < 6) {
-          if (AX) {
-            b = b + sh[rc];
-          } else {  // + (W_{t-1}^dag w) on spin sr
-            const int sl = stab[t - 1];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) b = cfmaconj(b, ut[(size_t)(3 * c + cr) * tp + sl], sh[3 * sr + c]);
-          }
-        }
-        __syncwarp(mask);
-      }
-      z = b;
-      if (act) out[stab[t]] = z;
-    }
-    cp_wait<0>();
-  }
-
-  // backward sweep: chi_t to out
-  Cx<R> y0 = czero<R>(), yT = czero<R>();
-  {
-    auto issue = [&](int u) {  // step u (t = N_t - 1 - u): row rc of Sigma_t^-1
-      if (u < T && act) {
-        cp_row<R>(rg[u % D][rc], S + (size_t)(T - 1 - u) * kBlk);
-      }
-      cp_commit();
-    };
-    for (int u = 0; u < D - 1; ++u) issue(u);
-    Cx<R> zt = z;
-    Cx<R> znext = act && T >= 2 ? out[stab[T - 2]] : czero<R>();
-    Cx<R> y = czero<R>();
-    for (int u = 0; u < T; ++u) {
-      const int t = T - 1 - u;
-      issue(u + D - 1);
-      cp_wait<D - 1>();
-      const Cx<R>* d = rg[u % D][rc];
-      Cx<R> v = zt;
-      zt = znext;
-      if (act && t >= 2) znext = out[stab[t - 2]];  // used two steps on
-      if (u > 0) {  // + [P_- (x) W_t] y_{t+1}
-        if (act) sh[rc] = y;
-        __syncwarp(mask);
-        if (act && r >= 6) {
-          if (AX) {
-            v = v + sh[rc];
-          } else {
-            const int sl = stab[t];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) v = cfma(v, ut[(size_t)(3 * cr + c) * tp + sl], sh[3 * sr + c]);
-          }
-        }
-        __syncwarp(mask);
-      }
-      if (act) sh[rc] = v;
-      __syncwarp(mask);
-      y = act ? row_dot(d, sh) : czero<R>();
-      __syncwarp(mask);
-      if (act) out[stab[t]] = y;
-      if (t == 0) y0 = y;
-      if (t == T - 1) yT = y;
-    }
-    cp_wait<0>();
-  }
-
-  // c = Lambda W^dag chi (W^dag chi: the P_+ half of chi_{N_t-1}, the P_- half of chi_0)
-  if (act) sh[rc] = r < 6 ? yT : y0;
-  __syncwarp(mask);
-  Cx<R> c = czero<R>();
-  if (act) c = row_times(A.lam + (size_t)l * kBlk, rc, sh);
-  __syncwarp(mask);
-  if (act) sh[rc] = c;
-  __syncwarp(mask);
-  Cx<R> cv[12];
-#pragma unroll
-  for (int kk = 0; kk < 12; ++kk) cv[kk] = sh[kk];
-  __syncwarp(mask);
-
-  // out_t = xpost_t + apost (chi_t - Z_t c): independent steps
-  {
-    const bool post = xp != nullptr;
-    auto issue = [&](int t) {  // step t: row rc of Z_t, and xpost_t
-      if (t < T && act) {
-        Cx<R>* d = rg[t % D][rc];
-        cp_row<R>(d, Zl + (size_t)t * kBlk);
-        if (post) cp_async<R>(d + 12, xp + stab[t]);
-      }
-      cp_commit();
-    };
-    for (int t = 0; t < D - 1; ++t) issue(t);
-    Cx<R> ct = act ? out[stab[0]] : czero<R>();
-    Cx<R> cnext = act && T >= 2 ? out[stab[1]] : czero<R>();
-    for (int t = 0; t < T; ++t) {
-      issue(t + D - 1);
-      cp_wait<D - 1>();
-      const Cx<R>* d = rg[t % D][rc];
-      Cx<R> x = ct;
-      ct = cnext;
-      if (act && t + 2 < T) cnext = out[stab[t + 2]];
-      if (act) {
-        x = x - row_dot_reg(d, cv);
-        out[stab[t]] = post ? d[12] + A.apost * x : x;
-      }
-    }
-    cp_wait<0>();
-  }
-  if (act)
-    for (int t = T; t < tp; ++t) out[stab[t]] = czero<R>();  // padding slots stay zero
+__device__ __forceinline__ Cx<R> pair_sum(Cx<R> a) {
+  return mk<R>(a.re + __shfl_xor_sync(0xffffffffu, a.re, 1), a.im + __shfl_xor_sync(0xffffffffu, a.im, 1));
 }
 
-// The same Q^-1 for four or more sources: a CTA holds kQGroups consecutive sources of one line,
-// which read the same block rows, so one ring serves all its groups. The first group's lanes fill
-// it D - 1 steps ahead; a CTA barrier per step publishes a slot to every group and also tells the
-// filling lanes that the slot they refill next has been read. Each group's own operands (b_t,
-// z_t, chi_t and the post-axpy operand) come from global memory two steps ahead in registers.
-// Groups past the last source compute on zeros and store nothing, but join every barrier.
-template <typename R, bool AX>
-__global__ void __launch_bounds__(kQGroups * kGrp) k_qinv_apply_shared(const QinvArgs<R> A) {
-  constexpr int D = QRing<R>::depth, RW = QRing<R>::row;
-  __shared__ __align__(16) Cx<R> ring[D][12][RW];
-  __shared__ __align__(16) Cx<R> gsh[kQGroups][kGrp];
-  __shared__ int stab[kTMax];  // slot of every time
+constexpr int kTMax = 256;     // longest time line
+constexpr int kQMaxWarps = 4;  // sources (warps) of a CTA of k_qinv_line
+// Ring of k_qinv_line: CS time slices per chunk, NST chunks (NST - 1 in flight)
+// (16^3 x 128, us with one / twelve sources: FP32 8 x 2 136 / 1013, 4 x 3 145 / 1118, 4 x 4 139 / 1115,
+// 8 x 3 152 / 1184, 4 x 2 166 / 1127; FP64 2 x 2 1408 / 14898, 4 x 2 1320 / 16411, 2 x 3 1361 / 17273)
+template <typename R>
+struct QRing {
+  static constexpr int CS = sizeof(R) == 8 ? 2 : 8;
+  static constexpr int NST = 2;
+};
+// row stride (elements) of a line's 12 components, in time order, in shared memory: 16-byte aligned
+// rows, whose 12 lanes meet at most twice on a bank
+__host__ __device__ constexpr int line_stride(int T) { return T + 2 + (T & 1); }
+// shared memory of a CTA of G sources: ring, then per source its line and exchange vectors
+template <typename R>
+constexpr size_t qinv_smem(int T, int G) {
+  return sizeof(Cx<R>) * ((size_t)QRing<R>::NST * QRing<R>::CS * kBlk + (size_t)G * (12 * line_stride(T) + 36));
+}
+
+// n 16-byte pieces by NT threads, at most MAXN (the loop unrolls to immediate offsets)
+template <int MAXN, int NT>
+__device__ __forceinline__ void copy_pieces(void* dst, const void* src, int n) {
+  unsigned char* d = static_cast<unsigned char*>(dst) + 16 * threadIdx.x;
+  const unsigned char* s = static_cast<const unsigned char*>(src) + 16 * threadIdx.x;
+#pragma unroll
+  for (int j = 0; j < (MAXN + NT - 1) / NT; ++j)
+    if ((int)threadIdx.x + j * NT < n) cp_async16(d + 16 * NT * j, s + 16 * NT * j);
+}
+
+// Q^-1: warp w of a CTA takes source k0 + w of line l; the G warps of a CTA share the line's blocks.
+// Lane 2r + h < 24 holds columns 6h .. 6h + 5 (backward sweep: 3h .. 3h + 2 of the P_- columns) of
+// row r, the even lane component r itself: a step is three 16-byte reads of the block, three of the
+// exchanged vector, 24 multiply-adds and one pair sum, about 150 cycles of serial chain, and the
+// correction has no chain. Chunks of CS slices of the block stream (forward, backward, correction) are
+// copied 16 bytes per thread, NST - 1 chunks ahead across the three passes; the one barrier per chunk
+// publishes a chunk and frees the one before it.
+// FP32 is bound by DRAM (every block entry of the forward sweep and of Z once, the P_- columns again
+// in the backward sweep: 2880 B per site, and 192 B per source), FP64 by the FP64 pipe (78 warp
+// instructions per line and slice). Measured on 16^3 x 128, FP32 136 us with one source
+// (755 MB of block entries: 0.82 of the copy bandwidth) and 1.01 ms with twelve (the sources' reads of
+// the shared blocks bound it), FP64 1.24 and 12.6 ms. The form before (16-lane groups
+// copying their own rows, vectors through global memory in 8-byte elements a component apart) was
+// bound by the L1's tag stage: FP32 0.44 ms with one source and 2.33 ms with twelve, FP64 1.47 and
+// 13.8 ms.
+template <typename R, bool AX, int G>
+__global__ void __launch_bounds__(32 * G) k_qinv_line(const QinvArgs<R> A, int ngrp) {
+  constexpr int CS = QRing<R>::CS, NST = QRing<R>::NST;
+  constexpr int P = 72 * (int)sizeof(Cx<R>) / 16;  // 16-byte pieces of half a block
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geom& g = A.g;
-  for (int i = threadIdx.x; i < g.tp; i += blockDim.x) stab[i] = slot_of(g, i);
-  __syncthreads();
-  const int q = threadIdx.x, r = q % kGrp, gi = q / kGrp;
-  const unsigned mask = 0xFFFFu << (q & 16);
-  const int nq = (A.nrhs + kQGroups - 1) / kQGroups;
-  const int l = (int)(blockIdx.x / nq), k = (int)(blockIdx.x % nq) * kQGroups + gi;
-  const int T = g.T, tp = g.tp;
-  const bool act = r < 12;
-  const bool io = act && k < A.nrhs;   // lanes that load and store this group's source
-  const bool fill = act && gi == 0;    // lanes that fill the ring
-  const int rc = act ? r : 0;
-  const int sr = rc / 3, cr = rc - 3 * (rc / 3);
-  const size_t base = ((size_t)(k < A.nrhs ? k : 0) * g.Nl + l) * NSPIN_C * tp;
-  const Cx<R>* in = A.in + base + (size_t)(A.swap_in ? (rc + 6) % 12 : rc) * tp;
-  Cx<R>* out = A.out + base + (size_t)rc * tp;
-  const Cx<R>* xp = A.xpost ? A.xpost + base + (size_t)rc * tp : nullptr;
-  const Cx<R>* S = A.sinv + (size_t)l * T * kBlk + 12 * rc;
-  const Cx<R>* Zl = A.zv + (size_t)l * T * kBlk + 12 * rc;
+  const int T = g.T, tp = g.tp, ls = line_stride(T);
+  const int warp = G > 1 ? (int)threadIdx.x >> 5 : 0, lane = threadIdx.x & 31;
+  Cx<R>* ring = reinterpret_cast<Cx<R>*>(smem_raw);
+  Cx<R>* line = ring + NST * CS * kBlk + warp * (12 * ls + 36);
+  Cx<R>* sh = line + 12 * ls;  // two exchange vectors of 12, and 12 for the general frame
+  const int l = (int)(blockIdx.x / ngrp), k = (int)(blockIdx.x % ngrp) * G + warp;
+  const bool io = k < A.nrhs;  // a warp past the last source copies and joins the barriers only
+  const int r = lane < 24 ? lane >> 1 : 11, h = lane & 1;
+  const bool own = lane < 24 && h == 0;  // the lane of component r
+  const Cx<R>* S = A.sinv + (size_t)l * T * kBlk;
+  const Cx<R>* Z = A.zv + (size_t)l * T * kBlk;
+  const int NC = (T + CS - 1) / CS;
+  Cx<R>* mine = line + r * ls;  // component r over time: touched by its own lane only
+
+  // the line's source into shared memory, in time order
+  if (io) {
+    const Cx<R>* in = A.in + ((size_t)k * g.Nl + l) * NSPIN_C * tp;
+    for (int sl = lane; sl < tp; sl += 32) {
+      const int t = (sl % g.lpl) * g.n + sl / g.lpl;
+      if (t < T) {
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+          const Cx<R>* src = in + (size_t)(A.swap_in ? (c + 6) % 12 : c) * tp + sl;
+          if constexpr (sizeof(R) == 8)
+            cp_async16(line + c * ls + t, src);
+          else
+            cp_async8(line + c * ls + t, src);
+        }
+      }
+    }
+  }
+  cp_commit();
+
+  // the next chunk of the block stream into its ring slot: a slot holds [2][CS][72] (forward), the
+  // second half alone (backward; slices in stored order, so processed from the last), [CS][144] (Z)
+  int ip = 0, ic = 0, is = 0;  // pass, chunk of the pass, ring slot
+  auto issue = [&]() {
+    if (ip < 3) {
+      Cx<R>* dst = ring + is * CS * kBlk;
+      const int n = min(CS, T - ic * CS);
+      if (ip == 0) {
+        copy_pieces<P * CS, 32 * G>(dst, S + (size_t)ic * CS * 72, n * P);
+        copy_pieces<P * CS, 32 * G>(dst + CS * 72, S + (size_t)(T + ic * CS) * 72, n * P);
+      } else if (ip == 1) {
+        copy_pieces<P * CS, 32 * G>(dst + CS * 72, S + (size_t)(2 * T - ic * CS - n) * 72, n * P);
+      } else {
+        copy_pieces<2 * P * CS, 32 * G>(dst, Z + (size_t)ic * CS * kBlk, 2 * n * P);
+      }
+      if (++ic == NC) {
+        ic = 0;
+        ++ip;
+      }
+      if (++is == NST) is = 0;
+    }
+    cp_commit();
+  };
+  int cs = 0;  // ring slot of the next chunk to use
+  auto next_chunk = [&]() -> const Cx<R>* {
+    cp_wait<NST - 2>();
+    if (G > 1)
+      __syncthreads();
+    else
+      __syncwarp();
+    issue();
+    const Cx<R>* c = ring + cs * CS * kBlk;
+    if (++cs == NST) cs = 0;
+    return c;
+  };
+  // general frame: row r's three entries of W_t^dag (r < 6) or W_t (r >= 6)
   const Cx<R>* ut = AX ? nullptr : A.ut + (size_t)l * 9 * tp;
-  Cx<R>* sh = gsh[gi];
-  auto ld = [&](const Cx<R>* p, int t) { return io && t < T ? p[stab[t]] : czero<R>(); };
-
-  // forward sweep: z_t to out
-  Cx<R> z = czero<R>();
-  {
-    auto issue = [&](int t) {  // step t: rows 0-5 of Sigma_{t-1}^-1
-      if (fill && r < 6 && t >= 1 && t < T) cp_row<R>(ring[t % D][rc], S + (size_t)(t - 1) * kBlk);
-      if (gi == 0) cp_commit();
-    };
-    for (int t = 0; t < D - 1; ++t) issue(t);
-    Cx<R> bt = ld(in, 0), bn = ld(in, 1);
-    for (int t = 0; t < T; ++t) {
-      if (gi == 0) cp_wait<D - 2>();
-      __syncthreads();
-      issue(t + D - 1);
-      const Cx<R>* d = ring[t % D][rc];
-      Cx<R> b = bt;
-      bt = bn;
-      bn = ld(in, t + 2);
-      if (t > 0) {
-        if (act) sh[rc] = z;
-        __syncwarp(mask);
-        const Cx<R> w = r < 6 ? row_dot(d, sh) : czero<R>();
-        __syncwarp(mask);
-        if (r < 6) sh[rc] = w;
-        __syncwarp(mask);
-        if (r < 6) {
-          if (AX) {
-            b = b + sh[rc];
-          } else {
-            const int sl = stab[t - 1];
+  const int sr = r / 3, cr = r - 3 * (r / 3);
+  Cx<R> wn[3];
+  auto link = [&](int t) {
+    const int sl = slot_of(g, t < 0 ? 0 : t);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) b = cfmaconj(b, ut[(size_t)(3 * c + cr) * tp + sl], sh[3 * sr + c]);
-          }
-        }
-        __syncwarp(mask);
-      }
-      z = b;
-      if (io) out[stab[t]] = z;
+    for (int c = 0; c < 3; ++c) {
+      wn[c] = ut[(size_t)(r < 6 ? 3 * c + cr : 3 * cr + c) * tp + sl];
+      if (r < 6) wn[c].im = -wn[c].im;
     }
-    if (gi == 0) cp_wait<0>();
-    __syncthreads();
+  };
+  auto times_link = [&]() {  // (W y) on row r, y being in sh + 24
+    Cx<R> x = czero<R>();
+#pragma unroll
+    for (int c = 0; c < 3; ++c) x = cfma(x, wn[c], sh[24 + 3 * sr + c]);
+    return x;
+  };
+
+  for (int q = 0; q < NST - 1; ++q) issue();
+  Cx<R> y = czero<R>();  // component r of c_t (forward), y_t (backward)
+
+  // forward
+  auto fwd = [&](const Cx<R>* blk, int t, int i) {
+    Cx<R> m[6], v[6];
+    ld_row<6>(blk + h * CS * 72 + i * 72 + 6 * r, m);
+    Cx<R>* ex = sh + 12 * (i & 1);
+    if (AX) {
+      if (own) {
+        const Cx<R> b = mine[t];
+        ex[r] = r < 6 ? b + y : b;  // y = 0 at t = 0
+      }
+    } else {
+      if (own) {
+        const Cx<R> b = mine[t];
+        ex[r] = r < 6 && t > 0 ? b + times_link() : b;
+      }
+      link(t);  // W_t^dag for the next step (W_{T-1}: unused)
+    }
+    __syncwarp();
+    ld_row<6>(ex + 6 * h, v);
+    y = pair_sum(dot(czero<R>(), m, v));
+    if (own) {
+      mine[t] = y;
+      if (!AX) sh[24 + r] = y;
+    }
+    if (!AX) __syncwarp();
+  };
+  for (int c = 0; c < NC; ++c) {
+    const Cx<R>* blk = next_chunk();
+    if (!io) continue;
+    const int t0 = c * CS;
+    if (t0 + CS <= T) {
+#pragma unroll
+      for (int i = 0; i < CS; ++i) fwd(blk, t0 + i, i);
+    } else {
+      for (int i = 0; t0 + i < T; ++i) fwd(blk, t0 + i, i);
+    }
+  }
+  const Cx<R> yT = y;  // y_{T-1} = c_{T-1}
+
+  // backward
+  Cx<R> lm[6];
+  if (io) ld_row<6>(A.lam + (size_t)l * kBlk + 12 * r + 6 * h, lm);
+  if (!AX) link(T - 2);
+  __syncwarp();
+  auto bwd = [&](const Cx<R>* blk, int t, int i) {
+    Cx<R> m[3], v[3];
+    ld_row<3>(blk + CS * 72 + i * 72 + 6 * r + 3 * h, m);
+    Cx<R>* ex = sh + 12 * (i & 1);
+    if (AX) {
+      if (own && r >= 6) ex[r - 6] = y;
+    } else {  // W_t y_{t+1} on the P_- half
+      if (own) sh[24 + r] = y;
+      __syncwarp();
+      if (own && r >= 6) ex[r - 6] = times_link();
+      link(t - 1);
+    }
+    __syncwarp();
+    ld_row<3>(ex + 3 * h, v);
+    y = pair_sum(dot(own ? mine[t] : czero<R>(), m, v));
+    if (own) mine[t] = y;
+  };
+  for (int c = 0; c < NC; ++c) {
+    const Cx<R>* blk = next_chunk();
+    if (!io) continue;
+    const int n = min(CS, T - c * CS), t0 = T - c * CS - n;  // slices t0 .. t0 + n - 1, last first
+    if (c > 0 && n == CS) {
+#pragma unroll
+      for (int i = CS - 1; i >= 0; --i) bwd(blk, t0 + i, i);
+    } else {
+      for (int i = c == 0 ? n - 2 : n - 1; i >= 0; --i) bwd(blk, t0 + i, i);
+    }
   }
 
-  // backward sweep: chi_t to out
-  Cx<R> y0 = czero<R>(), yT = czero<R>();
-  {
-    auto issue = [&](int u) {  // step u (t = N_t - 1 - u): row rc of Sigma_t^-1
-      if (fill && u < T) cp_row<R>(ring[u % D][rc], S + (size_t)(T - 1 - u) * kBlk);
-      if (gi == 0) cp_commit();
-    };
-    for (int u = 0; u < D - 1; ++u) issue(u);
-    Cx<R> zt = z;
-    Cx<R> zn = ld(out, T - 2);
-    Cx<R> y = czero<R>();
-    for (int u = 0; u < T; ++u) {
-      const int t = T - 1 - u;
-      if (gi == 0) cp_wait<D - 2>();
-      __syncthreads();
-      issue(u + D - 1);
-      const Cx<R>* d = ring[u % D][rc];
-      Cx<R> v = zt;
-      zt = zn;
-      zn = t >= 2 ? ld(out, t - 2) : czero<R>();
-      if (u > 0) {
-        if (act) sh[rc] = y;
-        __syncwarp(mask);
-        if (act && r >= 6) {
-          if (AX) {
-            v = v + sh[rc];
-          } else {
-            const int sl = stab[t];
+  // c = Lambda W^dag chi: the P_+ half of chi_{T-1}, the P_- half of chi_0
+  Cx<R> cv[6];
+  if (io) {
+    __syncwarp();
+    if (own) sh[r] = r < 6 ? yT : y;
+    __syncwarp();
+    ld_row<6>(sh + 6 * h, cv);
+    const Cx<R> cc = pair_sum(dot(czero<R>(), lm, cv));
+    if (own) sh[12 + r] = cc;
+    __syncwarp();
+    ld_row<6>(sh + 12 + 6 * h, cv);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) v = cfma(v, ut[(size_t)(3 * cr + c) * tp + sl], sh[3 * sr + c]);
-          }
-        }
-        __syncwarp(mask);
-      }
-      if (act) sh[rc] = v;
-      __syncwarp(mask);
-      y = act ? row_dot(d, sh) : czero<R>();
-      __syncwarp(mask);
-      if (io) out[stab[t]] = y;
-      if (t == 0) y0 = y;
-      if (t == T - 1) yT = y;
-    }
-    if (gi == 0) cp_wait<0>();
-    __syncthreads();
+    for (int i = 0; i < 6; ++i) cv[i] = mk<R>(-cv[i].re, -cv[i].im);
   }
 
-  // c = Lambda W^dag chi
-  if (act) sh[rc] = r < 6 ? yT : y0;
-  __syncwarp(mask);
-  Cx<R> c = czero<R>();
-  if (act) c = row_times(A.lam + (size_t)l * kBlk, rc, sh);
-  __syncwarp(mask);
-  if (act) sh[rc] = c;
-  __syncwarp(mask);
-  Cx<R> cv[12];
+  // chi_t - Z_t c
+  auto corr = [&](const Cx<R>* blk, int t, int i) {
+    Cx<R> m[6];
+    ld_row<6>(blk + i * kBlk + 12 * r + 6 * h, m);
+    const Cx<R> x = pair_sum(dot(own ? mine[t] : czero<R>(), m, cv));
+    if (own) mine[t] = x;
+  };
+  for (int c = 0; c < NC; ++c) {
+    const Cx<R>* blk = next_chunk();
+    if (!io) continue;
+    const int t0 = c * CS;
+    if (t0 + CS <= T) {
 #pragma unroll
-  for (int kk = 0; kk < 12; ++kk) cv[kk] = sh[kk];
-  __syncwarp(mask);
-
-  // out_t = xpost_t + apost (chi_t - Z_t c)
-  {
-    auto issue = [&](int t) {  // step t: row rc of Z_t
-      if (fill && t < T) cp_row<R>(ring[t % D][rc], Zl + (size_t)t * kBlk);
-      if (gi == 0) cp_commit();
-    };
-    for (int t = 0; t < D - 1; ++t) issue(t);
-    Cx<R> ct = ld(out, 0), cn = ld(out, 1);
-    Cx<R> xt = xp ? ld(xp, 0) : czero<R>(), xn = xp ? ld(xp, 1) : czero<R>();
-    for (int t = 0; t < T; ++t) {
-      if (gi == 0) cp_wait<D - 2>();
-      __syncthreads();
-      issue(t + D - 1);
-      const Cx<R>* d = ring[t % D][rc];
-      Cx<R> x = ct, xv = xt;
-      ct = cn;
-      cn = ld(out, t + 2);
-      if (xp) {
-        xt = xn;
-        xn = ld(xp, t + 2);
-      }
-      x = x - row_dot_reg(d, cv);
-      if (io) out[stab[t]] = xp ? xv + A.apost * x : x;
+      for (int i = 0; i < CS; ++i) corr(blk, t0 + i, i);
+    } else {
+      for (int i = 0; t0 + i < T; ++i) corr(blk, t0 + i, i);
     }
-    if (gi == 0) cp_wait<0>();
   }
-  if (io)
-    for (int t = T; t < tp; ++t) out[stab[t]] = czero<R>();  // padding slots stay zero
+  cp_wait<0>();
+  if (!io) return;
+  __syncwarp();
+
+  // out = xpost + apost Q^-1 in (or Q^-1 in); padding slots zero
+  const size_t base = ((size_t)k * g.Nl + l) * NSPIN_C * tp;
+  const Cx<R>* xp = A.xpost ? A.xpost + base : nullptr;
+  Cx<R>* out = A.out + base;
+  for (int sl = lane; sl < tp; sl += 32) {
+    const int t = (sl % g.lpl) * g.n + sl / g.lpl;
+    Cx<R> x[12];
+    if (xp) {
+#pragma unroll
+      for (int c = 0; c < 12; ++c) x[c] = t < T ? xp[(size_t)c * tp + sl] : czero<R>();
+    }
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+      Cx<R> v = t < T ? line[c * ls + t] : czero<R>();
+      out[(size_t)c * tp + sl] = xp ? x[c] + A.apost * v : v;
+    }
+  }
 }
 
 // ----------------------------------------------------------------------------
@@ -913,21 +842,22 @@ void qinv(wf_handle* h, const QFactors<R>& F, int p, const Cx<R>* in, Cx<R>* out
   a.pl = gauge_pl<R>(h, p);
   a.s = (R)h->g.bc;
   if (h->g.tp > kTMax) throw Error(WF_EINVAL, "Q^-1 kernel: padded time line longer than 256 slots");
-  const size_t groups = (size_t)nrhs * h->g.Nl;
-  const unsigned blocks = (unsigned)((groups + kQGroups - 1) / kQGroups);
+  // up to kQMaxWarps sources of a line share its block stream, in groups of equal size
+  const int ngrp = (nrhs + kQMaxWarps - 1) / kQMaxWarps, G = (nrhs + ngrp - 1) / ngrp;
+  const size_t smem = qinv_smem<R>(h->g.T, G);
+  const unsigned blocks = (unsigned)((size_t)h->g.Nl * ngrp);
   Prof P(h, tag<R>("qinv_apply_f64", "qinv_apply_f32"));
-  if (nrhs >= kQGroups) {  // one ring per CTA of kQGroups sources of one line
-    const unsigned sblocks = (unsigned)((size_t)h->g.Nl * ((nrhs + kQGroups - 1) / kQGroups));
-    if (h->axial)
-      k_qinv_apply_shared<R, true><<<sblocks, kQGroups * kGrp, 0, h->stream>>>(a);
-    else
-      k_qinv_apply_shared<R, false><<<sblocks, kQGroups * kGrp, 0, h->stream>>>(a);
-  } else if (h->axial) {
-    k_qinv_apply<R, true><<<blocks, kQGroups * kGrp, 0, h->stream>>>(a);
-  } else {
-    k_qinv_apply<R, false><<<blocks, kQGroups * kGrp, 0, h->stream>>>(a);
+  auto run = [&](auto kernel) {
+    WF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kernel<<<blocks, 32 * G, smem, h->stream>>>(a, ngrp);
+    WF_CUDA(cudaGetLastError());
+  };
+  switch (G) {
+    case 1: h->axial ? run(k_qinv_line<R, true, 1>) : run(k_qinv_line<R, false, 1>); break;
+    case 2: h->axial ? run(k_qinv_line<R, true, 2>) : run(k_qinv_line<R, false, 2>); break;
+    case 3: h->axial ? run(k_qinv_line<R, true, 3>) : run(k_qinv_line<R, false, 3>); break;
+    default: h->axial ? run(k_qinv_line<R, true, 4>) : run(k_qinv_line<R, false, 4>); break;
   }
-  WF_CUDA(cudaGetLastError());
 }
 
 // out = xpost + apost (S) D_s in on the lines of parity p (in: the other parity)
