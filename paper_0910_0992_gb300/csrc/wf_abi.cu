@@ -273,6 +273,9 @@ std::vector<int2> build_unit_table(const Geom& g, int nrhs, int gsrc) {
   return t;
 }
 
+}  // namespace
+
+namespace wf {
 // index tables for the wide kernels (built once per handle and per nrhs, on the handle's stream)
 void attach_tables(wf_handle* h, LineArgs<float>& a) {
   const Geom& g = h->g;
@@ -294,6 +297,9 @@ void attach_tables(wf_handle* h, LineArgs<float>& a) {
   a.nbr = nb.as<int>();
   a.order = ob->as<int2>();
 }
+}  // namespace wf
+
+namespace {
 
 // unit table of the bulk-fed hop kernels: the tiled line order of line_rhs with the sources of a
 // line in groups of gsrc side by side, as (first source, line) pairs (built once per handle, nrhs,
@@ -1616,8 +1622,9 @@ void solve_temporal_schur_dc(int nl, wf_handle* const* hs, const std::vector<con
         a.opl = OP_BWD;
         a.src = SRC_HOP;
         a.out = P.w32_o;
+        if (h->axial) attach_tables(h, a);
         Prof Q(h, "prep_hop_f32");
-        launch_line<float>(a, LK_GENERIC, h->axial, sj);
+        launch_line<float>(a, LK_SCHUR_C, h->axial, sj);
       }
       WF_CUDA(cudaMemsetAsync(b_o, 0, nt * sizeof(Cx<double>), sj));
       { Prof Q(h, "add_f_to_d"); launch_add_f_to_d(b_o, P.w32_o, nt, sj); }
@@ -1664,8 +1671,9 @@ void solve_temporal_schur_dc(int nl, wf_handle* const* hs, const std::vector<con
         a.opl = OP_BWD;
         a.src = SRC_HOP;
         a.out = P.w32_e;
+        if (h->axial) attach_tables(h, a);
         Prof Q(h, "recon_hop_f32");
-        launch_line<float>(a, LK_GENERIC, h->axial, sj);
+        launch_line<float>(a, LK_SCHUR_B, h->axial, sj);
       }
       { Prof Q(h, "add_f_to_d", 2); launch_add_f_to_d(P.psi_e, P.w32_e, nt, sj); launch_add_f_to_d(P.psi_o, P.w32_o, nt, sj); }
       m_apply<double>(h, P.psi_e, P.psi_o, P.r_e, P.r_o, P.eta_e, P.eta_o, -1.0, m);
@@ -2179,8 +2187,10 @@ void hop_to(wf_handle* h, int par_out, const Cx<R>* in, Cx<R>* out, const char* 
   a.opl = OP_COPY;
   a.src = SRC_HOP;
   a.out = out;
+  if constexpr (sizeof(R) == 4)
+    if (h->axial) attach_tables(h, a);
   Prof P(h, pname<R>(name));
-  launch_line<R>(a, LK_GENERIC, h->axial, h->stream);
+  launch_line<R>(a, LK_HOP, h->axial, h->stream);
 }
 
 // out = acc + alpha A^pp in
@@ -2210,6 +2220,8 @@ void line_step(wf_handle* h, int parity, int src, const Cx<R>* in, Cx<R>* out, i
   // a hop followed by C_L has the compiled variant of the Schur operator's K-c (in FP32 in the
   // axial frame: the one-thread-per-site kernel)
   const int kind = src == SRC_HOP && opu == OP_COPY && opl == OP_BWD ? LK_SCHUR_C : LK_GENERIC;
+  if constexpr (sizeof(R) == 4)
+    if (h->axial && kind == LK_SCHUR_C) attach_tables(h, a);
   Prof P(h, pname<R>(name));
   launch_line<R>(a, kind, h->axial, h->stream);
 }

@@ -885,8 +885,10 @@ void hop(wf_handle* h, int p, const Cx<R>* in, Cx<R>* out, int nrhs, const Cx<R>
   a.swap_out = swap_out;
   a.out = out;
   a.drop_job = -1;
+  if constexpr (sizeof(R) == 4)
+    if (h->axial && wide_supported(h->g)) attach_tables(h, a);
   Prof P(h, tag<R>("fsw_hop_f64", "fsw_hop_f32"));
-  launch_line<R>(a, LK_GENERIC, h->axial, h->stream);
+  launch_line<R>(a, LK_HOP, h->axial, h->stream);
 }
 
 // M-hat_full (dagger: its adjoint) on internal odd fields x -> out; e1, e2 (even) and o1 (odd) are

@@ -153,6 +153,11 @@ struct Prof {
   }
 };
 
+// index tables of the one-thread-per-site kernels (neighbour lines, traversal order) for a.nrhs
+// sources, built on first use
+template <typename R> struct LineArgs;
+void attach_tables(wf_handle* h, LineArgs<float>& a);
+
 // M-hat (dagger: gamma_5 M-hat gamma_5) on internal odd fields x -> out; y (odd) and z (even)
 // are work fields of the same size as x.
 template <typename R>

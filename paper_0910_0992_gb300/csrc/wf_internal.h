@@ -61,9 +61,9 @@ struct DevBuf {
 template <typename R> struct LineArgs;
 
 // which compiled variant of the line kernel to launch: the three Schur-operator kernels
-// have their source and solve ops fixed at compile time; LK_GENERIC reads them from the
-// arguments
-enum LineKind { LK_GENERIC = 0, LK_SCHUR_A = 1, LK_SCHUR_B = 2, LK_SCHUR_C = 3 };
+// have their source and solve ops fixed at compile time, as has the plain hop (copy on both
+// halves); LK_GENERIC reads them from the arguments
+enum LineKind { LK_GENERIC = 0, LK_SCHUR_A = 1, LK_SCHUR_B = 2, LK_SCHUR_C = 3, LK_HOP = 4 };
 
 template <typename R>
 void launch_line(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s);

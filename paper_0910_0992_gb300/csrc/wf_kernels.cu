@@ -34,7 +34,7 @@ static bool use_wide(const Geom& g, int kind, bool fp32) {
     return (e && e[0] == '0') ? 0 : (e && e[0] == '2') ? 2 : 1;
   }();
   if (!mode || !wide_supported(g)) return false;
-  return mode == 2 || (fp32 && (kind == LK_SCHUR_B || kind == LK_SCHUR_C));
+  return mode == 2 || (fp32 && (kind == LK_SCHUR_B || kind == LK_SCHUR_C || kind == LK_HOP));
 }
 
 template <typename R>

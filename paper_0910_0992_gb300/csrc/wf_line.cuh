@@ -147,12 +147,12 @@ __device__ __forceinline__ Mat3<R> ldlink(const Cx<R>* __restrict__ base, int tp
   for (int k = 0; k < 6; ++k) U.e[k] = ldc(base + k * tp + slot);
   const Cx<R>* a = U.e;
   const Cx<R>* b = U.e + 3;
-  const Cx<R> c0 = cmul(a[1], b[2]) - cmul(a[2], b[1]);
-  const Cx<R> c1 = cmul(a[2], b[0]) - cmul(a[0], b[2]);
-  const Cx<R> c2 = cmul(a[0], b[1]) - cmul(a[1], b[0]);
-  U.e[6] = mk<R>(c0.re, -c0.im);
-  U.e[7] = mk<R>(c1.re, -c1.im);
-  U.e[8] = mk<R>(c2.re, -c2.im);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {  // conj(a_i b_j - a_j b_i), one multiply-add chain per part
+    const Cx<R> ai = a[(c + 1) % 3], aj = a[(c + 2) % 3], bi = b[(c + 1) % 3], bj = b[(c + 2) % 3];
+    U.e[6 + c] = mk<R>(fma(aj.im, bi.im, fma(-aj.re, bi.re, fma(-ai.im, bj.im, ai.re * bj.re))),
+                       fma(aj.im, bi.re, fma(aj.re, bi.im, fma(-ai.im, bj.re, -(ai.re * bj.im)))));
+  }
   return U;
 }
 

@@ -342,6 +342,136 @@ __device__ __forceinline__ void spin_solve4(Vec3<R> (&w)[4], int j, int T, const
   }
 }
 
+// The same solve for unpadded 128-site lines of w scaled by s (s inv_mu once, then one multiply-add
+// per site and pass); every lane group then has the same map a = mu^-4, so the scan's factors
+// mu^-4d need no shuffles.
+template <typename R, bool FWD>
+__device__ __forceinline__ void spin_solve4_full(Vec3<R> (&w)[4], int j, const Cx<R>* __restrict__ K_line, R inv_mu,
+                                                 R bc, R s) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w[i] = vscale(s * inv_mu, w[i]);
+  Vec3<R> c = w[FWD ? 0 : 3];
+#pragma unroll
+  for (int i = 1; i < 4; ++i) c = vaxpy(inv_mu, c, w[FWD ? i : 3 - i]);
+  const int jo = FWD ? j : 31 - j;  // groups before this one in time order
+  const R a4 = (inv_mu * inv_mu) * (inv_mu * inv_mu);
+  R ad = a4, ap = R(1);
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const Vec3<R> cn = FWD ? vshfl_up(c, d, 32) : vshfl_down(c, d, 32);
+    if (jo >= d) c = vaxpy(ad, cn, c);
+    if (jo & d) ap *= ad;
+    ad *= ad;
+  }
+  // the line's composite is at its last lane in time order; the wrap value enters the first
+  const Vec3<R> C = vshfl_idx(c, FWD ? 31 : 0, 32);
+  const Mat3<R> K = ldmat(K_line, 1, 0);
+  Vec3<R> e = vscale(bc, FWD ? matvec_dag(K, C) : matvec(K, C));
+  const Vec3<R> cp = FWD ? vshfl_up(c, 1, 32) : vshfl_down(c, 1, 32);
+  if (jo > 0) e = vaxpy(ap, e, cp);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int mm = FWD ? i : 3 - i;
+    e = vaxpy(inv_mu, e, w[mm]);
+    w[mm] = e;
+  }
+}
+
+// D_s of hop_site, without its factor 1/2, for 128-slot lines in FP32 with the operands staged through
+// shared memory: each warp copies a direction's 18 components (a neighbour spinor and a two-row link,
+// 32 slots of 8 bytes each) asynchronously, 16 bytes per lane, into one of its own two stages while
+// it computes the direction before from the other: the loads in flight then cost no registers (the
+// register-fed hop_site holds at most one direction's, and waits for them before it computes). Two
+// stages leave room for 6 CTAs per SM. Measured on 24^3 x 128, K-b / K-c: 643 / 681 us with 12 sources
+// and 80 / 83 us with one (register-fed, 7 CTAs: 721 / 789 and 87 / 92; one stage emptied into
+// registers before the next copy, 7 CTAs: 705 / 738 and 86 / 86; two stages at 5 CTAs: 712 / 743 with
+// 12). K-c's 3.9 GB of DRAM traffic then run at 0.85 of the copy bandwidth; K-b is bound by issue
+// slots (0.69 busy) beside 0.52 of DRAM. Once the last direction's operands are in registers,
+// free_stage() runs.
+constexpr int kStageElems = 18 * 32;  // elements of one stage of one warp
+constexpr int kWarpStage = 2 * kStageElems;  // a warp's shared memory: its stages, later its part of
+                                             // the transpose (384 elements, in the first stage) and
+                                             // K-c's post-axpy operand (384, in the second)
+
+__device__ __forceinline__ void stage_copy(Cx<float>* dst, const Cx<float>* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+               "l"(__cvta_generic_to_global(src))
+               : "memory");
+}
+
+template <class FreeStage>
+__device__ __forceinline__ void hop_site_staged(Vec3<float> (&h)[4], const LineArgs<float>& A, int rhs, int l,
+                                                Cx<float>* stage, FreeStage free_stage) {
+  typedef float R;
+  constexpr int tp = 128;
+  static_assert(SpatialLinkNC<float>::value == 6, "staged hop: two-row links");
+  const int Nl = A.g.Nl, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int nb[6];
+  neighbours(A, l, nb);
+  // this lane's 16 bytes of a pair of components: component lane / 16, elements 2 (lane % 16) ..
+  const int off = (lane >> 4) * tp + warp * 32 + 2 * (lane & 15);
+  const Cx<R>* up = A.src_up + (size_t)rhs * Nl * NSPIN_C * tp + off;
+  const Cx<R>* lo = A.src_lo + (size_t)rhs * Nl * NSPIN_C * tp + off;
+  auto issue = [&](int d) {
+    const int k = d >> 1, ln = nb[d];
+    const Cx<R>* u = up + (size_t)ln * (NSPIN_C * tp);
+    const Cx<R>* v = lo + (size_t)ln * (NSPIN_C * tp);
+    const Cx<R>* lk = (d & 1) == 0 ? A.us_out + (size_t)(k * Nl + l) * (6 * tp) + off
+                                   : A.us_nbr + (size_t)(k * Nl + ln) * (6 * tp) + off;
+    Cx<R>* st = stage + (d & 1) * kStageElems + 2 * lane;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      stage_copy(st + 64 * i, u + 2 * i * tp);
+      stage_copy(st + 64 * (3 + i), v + 2 * i * tp);
+      stage_copy(st + 64 * (6 + i), lk + 2 * i * tp);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int s = 0; s < 4; ++s) h[s] = vzero<R>();
+  issue(0);
+#pragma unroll
+  for (int d = 0; d < 6; ++d) {
+    const int k = d >> 1, dir = d & 1;
+    if (d < 5) {
+      issue(d + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncwarp();
+    const Cx<R>* st = stage + (d & 1) * kStageElems;
+    const Vec3<R> u0 = ldvec(st, 32, lane), u1 = ldvec(st + 96, 32, lane);
+    const Vec3<R> d0 = ldvec(st + 192, 32, lane), d1 = ldvec(st + 288, 32, lane);
+    const Mat3<R> U = ldlink(st + 384, 32, lane);
+    __syncwarp();
+    if (d == 5) free_stage();
+    Vec3<R> s0, s1;
+    isigma(k, d0, d1, s0, s1);
+    Vec3<R> h0, h1;
+    if (dir == 0) {
+      h0 = vadd(u0, s0);
+      h1 = vadd(u1, s1);
+    } else {
+      h0 = vaxpy(R(-1), s0, u0);
+      h1 = vaxpy(R(-1), s1, u1);
+    }
+    const Vec3<R> w0 = dir == 0 ? matvec(U, h0) : matvec_dag(U, h0);
+    const Vec3<R> w1 = dir == 0 ? matvec(U, h1) : matvec_dag(U, h1);
+    h[0] = vadd(h[0], w0);
+    h[1] = vadd(h[1], w1);
+    Vec3<R> r0, r1;
+    isigma(k, w0, w1, r0, r1);
+    if (dir == 0) {
+      h[2] = vaxpy(R(-1), r0, h[2]);
+      h[3] = vaxpy(R(-1), r1, h[3]);
+    } else {
+      h[2] = vadd(h[2], r0);
+      h[3] = vadd(h[3], r1);
+    }
+  }
+}
+
 // one atomic per line for |out|^2 (lines of whole warps)
 template <typename R>
 __device__ __forceinline__ void line_norm_whole_warps(double* nrm_s, R nrm, int q, int tp, int li, int sl, bool line_ok,
@@ -363,15 +493,16 @@ __device__ __forceinline__ void line_norm_whole_warps(double* nrm_s, R nrm, int 
 // offset is an immediate), or 0 to read the layout at run time.
 // The kernel body (wf_wide_body.inc) as a device function for block blk of one lattice's part of a
 // multi-lattice launch; k_line_wide includes the same body directly.
-template <typename R, int SRC, int OPU, int OPL, int TPC, bool H = false>
+template <typename R, int SRC, int OPU, int OPL, int TPC, bool H = false, bool STG = false>
 __device__ __forceinline__ void line_wide_body(const LineArgs<R>& A, int blk) {
 #define WF_WIDE_BLOCK blk
 #include "wf_wide_body.inc"
 #undef WF_WIDE_BLOCK
 }
 
-template <typename R, int SRC, int OPU, int OPL, int TPC, bool H = false>
-__global__ void __launch_bounds__(kWideCta, WideMinBlocks<R, SRC == SRC_HOP && OPU == OP_COPY>::value)
+// STG: the staged hop (FP32, 128-slot lines) instead of the register-fed one
+template <typename R, int SRC, int OPU, int OPL, int TPC, bool H = false, bool STG = false>
+__global__ void __launch_bounds__(kWideCta, STG ? 6 : WideMinBlocks<R, SRC == SRC_HOP && OPU == OP_COPY>::value)
     k_line_wide(const LineArgs<R> A) {
 #define WF_WIDE_BLOCK ((int)blockIdx.x)
 #include "wf_wide_body.inc"
@@ -458,7 +589,8 @@ void launch_line_wide(const LineArgs<R>& a, int kind, cudaStream_t s) {
       else                                                                                        \
         wide::k_line_wide<R, SRCV, OPUV, OPLV, 0, kH><<<blocks, wide::kWideCta, 0, s>>>(a);       \
     } else if (t128) {                                                                            \
-      wide::k_line_wide<R, SRCV, OPUV, OPLV, 128><<<blocks, wide::kWideCta, 0, s>>>(a);           \
+      constexpr bool kS = kF32 && (SRCV) == SRC_HOP; /* staged */                                 \
+      wide::k_line_wide<R, SRCV, OPUV, OPLV, 128, false, kS><<<blocks, wide::kWideCta, 0, s>>>(a); \
     } else {                                                                                      \
       wide::k_line_wide<R, SRCV, OPUV, OPLV, 0><<<blocks, wide::kWideCta, 0, s>>>(a);             \
     }                                                                                             \
@@ -467,6 +599,7 @@ void launch_line_wide(const LineArgs<R>& a, int kind, cudaStream_t s) {
     case LK_SCHUR_A: WF_KW(SRC_LOAD, OP_FWD, OP_SKIP); break;
     case LK_SCHUR_B: WF_KW(SRC_HOP, OP_FWD, OP_BWD); break;
     case LK_SCHUR_C: WF_KW(SRC_HOP, OP_COPY, OP_BWD); break;
+    case LK_HOP: WF_KW(SRC_HOP, OP_COPY, OP_COPY); break;
     default: WF_KW(-1, -1, -1); break;
   }
 #undef WF_KW
