@@ -140,6 +140,8 @@ LineArgs<R> line_args(wf_handle* h, int parity, int nrhs) {
   a.opl = OP_COPY;
   a.drop_job = -1;
   a.df = (sizeof(R) == 8 && h->df_ops) ? 1 : 0;
+  a.fx_out = h->usfx[parity].as<int4>();
+  a.fx_nbr = h->usfx[1 - parity].as<int4>();
   return a;
 }
 
@@ -526,6 +528,8 @@ void m_apply(wf_handle* h, const Cx<R>* in_e, const Cx<R>* in_o, Cx<R>* out_e, C
     m.pl = G.pl[p];
     m.us_out = G.us[p];
     m.us_nbr = G.us[1 - p];
+    m.fx_out = h->usfx[p].as<int4>();
+    m.fx_nbr = h->usfx[1 - p].as<int4>();
     m.x = p ? x_o : x_e;
     m.a = (R)a;
     m.out = p ? out_o : out_e;
@@ -2045,6 +2049,8 @@ OpFn<R> full_op(wf_handle* h, bool temporal) {
         m.pl = G.pl[p];
         m.us_out = G.us[p];
         m.us_nbr = G.us[1 - p];
+        m.fx_out = h->usfx[p].as<int4>();
+        m.fx_nbr = h->usfx[1 - p].as<int4>();
         m.swap = swap;
         m.out = out + p * hn;
         m.mu = (R)h->g.mu;
@@ -2831,6 +2837,7 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
       h->lamf64[p].ensure(nlam * sizeof(Cx<double>), s);
       if (!h->axial) h->ut32[p].ensure(nut * sizeof(Cx<float>), s);
       h->us32[p].ensure(nus32 * sizeof(Cx<float>), s);
+      h->usfx[p].ensure(nus * sizeof(int4), s);
       h->lamb32[p].ensure(nlam * sizeof(Cx<float>), s);
       h->lamf32[p].ensure(nlam * sizeof(Cx<float>), s);
     }
@@ -2838,7 +2845,7 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
     WF_CUDA(cudaMemsetAsync(h->iflag.p, 0, sizeof(int), s));
     Cx<double>* ut[2] = {h->ut64[0].as<Cx<double>>(), h->ut64[1].as<Cx<double>>()};
     Cx<double>* us[2] = {h->us64[0].as<Cx<double>>(), h->us64[1].as<Cx<double>>()};
-    Prof P(h, "gauge_ingest", 1 + 2 * 5);
+    Prof P(h, "gauge_ingest", 1 + 2 * 6);
     launch_import_gauge(g, dU, ut, us, s);
     if (h->axial) {
       // axial frame: ut becomes the rotation g, spatial links rotated in place, P, Lambda and the
@@ -2866,6 +2873,7 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
         launch_d2f(h->lamf64[p].as<Cx<double>>(), h->lamf32[p].as<Cx<float>>(), nlam, s);
       }
     }
+    for (int p = 0; p < 2; ++p) launch_links_fx(us[p], h->usfx[p].as<int4>(), nus, s);
     int flag = 0;
     WF_CUDA(cudaMemcpyAsync(&flag, h->iflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     WF_CUDA(cudaStreamSynchronize(s));

@@ -1,0 +1,182 @@
+// FP64 spatial hops in block fixed point.
+//
+// GB300 issues two FP64 multiply-adds per clock and SM, but 64 32 x 32 -> 64-bit integer ones: the
+// 648 FP64 operations of a spatial hop cost 324 clocks per site and SM, the same hop in 64-bit fixed
+// point about 90 (M, both parities, 24^3 x 128, 12 sources: 30.4 -> 8.9 ms; 12^3 x 48, 4 sources: 548 ->
+// 188 us). The direction d of a site's stencil is a half-spinor of 12 real numbers times one
+// SU(3) link, and
+//   * the 24 real numbers of the neighbour spinor share an exponent E (the largest of theirs, and of
+//     the directions before): v = x 2^(55 - E), |v| < 2^56, an exact shift of the 53-bit mantissa but
+//     for bits below 2^(E - 55), a quarter of half an ulp of the largest number;
+//   * links are stored beside their FP64 form as u = U 2^58 in two 32-bit limbs (|U| <= 1);
+//   * projections are integer sums (< 2^57); a product takes three limb products, accumulated over
+//     the six of a matrix row in two 64-bit sums: H of the high limbs' products and X of the mixed ones
+//     (the low limbs' product is below 1/4 of a unit of v), w = H + X / 2^28 in units of v / 4;
+//   * the six directions add up in 64 bits (|sum| < 2^(56 + 6.9)).
+// So the only roundings are those of v, U 2^58 and X / 2^28, each below an FP64 rounding of the
+// largest term: the result is at least as close to the exact one as FP64 arithmetic's (measured on
+// 12^3 x 48, M against 64-bit reference arithmetic: relative error 3.5e-15 either way). Spinors with a NaN,
+// an infinity or exponents near the ends of FP64's range take the FP64 form (hop_site_fp64).
+#pragma once
+
+#include "wf_line.cuh"
+
+namespace wf {
+
+// one real number of a link: limbs of U 2^58, hi 2^28 + lo, 0 <= lo < 2^28
+__device__ __forceinline__ int2 link_limbs(double u) {
+  const long long v = llrint(u * 288230376151711744.0);  // 2^58
+  return make_int2((int)(v >> 28), (int)(v & 0xfffffff));
+}
+
+// acc + a b (a limb of each sign; left to the compiler, the products with the limbs it knows to be
+// non-negative became full 64-bit multiplications)
+__device__ __forceinline__ void fx_mac(long long& acc, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
+
+struct FxAcc {
+  long long a[4][3][2];  // [spin][colour][re, im], in units of 2^(E - 1023 - 57)
+  int E;                 // biased FP64 exponent
+  bool wide;             // some spinor was out of range: the result is not valid
+};
+
+constexpr int kFxMinExp = 80, kFxMaxExp = 2030;  // biased exponents served
+
+__device__ __forceinline__ void fx_clear(FxAcc& f) {
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f.a[s][c][0] = f.a[s][c][1] = 0;
+  f.E = kFxMinExp;
+  f.wide = false;
+}
+
+// x as v = x 2^(55 - E) (E >= x's exponent; zero and subnormal x: 0)
+__device__ __forceinline__ long long fx_from(double x, int E) {
+  const unsigned hw = (unsigned)__double2hiint(x), lw = (unsigned)__double2loint(x);
+  const int s = min(E - (int)((hw >> 20) & 0x7ff), 63);
+  const unsigned mh = (hw & 0xfffff) | 0x100000;
+  unsigned long long m = ((unsigned long long)__funnelshift_l(lw, mh, 3) << 32) | (lw << 3);
+  m >>= s;
+  const long long neg = (long long)((int)hw >> 31);
+  return ((long long)m ^ neg) - neg;
+}
+
+// One direction d = 2 k + dir of D_s (without its factor 1/2): axis k, dir 0: (1 - gamma_k) U x,
+// 1: (1 + gamma_k) U^dag x, x the neighbour spinor. The directions share one copy of this code (d is
+// uniform; only the spin algebra branches on it): unrolled six times, the kernel missed the instruction
+// cache on 45 % of its issue slots.
+struct FxHalf {  // the half-spinor in limbs; nh, nl: minus the imaginary part's
+  int hh[2][3][2], hl[2][3][2], nh[2][3], nl[2][3];
+};
+__device__ __forceinline__ void fx_project(FxAcc& f, FxHalf& q, int d, const Vec3<double> (&x)[4]) {
+  unsigned mx = 0;
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      mx = max(mx, (unsigned)__double2hiint(x[s].c[c].re) & 0x7fffffffu);
+      mx = max(mx, (unsigned)__double2hiint(x[s].c[c].im) & 0x7fffffffu);
+    }
+  const int e = (int)(mx >> 20);
+  f.wide = f.wide || (mx != 0 && (e < kFxMinExp || e >= kFxMaxExp));
+  if (e > f.E) {
+    const int s = min(e - f.E, 63);
+    f.E = e;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        f.a[i][c][0] >>= s;
+        f.a[i][c][1] >>= s;
+      }
+  }
+  // h = u +- i sigma_k d (isigma of wf_line.cuh)
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    long long u[2][2], v[2][2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      u[s][0] = fx_from(x[s].c[c].re, f.E);
+      u[s][1] = fx_from(x[s].c[c].im, f.E);
+      v[s][0] = fx_from(x[2 + s].c[c].re, f.E);
+      v[s][1] = fx_from(x[2 + s].c[c].im, f.E);
+    }
+    switch (d) {
+      case 0: u[0][0] -= v[1][1]; u[0][1] += v[1][0]; u[1][0] -= v[0][1]; u[1][1] += v[0][0]; break;
+      case 1: u[0][0] += v[1][1]; u[0][1] -= v[1][0]; u[1][0] += v[0][1]; u[1][1] -= v[0][0]; break;
+      case 2: u[0][0] += v[1][0]; u[0][1] += v[1][1]; u[1][0] -= v[0][0]; u[1][1] -= v[0][1]; break;
+      case 3: u[0][0] -= v[1][0]; u[0][1] -= v[1][1]; u[1][0] += v[0][0]; u[1][1] += v[0][1]; break;
+      case 4: u[0][0] -= v[0][1]; u[0][1] += v[0][0]; u[1][0] += v[1][1]; u[1][1] -= v[1][0]; break;
+      default: u[0][0] += v[0][1]; u[0][1] -= v[0][0]; u[1][0] -= v[1][1]; u[1][1] += v[1][0]; break;
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        q.hh[s][c][p] = (int)(u[s][p] >> 28);
+        q.hl[s][c][p] = (int)u[s][p] & 0xfffffff;
+      }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      q.nh[s][c] = -q.hh[s][c][1];
+      q.nl[s][c] = -q.hl[s][c][1];
+    }
+  }
+}
+// acc += the link times the half-spinor and its lower spins; lk[e * stride]: the link's entries as
+// {re.hi, re.lo, im.hi, im.lo}
+__device__ __forceinline__ void fx_multiply(FxAcc& f, const FxHalf& q, int d, const int4* __restrict__ lk, int stride) {
+  // w = V h, V = U or U^dag (entry (a, b) at a sa + b sb, imaginary limbs with sign sg)
+  const int dir = d & 1, sg = -dir;
+  const int sa = (dir ? 1 : 3) * stride, sb = (dir ? 3 : 1) * stride;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    long long H[2][2] = {}, X[2][2] = {};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      int4 U = lk[a * sa + b * sb];
+      U.z = (U.z ^ sg) - sg;
+      U.w = (U.w ^ sg) - sg;
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const int rh = q.hh[s][b][0], rl = q.hl[s][b][0], ih = q.hh[s][b][1], il = q.hl[s][b][1];
+        fx_mac(H[s][0], U.x, rh);
+        fx_mac(X[s][0], U.x, rl);
+        fx_mac(X[s][0], U.y, rh);
+        fx_mac(H[s][0], U.z, q.nh[s][b]);
+        fx_mac(X[s][0], U.z, q.nl[s][b]);
+        fx_mac(X[s][0], U.w, q.nh[s][b]);
+        fx_mac(H[s][1], U.x, ih);
+        fx_mac(X[s][1], U.x, il);
+        fx_mac(X[s][1], U.y, ih);
+        fx_mac(H[s][1], U.z, rh);
+        fx_mac(X[s][1], U.z, rl);
+        fx_mac(X[s][1], U.w, rh);
+      }
+    }
+    long long w[2][2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        w[s][p] = H[s][p] + (X[s][p] >> 28);
+        f.a[s][a][p] += w[s][p];
+      }
+    long long(&l0)[2] = f.a[2][a], (&l1)[2] = f.a[3][a];  // lower spins: -+ i sigma_k w
+    switch (d) {
+      case 0: l0[0] += w[1][1]; l0[1] -= w[1][0]; l1[0] += w[0][1]; l1[1] -= w[0][0]; break;
+      case 1: l0[0] -= w[1][1]; l0[1] += w[1][0]; l1[0] -= w[0][1]; l1[1] += w[0][0]; break;
+      case 2: l0[0] -= w[1][0]; l0[1] -= w[1][1]; l1[0] += w[0][0]; l1[1] += w[0][1]; break;
+      case 3: l0[0] += w[1][0]; l0[1] += w[1][1]; l1[0] -= w[0][0]; l1[1] -= w[0][1]; break;
+      case 4: l0[0] += w[0][1]; l0[1] -= w[0][0]; l1[0] -= w[1][1]; l1[1] += w[1][0]; break;
+      default: l0[0] -= w[0][1]; l0[1] += w[0][0]; l1[0] += w[1][1]; l1[1] -= w[1][0]; break;
+    }
+  }
+}
+
+// 2^(E - 1023 - 58): a unit of the accumulators times the projectors' factor 1/2 (E >= kFxMinExp)
+__device__ __forceinline__ double fx_unit(const FxAcc& f) { return __hiloint2double((f.E - 58) << 20, 0); }
+
+}  // namespace wf

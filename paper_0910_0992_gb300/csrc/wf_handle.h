@@ -35,6 +35,7 @@ struct wf_handle {
   // gauge, per parity: U_t [Nl][9][tp], spatial [3][Nl][9][tp], Lambda [Nl][9]
   wf::DevBuf ut64[2], us64[2], lamb64[2], lamf64[2];
   wf::DevBuf ut32[2], us32[2], lamb32[2], lamf32[2];
+  wf::DevBuf usfx[2];  // spatial links in fixed point (wf_fixed.cuh), [3][Nl][9][tp]
   // axial frame: ut64 holds the rotation g(x) instead of U_t; P per line
   wf::DevBuf pl64[2], pl32[2];
   // clover term of the SW operator (wf_load_gauge_clover): half its chiral blocks per parity,

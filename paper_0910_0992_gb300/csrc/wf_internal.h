@@ -103,6 +103,8 @@ struct MArgs {
   const Cx<R>* pl;     // per-line boundary link P (axial frame)
   const Cx<R>* us_out; // forward spatial links, own parity
   const Cx<R>* us_nbr; // forward spatial links, other parity
+  const int4* fx_out;  // R = double: both in fixed point (wf_fixed.cuh)
+  const int4* fx_nbr;
   const Cx<R>* x;      // out = x + a * (M psi) if x != nullptr
   R a;
   int swap;            // read psi and write the result with the spin halves exchanged (M^dag = S M S)
@@ -111,6 +113,11 @@ struct MArgs {
 };
 template <typename R>
 void launch_apply_M(const MArgs<R>& a, bool axial, cudaStream_t s);
+// FP64 with the spatial hops in block fixed point (wf_fixed.cu): the links' limbs (n entries), out = hop
+// (post: with the post-axpy and the exchange of the halves) and M
+void launch_links_fx(const Cx<double>* in, int4* out, size_t n, cudaStream_t s);
+void launch_hop_fx(const LineArgs<double>& a, bool post, cudaStream_t s);
+void launch_apply_M_fx(const MArgs<double>& a, bool axial, cudaStream_t s);
 // the long-line variants (lines of 129 to 256 slots; wf_kernels_long_f32.cu, wf_kernels_long_f64.cu)
 template <typename R>
 void launch_line_long(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s);

@@ -67,20 +67,23 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
     launch_line_long<R>(a, kind, axial, s);
     return;
   }
+  // FP64 kernels only load their own site: their hops have run in fixed point (launch_line)
+  constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;
+  constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
 #define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV><<<b, kLineThreads, 0, s>>>(a)
   if (axial) {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(true, SRC_LOAD, OP_FWD, OP_SKIP); break;
-      case LK_SCHUR_B: WF_KL(true, SRC_HOP, OP_FWD, OP_BWD); break;
-      case LK_SCHUR_C: WF_KL(true, SRC_HOP, OP_COPY, OP_BWD); break;
-      default: WF_KL(true, -1, -1, -1); break;
+      case LK_SCHUR_B: WF_KL(true, HOP, OP_FWD, OP_BWD); break;
+      case LK_SCHUR_C: WF_KL(true, HOP, OP_COPY, OP_BWD); break;
+      default: WF_KL(true, ANY, -1, -1); break;
     }
   } else {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(false, SRC_LOAD, OP_FWD, OP_SKIP); break;
-      case LK_SCHUR_B: WF_KL(false, SRC_HOP, OP_FWD, OP_BWD); break;
-      case LK_SCHUR_C: WF_KL(false, SRC_HOP, OP_COPY, OP_BWD); break;
-      default: WF_KL(false, -1, -1, -1); break;
+      case LK_SCHUR_B: WF_KL(false, HOP, OP_FWD, OP_BWD); break;
+      case LK_SCHUR_C: WF_KL(false, HOP, OP_COPY, OP_BWD); break;
+      default: WF_KL(false, ANY, -1, -1); break;
     }
   }
 #undef WF_KL
@@ -135,6 +138,25 @@ void launch_line(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s) {
       launch_line_wide(line_args_df(a), kind, s);
       return;
     }
+    // FP64 hops: the hop in fixed point into out, then the time-line operations there in place (a line
+    // is read in full by its warp before it is written)
+    if (kind == LK_SCHUR_B || kind == LK_SCHUR_C || kind == LK_HOP || (kind == LK_GENERIC && a.src == SRC_HOP)) {
+      LineArgs<double> b = a;
+      if (kind == LK_SCHUR_B || kind == LK_SCHUR_C) {
+        b.opu = kind == LK_SCHUR_B ? OP_FWD : OP_COPY;
+        b.opl = OP_BWD;
+      }
+      const bool plain = kind == LK_HOP || (b.opu == OP_COPY && b.opl == OP_COPY);
+      launch_hop_fx(b, plain, s);
+      if (plain && !b.norm2) return;
+      if (plain) throw Error(1, "FP64 hop: no norm of a plain hop");
+      b.src = SRC_LOAD;
+      b.src_up = b.out;
+      b.src_lo = b.out + 6 * b.g.tp;
+      b.xpre = nullptr;
+      launch_line_impl<double>(b, kind == LK_SCHUR_B || kind == LK_SCHUR_C ? kind : LK_GENERIC, axial, s);
+      return;
+    }
   }
   launch_line_impl<R>(a, kind, axial, s);
 }
@@ -174,6 +196,10 @@ template void launch_line<double>(const LineArgs<double>&, int, bool, cudaStream
 
 template <typename R>
 void launch_apply_M(const MArgs<R>& a, bool axial, cudaStream_t s) {
+  if constexpr (std::is_same<R, double>::value) {
+    launch_apply_M_fx(a, axial, s);
+    return;
+  } else {
   if (a.g.n < 1 || a.g.n > NMAX_LONG) throw Error(1, "unsupported sites per lane");
   const int lines = a.nrhs * a.g.Nl;
   const int warps = (lines + a.g.lpw - 1) / a.g.lpw;
@@ -187,6 +213,7 @@ void launch_apply_M(const MArgs<R>& a, bool axial, cudaStream_t s) {
   else
     k_apply_M<R, false, NMAX><<<blocks, kLineThreads, 0, s>>>(a);
   WF_CUDA(cudaGetLastError());
+  }
 }
 template void launch_apply_M<float>(const MArgs<float>&, bool, cudaStream_t);
 template void launch_apply_M<double>(const MArgs<double>&, bool, cudaStream_t);

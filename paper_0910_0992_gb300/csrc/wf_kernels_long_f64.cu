@@ -3,5 +3,4 @@
 
 namespace wf {
 template void launch_line_long<double>(const LineArgs<double>&, int, bool, cudaStream_t);
-template void launch_apply_M_long<double>(const MArgs<double>&, bool, cudaStream_t);
 }  // namespace wf

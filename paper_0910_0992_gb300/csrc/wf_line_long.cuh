@@ -11,20 +11,22 @@ template <typename R>
 void launch_line_long(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s) {
   if (a.g.n <= NMAX || a.g.n > NMAX_LONG || a.h16) throw Error(1, "long-line kernel: unsupported line layout");
   const int b = line_blocks(a);
+  constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;  // as in launch_line
+  constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
 #define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV, false, NMAX_LONG><<<b, kLineThreads, 0, s>>>(a)
   if (axial) {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(true, SRC_LOAD, OP_FWD, OP_SKIP); break;
-      case LK_SCHUR_B: WF_KL(true, SRC_HOP, OP_FWD, OP_BWD); break;
-      case LK_SCHUR_C: WF_KL(true, SRC_HOP, OP_COPY, OP_BWD); break;
-      default: WF_KL(true, -1, -1, -1); break;
+      case LK_SCHUR_B: WF_KL(true, HOP, OP_FWD, OP_BWD); break;
+      case LK_SCHUR_C: WF_KL(true, HOP, OP_COPY, OP_BWD); break;
+      default: WF_KL(true, ANY, -1, -1); break;
     }
   } else {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(false, SRC_LOAD, OP_FWD, OP_SKIP); break;
-      case LK_SCHUR_B: WF_KL(false, SRC_HOP, OP_FWD, OP_BWD); break;
-      case LK_SCHUR_C: WF_KL(false, SRC_HOP, OP_COPY, OP_BWD); break;
-      default: WF_KL(false, -1, -1, -1); break;
+      case LK_SCHUR_B: WF_KL(false, HOP, OP_FWD, OP_BWD); break;
+      case LK_SCHUR_C: WF_KL(false, HOP, OP_COPY, OP_BWD); break;
+      default: WF_KL(false, ANY, -1, -1); break;
     }
   }
 #undef WF_KL
