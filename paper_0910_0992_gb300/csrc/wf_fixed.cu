@@ -159,8 +159,8 @@ __device__ __forceinline__ bool site_at(const Geom& g, int nrhs, int& rhs, int& 
   return in;
 }
 
-// out = v, v = xpre + apre D_s src (xpre null: D_s src); post: then out = xpost + apost v, with the
-// spin halves exchanged if swap_out. Padding slots zero (post: xpost).
+// out = v, v = xpre + apre D_s src (xpre null: D_s src), with the spin halves exchanged if swap_out;
+// post: out = xpost + apost v. Padding slots zero (post: xpost).
 __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_hop_fx(const LineArgs<double> A, int post) {
   const Geom& g = A.g;
   int rhs, l, sl, t;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_hop_fx(const LineA
   }
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
-    const int so = post && A.swap_out ? (s + 2) % 4 : s;
+    const int so = A.swap_out ? (s + 2) % 4 : s;
     Vec3<double> v;
     if (post && A.xpost)
       v = vaxpy(A.apost * unit, h[s], ldvec(A.xpost + base + 3 * so * tp, tp, sl));

@@ -62,7 +62,7 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
     }
   }
   if (a.g.n < 1 || a.g.n > NMAX_LONG) throw Error(1, "unsupported sites per lane");
-  const int b = line_blocks(a);
+  const int th = line_threads(a), b = line_blocks(a, th);
   if (a.g.n > NMAX) {  // lines longer than 128 slots: the long-line variant (wf_kernels_long_*.cu)
     launch_line_long<R>(a, kind, axial, s);
     return;
@@ -70,7 +70,7 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
   // FP64 kernels only load their own site: their hops have run in fixed point (launch_line)
   constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;
   constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
-#define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV><<<b, kLineThreads, 0, s>>>(a)
+#define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV><<<b, th, 0, s>>>(a)
   if (axial) {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(true, SRC_LOAD, OP_FWD, OP_SKIP); break;
@@ -150,9 +150,9 @@ void launch_line(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s) {
       launch_hop_fx(b, plain, s);
       if (plain && !b.norm2) return;
       if (plain) throw Error(1, "FP64 hop: no norm of a plain hop");
-      b.src = SRC_LOAD;
-      b.src_up = b.out;
-      b.src_lo = b.out + 6 * b.g.tp;
+      b.src = SRC_LOAD;  // with swap_out the hop has stored the halves exchanged: each is read where it goes
+      b.src_up = b.out + (b.swap_out ? 6 * b.g.tp : 0);
+      b.src_lo = b.out + (b.swap_out ? 0 : 6 * b.g.tp);
       b.xpre = nullptr;
       launch_line_impl<double>(b, kind == LK_SCHUR_B || kind == LK_SCHUR_C ? kind : LK_GENERIC, axial, s);
       return;

@@ -17,8 +17,8 @@ constexpr int kLineThreads = 128;
 #endif
 // resident CTAs per SM the line kernels are compiled for (3: 168 registers; measured best
 // on GB300 against 1 and 4, where 4 spills)
-template <typename R, bool AX, bool FWD, int NM>
-__device__ __forceinline__ void solve_half(Vec3<R> (&v)[NM][4], int s0, const LineArgs<R>& A, int l, int jj) {
+template <typename R, bool AX, bool FWD, int NM, int W>
+__device__ __forceinline__ void solve_half(Vec3<R> (&v)[NM][W], int s0, const LineArgs<R>& A, int l, int jj) {
   constexpr int NS = sizeof(R) == 4 ? 2 : 1;
   const Geom& g = A.g;
 #pragma unroll
@@ -29,7 +29,7 @@ __device__ __forceinline__ void solve_half(Vec3<R> (&v)[NM][4], int s0, const Li
 #pragma unroll
       for (int s = 0; s < NS; ++s) w[m][s] = v[m][s0 + sp + s];
     if (AX)
-      tline_solve_axial<R, NS, FWD>(w, A.pl + (size_t)l * 9, A.lamb + (size_t)l * 9, g, jj, A.inv_mu, A.bc);
+      tline_solve_axial<R, NS, FWD>(w, A.lamf + (size_t)l * 9, g, jj, A.inv_mu, A.bc);
     else
       tline_solve_general<R, NS, FWD>(w, A.ut + (size_t)l * NLINK_C * g.tp,
                                       (FWD ? A.lamf : A.lamb) + (size_t)l * 9, g, jj, A.inv_mu, A.bc);
@@ -40,12 +40,50 @@ __device__ __forceinline__ void solve_half(Vec3<R> (&v)[NM][4], int s0, const Li
   }
 }
 
-template <typename R, bool AX, int NM>
-__device__ __forceinline__ void apply_op(int op, Vec3<R> (&v)[NM][4], int s0, const LineArgs<R>& A, int l, int jj) {
+template <typename R, bool AX, int NM, int W>
+__device__ __forceinline__ void apply_op(int op, Vec3<R> (&v)[NM][W], int s0, const LineArgs<R>& A, int l, int jj) {
   if (op == OP_FWD)
     solve_half<R, AX, true>(v, s0, A, l, jj);
   else if (op == OP_BWD)
     solve_half<R, AX, false>(v, s0, A, l, jj);
+}
+
+// store spin s of half h at the lane's site m (slot sl, in the line or padding): out = xpost + apost v or v
+template <typename R, bool H>
+__device__ __forceinline__ void store_spin(const LineArgs<R>& A, size_t base, int h, int s, int sl, bool valid,
+                                           const Vec3<R>& v, R& nrm) {
+  const int tp = A.g.tp;
+  const int comp0 = (A.swap_out ? 1 - h : h) * 6 + s * 3;
+  Vec3<R> val = valid ? v : vzero<R>();
+  if (A.xpost) val = vaxpy(A.apost, val, ldv<R, H>(A.xpost, base + comp0 * tp, tp, sl));
+  stv<R, H>(A.out, base + comp0 * tp, tp, sl, val);
+  if (A.norm2) nrm += vnorm2(val);
+}
+
+// One spin half of a line kernel that loads its own site: load, pre-axpy, time-line operation, store
+template <typename R, bool AX, bool H, int NM>
+__device__ __forceinline__ void load_half(const LineArgs<R>& A, int h, int op, size_t base, int l, int jj, bool active,
+                                          R& nrm) {
+  const Geom& g = A.g;
+  const int tp = g.tp, n = g.n;
+  const Cx<R>* src = h ? A.src_lo : A.src_up;
+  Vec3<R> v[NM][2];
+#pragma unroll
+  for (int m = 0; m < NM; ++m)
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int sl = m * g.lpl + jj;
+      v[m][s] = m < n ? ldv<R, H>(src, base + 3 * s * tp, tp, sl) : vzero<R>();
+      if (A.xpre && m < n) v[m][s] = vaxpy(A.apre, v[m][s], ldv<R, H>(A.xpre, base + (6 * h + 3 * s) * tp, tp, sl));
+    }
+  apply_op<R, AX>(op, v, 0, A, l, jj);
+  if (!active) return;
+#pragma unroll
+  for (int m = 0; m < NM; ++m) {
+    if (m >= n) continue;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) store_spin<R, H>(A, base, h, s, m * g.lpl + jj, jj * n + m < g.T, v[m][s], nrm);
+  }
 }
 
 // SRC, OPU, OPL < 0: taken from the arguments at run time
@@ -77,6 +115,22 @@ __device__ __forceinline__ void line_body(const LineArgs<R>& A, int blk) {
   const size_t base = ((size_t)rhs * g.Nl + l) * NSPIN_C * tp;
   if (A.active && g.lpw == 1 && !A.active[rhs]) return;  // one line per warp: the whole warp leaves
 
+  R nrm = R(0);
+  const bool want_norm = A.norm2 != nullptr;
+  if constexpr (SRC == SRC_LOAD) {
+    // one spin half after the other: half the registers of a whole spinor per site (a half is written
+    // where it was read when the kernel works in place)
+    if constexpr (OPU >= 0) {
+      if (opu != OP_SKIP) load_half<R, AX, H, NM>(A, 0, opu, base, l, jj, active, nrm);
+      if (opl != OP_SKIP) load_half<R, AX, H, NM>(A, 1, opl, base, l, jj, active, nrm);
+    } else {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        const int op = h ? opl : opu;
+        if (op != OP_SKIP) load_half<R, AX, H, NM>(A, h, op, base, l, jj, active, nrm);
+      }
+    }
+  } else {
   Vec3<R> v[NM][4];
   if (src == SRC_HOP) {
     hop_spatial<R>(v, A, rhs, l, jj);
@@ -105,29 +159,19 @@ __device__ __forceinline__ void line_body(const LineArgs<R>& A, int blk) {
   apply_op<R, AX>(opu, v, 0, A, l, jj);
   apply_op<R, AX>(opl, v, 2, A, l, jj);
 
-  R nrm = R(0);
-  const bool want_norm = A.norm2 != nullptr;
   if (active) {
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
       if (m >= n) continue;
-      const int sl = m * g.lpl + jj;
-      const bool valid = jj * n + m < g.T;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int op = h ? opl : opu;
-        if (op == OP_SKIP) continue;
-        const int dh = A.swap_out ? 1 - h : h;
+        if ((h ? opl : opu) == OP_SKIP) continue;
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-          const int comp0 = dh * 6 + s * 3;
-          Vec3<R> val = valid ? v[m][2 * h + s] : vzero<R>();
-          if (A.xpost) val = vaxpy(A.apost, val, ldv<R, H>(A.xpost, base + comp0 * tp, tp, sl));
-          stv<R, H>(A.out, base + comp0 * tp, tp, sl, val);
-          if (want_norm) nrm += vnorm2(val);
-        }
+        for (int s = 0; s < 2; ++s)
+          store_spin<R, H>(A, base, h, s, m * g.lpl + jj, jj * n + m < g.T, v[m][2 * h + s], nrm);
       }
     }
+  }
   }
   if (want_norm) {
     // lanes of one line share rhs; reduce over the warp per line group, one atomic per line
@@ -154,11 +198,16 @@ __global__ void __launch_bounds__(kLineThreads, LineMinBlocks<R>::value) k_line_
   line_body<R, AX, SRC, OPU, OPL>(M.a[k], (int)blockIdx.x - M.blk0[k]);
 }
 
+inline int line_warps(const Geom& g, int nrhs) { return (nrhs * g.Nl + g.lpw - 1) / g.lpw; }
 template <typename R>
-inline int line_blocks(const LineArgs<R>& a) {
-  const int lines = a.nrhs * a.g.Nl;
-  const int warps = (lines + a.g.lpw - 1) / a.g.lpw;
-  return (warps * 32 + kLineThreads - 1) / kLineThreads;
+inline int line_blocks(const LineArgs<R>& a, int threads = kLineThreads) {
+  return (line_warps(a.g, a.nrhs) * 32 + threads - 1) / threads;
+}
+// CTA size: one warp where the lattice has fewer than four per SM, so that they spread over all SMs
+// (an FP64 warp then shares an SM's FP64 pipe with no other; K-a in FP64 on 4^3 x 16: 17 -> 14 us)
+template <typename R>
+inline int line_threads(const LineArgs<R>& a) {
+  return line_warps(a.g, a.nrhs) < 4 * 152 ? 32 : kLineThreads;
 }
 
 // ----------------------------------------------------------------------------

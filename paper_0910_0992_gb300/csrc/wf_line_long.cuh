@@ -10,10 +10,10 @@ namespace wf {
 template <typename R>
 void launch_line_long(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s) {
   if (a.g.n <= NMAX || a.g.n > NMAX_LONG || a.h16) throw Error(1, "long-line kernel: unsupported line layout");
-  const int b = line_blocks(a);
+  const int th = line_threads(a), b = line_blocks(a, th);
   constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;  // as in launch_line
   constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
-#define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV, false, NMAX_LONG><<<b, kLineThreads, 0, s>>>(a)
+#define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV, false, NMAX_LONG><<<b, th, 0, s>>>(a)
   if (axial) {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(true, SRC_LOAD, OP_FWD, OP_SKIP); break;

@@ -93,7 +93,7 @@ __device__ __forceinline__ void solve_half_axial(Vec3<float> (&v)[NMAX][4], int 
     w[m][0] = v[m][s0];
     w[m][1] = v[m][s0 + 1];
   }
-  tline_solve_axial<float, 2, FWD>(w, A.pl + (size_t)l * 9, A.lamb + (size_t)l * 9, A.g, jj, A.inv_mu, A.bc);
+  tline_solve_axial<float, 2, FWD>(w, A.lamf + (size_t)l * 9, A.g, jj, A.inv_mu, A.bc);
 #pragma unroll
   for (int m = 0; m < NMAX; ++m) {
     v[m][s0] = w[m][0];
