@@ -494,12 +494,12 @@ void schur_apply(wf_handle* h, const Cx<R>* x, Cx<R>* out, int dagger, int nrhs,
     }
   }
   {
-    Prof P(h, pname<R>("schur_b_hop_tsolve"));
+    Prof P(h, pname<R>("schur_b_hop_tsolve"), sizeof(R) == 8 ? 2 : 1);
     launch_schur_hop<R>(h, ab, LK_SCHUR_B, tma);
   }
   {
     if (norm2) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
-    Prof P(h, pname<R>("schur_c_hop_tinv_axpy"));
+    Prof P(h, pname<R>("schur_c_hop_tinv_axpy"), sizeof(R) == 8 ? 2 : 1);
     launch_schur_hop<R>(h, ac, LK_SCHUR_C, tma);
   }
 }

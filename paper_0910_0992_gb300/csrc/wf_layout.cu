@@ -2,6 +2,7 @@
 // internal line layout, gauge ingest, and the per-line wrap-around matrices Lambda.
 #include <algorithm>
 
+#include "wf_fixed.cuh"
 #include "wf_internal.h"
 
 namespace wf {
@@ -37,8 +38,9 @@ __device__ __forceinline__ void site_coords(const Geom& g, size_t site, int& x, 
 // stays in registers for all sources the CTA loops over. Shared-memory rows of 13 elements keep
 // both orders free of bank conflicts.
 //
-// The rotation's 144 multiply-adds per site bound the FP64 form (GB300: two FP64 FMAs per clock and
-// SM; 0.10 ms of an 0.08 ms floor for a full field of 12^3 x 48 x 4 sources). FP32 fields take
+// The rotation's 144 multiply-adds per site would bound these kernels (GB300: two FP64 FMAs per clock
+// and SM): FP64 fields rotate in fixed point (rotate3_fx; full field of 24^3 x 128 x
+// 12 sources, import 5.1 -> 2.3 ms, export 5.1 -> 2.9; 12^3 x 48 x 4 0.10 -> 0.056 and 0.066 ms), FP32 fields with
 // rotate3_split instead, whose products are exact FP32 ones (below). Spins one after another and six
 // CTAs per SM: the loads of one CTA overlap the arithmetic of the others (unrolled, at 4 CTAs per SM,
 // 1.4 times slower). Measured, one odd field of 24^3 x 128 x 12 sources to and from FP32 (3.1 GB,
@@ -106,9 +108,65 @@ __device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl,
     split_unit(e.im, G.h[k].im, G.l[k].im);
   }
 }
-__device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl, int tp, int sl, Mat3<double>& G) {
+// A rotation matrix in fixed point (wf_fixed.cuh): limbs of g 2^55
+struct FxMat {
+  int2 re[9], im[9];
+};
+__device__ __forceinline__ int2 fx_limbs(long long v) { return make_int2((int)(v >> 28), (int)v & 0xfffffff); }
+__device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl, int tp, int sl, FxMat& G) {
 #pragma unroll
-  for (int k = 0; k < 9; ++k) G.e[k] = gl[(size_t)k * tp + sl];
+  for (int k = 0; k < 9; ++k) {
+    const Cx<double> e = gl[(size_t)k * tp + sl];
+    G.re[k] = fx_limbs(fx_from(e.re, 1023));  // |g| <= 1 + 1e-9: exponents up to 1023
+    G.im[k] = fx_limbs(fx_from(e.im, 1023));
+  }
+}
+// w = g v (DAG: g^dag v), the six numbers of v sharing one exponent; false (w unset) outside the
+// fixed-point range. Four spins of a site: about 1100 integer instructions and 24 conversions against 144
+// FP64 multiply-adds, i.e. some 20 clocks per site and SM against 72.
+template <bool DAG>
+__device__ __forceinline__ bool rotate3_fx(const FxMat& G, const double (&v)[6], double (&w)[6]) {
+  unsigned mx = 0;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7fffffffu);
+  const int e = (int)(mx >> 20), E = max(e, kFxMinExp);
+  if (mx != 0 && (e < kFxMinExp || e >= kFxMaxExp)) return false;
+  int2 h[6], n[6];  // limbs of v and of -v
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    h[i] = fx_limbs(fx_from(v[i], E));
+    n[i] = make_int2(-h[i].x, -h[i].y);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    long long H[2] = {}, X[2] = {};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int2 r = G.re[DAG ? 3 * b + a : 3 * a + b], i = G.im[DAG ? 3 * b + a : 3 * a + b];
+      // re: gr vr -+ gi vi, im: gr vi +- gi vr
+      const int2 vr = h[2 * b], vi = h[2 * b + 1], xi = DAG ? vi : n[2 * b + 1], xr = DAG ? n[2 * b] : vr;
+      fx_mac(H[0], r.x, vr.x);
+      fx_mac(X[0], r.x, vr.y);
+      fx_mac(X[0], r.y, vr.x);
+      fx_mac(H[0], i.x, xi.x);
+      fx_mac(X[0], i.x, xi.y);
+      fx_mac(X[0], i.y, xi.x);
+      fx_mac(H[1], r.x, vi.x);
+      fx_mac(X[1], r.x, vi.y);
+      fx_mac(X[1], r.y, vi.x);
+      fx_mac(H[1], i.x, xr.x);
+      fx_mac(X[1], i.x, xr.y);
+      fx_mac(X[1], i.y, xr.x);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      // g v = (H 2^56 + X 2^28) 2^-55 in units of 2^(E - 1023 - 55): H + X / 2^28 in units of 2^(E - 1077)
+      const double x = (double)(H[q] + (X[q] >> 28));
+      const int hi = __double2hiint(x);
+      w[2 * a + q] = __hiloint2double(hi ? hi + ((E - 1077) << 20) : 0, __double2loint(x));
+    }
+  }
+  return true;
 }
 
 // s + c = g v (DAG: g^dag v) for a vector v = f + lo (lo of relative size 2^-20 at most, or zero):
@@ -158,24 +216,30 @@ __device__ __forceinline__ void rotate3_split(const SplitMat& G, const float (&f
 }
 
 // One spin of a site on import: in (shared memory, 3 FP64 elements, negated for gamma_5) rotated by G
-// into out (components tp elements apart)
-__device__ __forceinline__ void import_spin(const Mat3<double>& G, const Cx<double>*, int, const Cx<double>* in, bool neg,
-                                            Cx<double>* out, int tp) {
-  Vec3<double> v;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) v.c[c] = neg ? mk<double>(-in[c].re, -in[c].im) : in[c];
-  const Vec3<double> w = matvec(G, v);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) out[(size_t)c * tp] = w.c[c];
-}
-// the same in FP64 for FP32 fields: extreme magnitudes, infinities, NaN (rare, kept out of line)
-__device__ __noinline__ void import_spin_wide(const Cx<double>* gl, const Cx<double>* in, bool neg, Cx<float>* out,
-                                              int tp) {
+// into out (components tp elements apart). The _wide forms are the rotation in FP64, out of line, for
+// extreme magnitudes, infinities and NaN.
+template <typename R>
+__device__ __noinline__ void import_spin_wide(const Cx<double>* gl, const Cx<double>* in, bool neg, Cx<R>* out, int tp) {
   for (int a = 0; a < 3; ++a) {
     Cx<double> w = czero<double>();
     for (int b = 0; b < 3; ++b) w = cfma(w, gl[(size_t)(3 * a + b) * tp], neg ? mk<double>(-in[b].re, -in[b].im) : in[b]);
-    out[(size_t)a * tp] = mk<float>((float)w.re, (float)w.im);
+    out[(size_t)a * tp] = mk<R>((R)w.re, (R)w.im);
   }
+}
+__device__ __forceinline__ void import_spin(const FxMat& G, const Cx<double>* gl, int sl, const Cx<double>* in, bool neg,
+                                            Cx<double>* out, int tp) {
+  double v[6], w[6];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    v[2 * c] = neg ? -in[c].re : in[c].re;
+    v[2 * c + 1] = neg ? -in[c].im : in[c].im;
+  }
+  if (!rotate3_fx<false>(G, v, w)) {
+    import_spin_wide<double>(gl + sl, in, neg, out, tp);
+    return;
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[(size_t)c * tp] = mk<double>(w[2 * c], w[2 * c + 1]);
 }
 __device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>* gl, int sl, const Cx<double>* in,
                                             bool neg, Cx<float>* out, int tp) {
@@ -188,7 +252,7 @@ __device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>*
     ok &= split_double(neg ? -v.im : v.im, f[2 * k + 1], lo[2 * k + 1]);
   }
   if (!ok) {
-    import_spin_wide(gl + sl, in, neg, out, tp);
+    import_spin_wide<float>(gl + sl, in, neg, out, tp);
     return;
   }
   float s[6], c[6];
@@ -197,19 +261,29 @@ __device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>*
   for (int k = 0; k < 3; ++k) out[(size_t)k * tp] = mk<float>(s[2 * k] + c[2 * k], s[2 * k + 1] + c[2 * k + 1]);
 }
 // One spin of a site on export: v rotated by G^dag into out (shared memory, 3 FP64 elements)
-__device__ __forceinline__ void export_spin(const Mat3<double>& G, const Cx<double>*, int, int, const Vec3<double>& v,
-                                            bool neg, Cx<double>* out) {
-  const Vec3<double> w = matvec_dag(G, v);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) out[c] = neg ? mk<double>(-w.c[c].re, -w.c[c].im) : w.c[c];
-}
-__device__ __noinline__ void export_spin_wide(const Cx<double>* gl, int tp, Vec3<float> v, bool neg, Cx<double>* out) {
+template <typename R>
+__device__ __noinline__ void export_spin_wide(const Cx<double>* gl, int tp, Vec3<R> v, bool neg, Cx<double>* out) {
   for (int a = 0; a < 3; ++a) {
     Cx<double> w = czero<double>();
     for (int b = 0; b < 3; ++b)
       w = cfmaconj(w, gl[(size_t)(3 * b + a) * tp], mk<double>((double)v.c[b].re, (double)v.c[b].im));
     out[a] = neg ? mk<double>(-w.re, -w.im) : w;
   }
+}
+__device__ __forceinline__ void export_spin(const FxMat& G, const Cx<double>* gl, int tp, int sl, const Vec3<double>& v,
+                                            bool neg, Cx<double>* out) {
+  double x[6], w[6];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    x[2 * c] = neg ? -v.c[c].re : v.c[c].re;
+    x[2 * c + 1] = neg ? -v.c[c].im : v.c[c].im;
+  }
+  if (!rotate3_fx<true>(G, x, w)) {
+    export_spin_wide<double>(gl + sl, tp, v, neg, out);
+    return;
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) out[c] = mk<double>(w[2 * c], w[2 * c + 1]);
 }
 __device__ __forceinline__ void export_spin(const SplitMat& G, const Cx<double>* gl, int tp, int sl,
                                             const Vec3<float>& v, bool neg, Cx<double>* out) {
@@ -222,7 +296,7 @@ __device__ __forceinline__ void export_spin(const SplitMat& G, const Cx<double>*
     ok &= a == 0 || (a >= (47u << 23) && a < (227u << 23));  // [2^-80, 2^100)
   }
   if (!ok) {
-    export_spin_wide(gl + sl, tp, v, neg, out);
+    export_spin_wide<float>(gl + sl, tp, v, neg, out);
     return;
   }
   const float lo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -244,7 +318,7 @@ struct RotationOf {
 };
 template <>
 struct RotationOf<double> {
-  typedef Mat3<double> type;
+  typedef FxMat type;
 };
 
 // Block and thread of a tile launch -> parity, lines and times. Caller's side: thread q < 96 moves
