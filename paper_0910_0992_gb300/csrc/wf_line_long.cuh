@@ -19,14 +19,24 @@ void launch_line_long(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s
       case LK_SCHUR_A: WF_KL(true, SRC_LOAD, OP_FWD, OP_SKIP); break;
       case LK_SCHUR_B: WF_KL(true, HOP, OP_FWD, OP_BWD); break;
       case LK_SCHUR_C: WF_KL(true, HOP, OP_COPY, OP_BWD); break;
-      default: WF_KL(true, ANY, -1, -1); break;
+      default:
+        if (a.src == SRC_LOAD)
+          WF_KL(true, SRC_LOAD, -1, -1);
+        else
+          WF_KL(true, ANY, -1, -1);
+        break;
     }
   } else {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(false, SRC_LOAD, OP_FWD, OP_SKIP); break;
       case LK_SCHUR_B: WF_KL(false, HOP, OP_FWD, OP_BWD); break;
       case LK_SCHUR_C: WF_KL(false, HOP, OP_COPY, OP_BWD); break;
-      default: WF_KL(false, ANY, -1, -1); break;
+      default:
+        if (a.src == SRC_LOAD)
+          WF_KL(false, SRC_LOAD, -1, -1);
+        else
+          WF_KL(false, ANY, -1, -1);
+        break;
     }
   }
 #undef WF_KL
