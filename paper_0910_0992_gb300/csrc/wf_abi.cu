@@ -498,7 +498,7 @@ void schur_apply(wf_handle* h, const Cx<R>* x, Cx<R>* out, int dagger, int nrhs,
     launch_schur_hop<R>(h, ab, LK_SCHUR_B, tma);
   }
   {
-    if (norm2) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
+    if (norm2 && !h->norm_cleared) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
     Prof P(h, pname<R>("schur_c_hop_tinv_axpy"), sizeof(R) == 8 ? 2 : 1);
     launch_schur_hop<R>(h, ac, LK_SCHUR_C, tma);
   }
@@ -642,6 +642,10 @@ std::vector<int> cgnr(wf_handle* h, const OpFn<R>& A, const OpFn<double>& A64, c
   int* upd = ist + 3 * nrhs;  // sources whose x update of this iteration is still pending
   double* lim = h->buf<double>("cg_limits", 2 * (size_t)nrhs);
   double* partial = h->buf<double>("cg_partial", 1024 * (size_t)nrhs);
+  unsigned* counter = h->buf<unsigned>("cg_counter", 2 * (size_t)nrhs);
+  WF_CUDA(cudaMemsetAsync(counter, 0, 2 * nrhs * sizeof(unsigned), s));
+  const CgState cst{active, state, dits, upd, lim, lim + nrhs, counter};
+  const CgAdvance adv{gam, gnew, qq, counter + nrhs};
   std::vector<int> act(nrhs, 1), iters(nrhs, 0);
   WF_CUDA(cudaMemcpyAsync(active, act.data(), nrhs * sizeof(int), cudaMemcpyHostToDevice, s));
 
@@ -729,12 +733,12 @@ std::vector<int> cgnr(wf_handle* h, const OpFn<R>& A, const OpFn<double>& A64, c
   // over the vectors less per iteration); a source that stops at the check still takes it there
   auto iteration = [&]() {
     A(p, q, 0, qq);  // q = A p, |q|^2
-    { Prof P(h, pname<R>("cg_xr"), 2); launch_cg_xr<R>(nullptr, r, p, q, n, nrhs, gam, qq, active, partial, rr, s, offs, upd); }
-    { Prof P(h, "cg_check"); launch_cg_check(rr, active, state, dits, lim, lim + nrhs, nrhs, s); }
+    { Prof P(h, pname<R>("cg_r_check")); launch_cg_r_check<R>(r, q, n, nrhs, gam, qq, partial, rr, cst, s, offs); }
     A(r, sv, 1, gnew);  // s = A^dag r, |s|^2
-    { Prof P(h, pname<R>("cg_p")); launch_cg_p<R>(p, sv, n, nrhs, gnew, gam, active, s, offs, xacc, qq, upd); }
-    { Prof P(h, "copy_scalar"); launch_copy_scalar(gam, gnew, nrhs, s, active); }
+    { Prof P(h, pname<R>("cg_p")); launch_cg_p<R>(p, sv, n, nrhs, gnew, gam, active, s, offs, xacc, qq, upd, adv); }
   };
+  auto clear_norms = [&]() { WF_CUDA(cudaMemsetAsync(gnew, 0, 2 * nrhs * sizeof(double), s)); };  // gnew and qq
+  clear_norms();
 
   bool graphs = h->stream != 0 && !h->prof;
   if (const char* e = std::getenv("WF_GRAPH"))
@@ -789,8 +793,14 @@ std::vector<int> cgnr(wf_handle* h, const OpFn<R>& A, const OpFn<double>& A64, c
   // a reliable update) while the blocks run
   struct ActiveScope {
     wf_handle* h;
-    ActiveScope(wf_handle* hh, const int* a) : h(hh) { h->op_active = a; }
-    ~ActiveScope() { h->op_active = nullptr; }
+    ActiveScope(wf_handle* hh, const int* a) : h(hh) {
+      h->op_active = a;
+      h->norm_cleared = true;
+    }
+    ~ActiveScope() {
+      h->op_active = nullptr;
+      h->norm_cleared = false;
+    }
   } active_scope(h, active);
   std::vector<double> rr_prev(nrhs, 0.0), rrh(nrhs);
   int total = 0, nb = 1;
@@ -842,9 +852,10 @@ std::vector<int> cgnr(wf_handle* h, const OpFn<R>& A, const OpFn<double>& A64, c
       }
       if (any_resume) {
         WF_CUDA(cudaMemcpyAsync(active, resume.data(), nrhs * sizeof(int), cudaMemcpyHostToDevice, s));
+        clear_norms();  // operators that do not skip stopped sources have added to theirs
         A(r, sv, 1, gnew);
-        { Prof P(h, pname<R>("cg_p")); launch_cg_p<R>(p, sv, n, nrhs, gnew, gam, active, s, offs); }
-        { Prof P(h, "copy_scalar"); launch_copy_scalar(gam, gnew, nrhs, s, active); }
+        { Prof P(h, pname<R>("cg_p")); launch_cg_p<R>(p, sv, n, nrhs, gnew, gam, active, s, offs, nullptr, nullptr, nullptr, adv); }
+        clear_norms();  // and, here, to the masked ones'
       }
       upload_state();
     }
@@ -936,7 +947,7 @@ void schur_apply_h16(wf_handle* h, const Cx16* x, Cx16* out, int dagger, int nrh
     launch_hop_config(h, ab, LK_SCHUR_B);
   }
   {
-    if (norm2) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
+    if (norm2 && !h->norm_cleared) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
     Prof P(h, "schur_c_hop_tinv_axpy_h16");
     launch_hop_config(h, ac, LK_SCHUR_C);
   }
@@ -1460,7 +1471,7 @@ OpFn<float> joint_schur_op(const std::vector<JointPart>& parts, Cx<float>* ty, C
       launch_line_multi<float>(B2, LK_SCHUR_B, s);
       for (const auto& o : own) launch_own(o.second, o.second.b, LK_SCHUR_B);
     }
-    if (norm2) WF_CUDA(cudaMemsetAsync(norm2, 0, nr * sizeof(double), s));
+    if (norm2 && !h0->norm_cleared) WF_CUDA(cudaMemsetAsync(norm2, 0, nr * sizeof(double), s));
     {
       Prof P(h0, "schur_c_hop_tinv_axpy_f32", nb);
       launch_line_wide_multi<float>(C, LK_SCHUR_C, s);
@@ -1874,7 +1885,7 @@ void eo4d_apply(wf_handle* h, const Cx<R>* x, Cx<R>* out, int dagger, int nrhs, 
     a.stream_out = 1;
     a.out = out;
     a.norm2 = norm2;
-    if (norm2) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
+    if (norm2 && !h->norm_cleared) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
     Prof P(h, pname<R>("eo4d_dslash_oe_axpy"));
     launch_dslash4<R>(a, h->axial, h->stream);
     return;
@@ -1897,7 +1908,7 @@ void eo4d_apply(wf_handle* h, const Cx<R>* x, Cx<R>* out, int dagger, int nrhs, 
     a.stream_out = 1;  // the operator's result is next read by the solver's vector update
     a.out = out;
     a.norm2 = norm2;
-    if (norm2) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
+    if (norm2 && !h->norm_cleared) WF_CUDA(cudaMemsetAsync(norm2, 0, nrhs * sizeof(double), h->stream));
     Prof P(h, pname<R>("eo4d_dslash_oe_axpy"));
     launch_dslash4<R>(a, h->axial, h->stream);
   }

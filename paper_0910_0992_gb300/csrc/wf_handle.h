@@ -32,6 +32,8 @@ struct wf_handle {
   // while a CG runs: its device flags of active right-hand sides; the Schur operator's kernels
   // skip the others
   const int* op_active = nullptr;
+  // while a CG iteration runs: the norm accumulators it passes to the operator are already zero
+  bool norm_cleared = false;
   // gauge, per parity: U_t [Nl][9][tp], spatial [3][Nl][9][tp], Lambda [Nl][9]
   wf::DevBuf ut64[2], us64[2], lamb64[2], lamf64[2];
   wf::DevBuf ut32[2], us32[2], lamb32[2], lamf32[2];

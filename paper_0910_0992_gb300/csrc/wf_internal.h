@@ -159,6 +159,23 @@ void launch_f2d(const Cx<float>* in, Cx<double>* out, size_t n, cudaStream_t s);
 template <typename R>
 void launch_norm2(const Cx<R>* x, size_t n, int nrhs, double* partial, double* out, cudaStream_t s,
                   const size_t* offs = nullptr);
+// Device state of a CG (per right-hand side): active flags, state (0 running, 1 converged, 2 wants a
+// reliable update), iterations, upd (took the last r update), target^2 and reliable-update threshold^2,
+// and block counters (zero between kernels)
+struct CgState {
+  int *active, *state, *iters, *upd;
+  const double *tgt2, *ru2;
+  unsigned* counter;
+};
+// what k_cg_p does for the next iteration when it is done (counter null: nothing)
+struct CgAdvance {
+  double *gold, *gnew, *qq;
+  unsigned* counter;
+};
+// r -= alpha q, |r|^2 and the check of a CG iteration
+template <typename R>
+void launch_cg_r_check(Cx<R>* r, const Cx<R>* q, size_t n, int nrhs, const double* gamma, const double* qq,
+                       double* partial, double* rr, const CgState& c, cudaStream_t s, const size_t* offs = nullptr);
 // CG updates: launch_cg_xr does r -= alpha q (alpha = gamma / qq) with |r|^2 into rr_out, and
 // x += alpha p unless x is null; then upd (if given) records the right-hand sides that took the
 // update. launch_cg_p does p = s + beta p (beta = gamma_new / gamma_old) for the active ones and,
@@ -170,7 +187,7 @@ void launch_cg_xr(Cx<R>* x, Cx<R>* r, const Cx<R>* p, const Cx<R>* q, size_t n, 
 template <typename R>
 void launch_cg_p(Cx<R>* p, const Cx<R>* sv, size_t n, int nrhs, const double* gamma_new, const double* gamma_old,
                  const int* active, cudaStream_t s, const size_t* offs = nullptr, Cx<R>* x = nullptr,
-                 const double* qq = nullptr, const int* upd = nullptr);
+                 const double* qq = nullptr, const int* upd = nullptr, const CgAdvance& adv = CgAdvance());
 template <typename R>
 void launch_axpby(Cx<R>* y, const Cx<R>* x, size_t n, double a, double b, cudaStream_t s);  // y = a x + b y
 void launch_add_f_to_d(Cx<double>* y, const Cx<float>* x, size_t n, cudaStream_t s);      // y += x
