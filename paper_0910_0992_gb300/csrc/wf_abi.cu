@@ -1827,6 +1827,7 @@ EoArgs<R> eo_args(wf_handle* h, int par, int nrhs) {
     a.ut[p] = G.ut[p];
     a.pl[p] = G.pl[p];
     a.us[p] = G.us[p];
+    a.fx[p] = h->usfx[p].as<int4>();
   }
   a.inv_gf = (R)(1.0 / h->g.gamma_f);
   a.bc = (R)h->g.bc;

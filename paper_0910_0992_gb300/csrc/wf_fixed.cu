@@ -13,140 +13,35 @@ namespace {
 constexpr int kFxThreads = 128;
 constexpr int kFxMinBlocks = 4;  // CTAs per SM (3, without spills: 4 % slower; 24^3 x 128, 12 sources)
 
-// D_s at one site in FP64 (with its factor 1/2): the form of the rare sites whose neighbours are out of
-// the fixed-point range (NaN, infinities, exponents near the ends of FP64's). Out of line and rolled.
-__device__ __noinline__ void hop_site_fp64(const Geom& g, int parity, const Cx<double>* src_up,
-                                           const Cx<double>* src_lo, const Cx<double>* us_out,
-                                           const Cx<double>* us_nbr, int rhs, int l, int sl, double* out) {
-  const int tp = g.tp;
-  int nb[6];
-  neighbour_lines(g, parity, l, nb);
-  Vec3<double> h[4];
-  for (int s = 0; s < 4; ++s) h[s] = vzero<double>();
-#pragma unroll 1
-  for (int d = 0; d < 6; ++d) {
-    const int k = d >> 1, dir = d & 1, ln = nb[d];
-    const size_t sb = (size_t)(rhs * g.Nl + ln) * NSPIN_C * tp;
-    Mat3<double> U = ldmat(dir == 0 ? us_out + (size_t)(k * g.Nl + l) * 9 * tp : us_nbr + (size_t)(k * g.Nl + ln) * 9 * tp, tp, sl);
-    if (dir) U = dagger(U);
-    Vec3<double> s0, s1;
-    isigma(k, ldvec(src_lo + sb, tp, sl), ldvec(src_lo + sb + 3 * tp, tp, sl), s0, s1);
-    if (dir) {
-      s0 = vneg(s0);
-      s1 = vneg(s1);
-    }
-    const Vec3<double> w0 = matvec(U, vadd(ldvec(src_up + sb, tp, sl), s0));
-    const Vec3<double> w1 = matvec(U, vadd(ldvec(src_up + sb + 3 * tp, tp, sl), s1));
-    h[0] = vadd(h[0], w0);
-    h[1] = vadd(h[1], w1);
-    isigma(k, w0, w1, s0, s1);
-    if (!dir) {
-      s0 = vneg(s0);
-      s1 = vneg(s1);
-    }
-    h[2] = vadd(h[2], s0);
-    h[3] = vadd(h[3], s1);
+// direction d of line l's site (parity, source rhs, slot sl) in the line layout
+struct LineDir {
+  const Geom& g;
+  int x, y, z, rhs, l, sl;
+  const Cx<double>*src_up, *src_lo, *us_out, *us_nbr;
+  const int4 *fx_out, *fx_nbr;
+  __device__ __forceinline__ LineDir(const Geom& gg, int parity, int r, int ll, int s, const Cx<double>* up,
+                                     const Cx<double>* lo, const int4* fo, const int4* fn, const Cx<double>* uo,
+                                     const Cx<double>* un)
+      : g(gg), rhs(r), l(ll), sl(s), src_up(up), src_lo(lo), us_out(uo), us_nbr(un), fx_out(fo), fx_nbr(fn) {
+    line_coords(g, parity, l, x, y, z);
   }
-  for (int s = 0; s < 4; ++s)
-    for (int c = 0; c < 3; ++c) {
-      out[2 * (3 * s + c)] = 0.5 * h[s].c[c].re;
-      out[2 * (3 * s + c) + 1] = 0.5 * h[s].c[c].im;
-    }
-}
-
-// 16 bytes of device memory into shared memory, asynchronously
-__device__ __forceinline__ void fx_copy(int4* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
-               "l"(__cvta_generic_to_global(src))
-               : "memory");
-}
-// shared memory of a warp: 12 spinor and 9 link entries per lane. A lane reads only what it copied, so
-// the copies need no barrier: a direction's spinor arrives while the one before multiplies its link, its
-// link while it is projected.
-constexpr int kFxStage = 21 * 32;
-
-// h unit = D_s at one site: unit times the integer-valued h (so that the scale joins the next
-// multiply-add). stage: the lane's first entry
-__device__ __forceinline__ double hop_site_fx(const Geom& g, int parity, const Cx<double>* __restrict__ src_up,
-                                              const Cx<double>* __restrict__ src_lo, const int4* __restrict__ fx_out,
-                                              const int4* __restrict__ fx_nbr, const Cx<double>* us_out,
-                                              const Cx<double>* us_nbr, int rhs, int l, int sl, int4* stage,
-                                              Vec3<double> (&h)[4]) {
-  const int tp = g.tp, L = g.L;
-  int x, y, z;
-  line_coords(g, parity, l, x, y, z);
-  FxAcc f;
-  fx_clear(f);
-  // direction d's neighbour and link into the thread's own places of shared memory
-  auto neighbour = [&](int d) {
-    const int k = d >> 1, st = d & 1 ? L - 1 : 1;
+  __device__ __forceinline__ HopDir operator()(int d) const {
+    const int k = d >> 1, st = d & 1 ? g.L - 1 : 1;
     int nx = x + (k == 0 ? st : 0), ny = y + (k == 1 ? st : 0), nz = z + (k == 2 ? st : 0);
-    nx -= nx >= L ? L : 0;
-    ny -= ny >= L ? L : 0;
-    nz -= nz >= L ? L : 0;
-    return line_of(g, nx, ny, nz);
-  };
-  auto fetch_spinor = [&](int ln) {
-    const size_t sb = (size_t)(rhs * g.Nl + ln) * NSPIN_C * tp + sl;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      fx_copy(stage + 32 * c, src_up + sb + c * tp);
-      fx_copy(stage + 32 * (6 + c), src_lo + sb + c * tp);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  auto fetch_link = [&](int d, int ln) {
-    const int k = d >> 1;
-    const int4* lk = (d & 1 ? fx_nbr + (size_t)(k * g.Nl + ln) * 9 * tp : fx_out + (size_t)(k * g.Nl + l) * 9 * tp) + sl;
-#pragma unroll
-    for (int e = 0; e < 9; ++e) fx_copy(stage + 32 * (12 + e), lk + e * tp);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  int ln = neighbour(0);
-  fetch_spinor(ln);
-  fetch_link(0, ln);
-#pragma unroll 1
-  for (int d = 0; d < 6; ++d) {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    FxHalf q;
-    {
-      Vec3<double> v[4];
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) v[s].c[c] = *reinterpret_cast<const Cx<double>*>(stage + 32 * (3 * s + c));
-      fx_project(f, q, d, v);
-    }
-    if (d < 5) {
-      ln = neighbour(d + 1);
-      fetch_spinor(ln);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    fx_multiply(f, q, d, stage + 32 * 12, 32);
-    if (d < 5) fetch_link(d + 1, ln);
+    nx -= nx >= g.L ? g.L : 0;
+    ny -= ny >= g.L ? g.L : 0;
+    nz -= nz >= g.L ? g.L : 0;
+    const int ln = line_of(g, nx, ny, nz);
+    const size_t sb = (size_t)(rhs * g.Nl + ln) * NSPIN_C * g.tp + sl;
+    const size_t lk = (size_t)(k * g.Nl + (d & 1 ? ln : l)) * 9 * g.tp + sl;
+    HopDir q;
+    q.up = src_up + sb;
+    q.lo = src_lo + sb;
+    q.fx = (d & 1 ? fx_nbr : fx_out) + lk;
+    q.u = (d & 1 ? us_nbr : us_out) + lk;
+    return q;
   }
-  if (f.wide) {
-    double o[24];
-    hop_site_fp64(g, parity, src_up, src_lo, us_out, us_nbr, rhs, l, sl, o);
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) h[s].c[c] = mk<double>(o[2 * (3 * s + c)], o[2 * (3 * s + c) + 1]);
-    return 1.0;
-  }
-#pragma unroll
-  for (int s = 0; s < 4; ++s)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) h[s].c[c] = mk<double>((double)f.a[s][c][0], (double)f.a[s][c][1]);
-  return fx_unit(f);
-}
-
-__device__ __forceinline__ int4* fx_stage() {
-  extern __shared__ int4 fx_shared[];
-  return fx_shared + (threadIdx.x >> 5) * kFxStage + (threadIdx.x & 31);
-}
+};
 
 // thread -> (source, line, slot), slots fastest, in the line kernels' traversal
 __device__ __forceinline__ bool site_at(const Geom& g, int nrhs, int& rhs, int& l, int& sl, int& t) {
@@ -171,7 +66,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_hop_fx(const LineA
   Vec3<double> h[4];
   double unit = 0.0;
   if (t < g.T) {
-    unit = hop_site_fx(g, A.parity, A.src_up, A.src_lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr, rhs, l, sl, fx_stage(), h);
+    unit = hop_fx(LineDir(g, A.parity, rhs, l, sl, A.src_up, A.src_lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, h);
   } else {
 #pragma unroll
     for (int s = 0; s < 4; ++s) h[s] = vzero<double>();
@@ -193,10 +88,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_hop_fx(const LineA
   }
 }
 
-// The Wilson matrix on the output parity (k_apply_M of wf_line_kernels.cuh), one thread per site. The
-// wrap's P (axial frame) is applied by six lanes of the warp, one result component each: as one
-// lane's two 3x3 products it would hold the FP64 pipe for the whole warp as long as the site's
-// other FP64 operations together.
+// The Wilson matrix on the output parity (k_apply_M of wf_line_kernels.cuh), one thread per site
 template <bool AX>
 __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_apply_M_fx(const MArgs<double> A) {
   const Geom& g = A.g;
@@ -209,38 +101,17 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_apply_M_fx(const M
   Vec3<double> h[4];
   double unit = 0.0;
   if (site) {
-    unit = hop_site_fx(g, A.parity, A.psi_q + (A.swap ? 6 * tp : 0), A.psi_q + (A.swap ? 0 : 6 * tp), A.fx_out, A.fx_nbr,
-                       A.us_out, A.us_nbr, rhs, l, sl, fx_stage(), h);
+    const Cx<double>* up = A.psi_q + (A.swap ? 6 * tp : 0);
+    const Cx<double>* lo = A.psi_q + (A.swap ? 0 : 6 * tp);
+    unit = hop_fx(LineDir(g, A.parity, rhs, l, sl, up, lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, h);
   }
   // axial frame: spins 0-1 at t = 0 need P^dag psi(T - 1), spins 2-3 at t = T - 1 P psi(0)
   Vec3<double> wr[2];
   wr[0] = wr[1] = vzero<double>();
   if (AX) {
-    const int lane = threadIdx.x & 31;
-    const int q = lane < 6 ? lane : 0, qs = q / 3, qr = q - 3 * (q / 3);
-#pragma unroll
-    for (int end = 0; end < 2; ++end) {
-      unsigned m = __ballot_sync(0xffffffffu, site && t == (end ? T - 1 : 0));
-      const int from = slot_of(g, end ? 0 : T - 1);  // the slot read
-      while (m) {
-        const int w = __ffs(m) - 1;
-        m &= m - 1;
-        const int wl = __shfl_sync(0xffffffffu, l, w), wk = __shfl_sync(0xffffffffu, rhs, w);
-        // spins of the result half, read from the other half's place if the halves are exchanged
-        const int sr = ((end ? 2 : 0) + qs + (A.swap ? 2 : 0)) % 4;
-        const Cx<double>* x = A.psi_p + (((size_t)wk * g.Nl + wl) * NSPIN_C + 3 * sr) * tp + from;
-        const Cx<double>* P = A.pl + (size_t)wl * 9;
-        Cx<double> v = czero<double>();
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-          v = end ? cfma(v, P[3 * qr + b], x[(size_t)b * tp]) : cfmaconj(v, P[3 * b + qr], x[(size_t)b * tp]);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-          const Cx<double> u = shfl_idx(v, i, 32);
-          if (lane == w) wr[i / 3].c[i % 3] = u;
-        }
-      }
-    }
+    const Cx<double>* P = A.pl + (size_t)l * 9;
+    warp_link_product(site && t == 0, P, pp + (A.swap ? 6 * tp : 0) + slot_of(g, T - 1), tp, true, wr);
+    warp_link_product(site && t == T - 1, P, pp + (A.swap ? 0 : 6 * tp) + slot_of(g, 0), tp, false, wr);
   }
   if (!in) return;
   const Cx<double>* ut_line = AX ? nullptr : A.ut + (size_t)l * NLINK_C * tp;
@@ -276,8 +147,6 @@ __global__ void k_links_fx(const Cx<double>* __restrict__ in, int4* __restrict__
 
 // CTA size: one warp where the lattice is too small to give every SM four
 int fx_threads(size_t sites) { return sites < (size_t)152 * kFxThreads ? 32 : kFxThreads; }
-
-size_t fx_smem(int threads) { return (size_t)threads / 32 * kFxStage * sizeof(int4); }
 
 }  // namespace
 

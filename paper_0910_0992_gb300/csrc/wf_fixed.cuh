@@ -16,7 +16,7 @@
 // So the only roundings are those of v, U 2^58 and X / 2^28, each below an FP64 rounding of the
 // largest term: the result is at least as close to the exact one as FP64 arithmetic's (measured on
 // 12^3 x 48, M against 64-bit reference arithmetic: relative error 3.5e-15 either way). Spinors with a NaN,
-// an infinity or exponents near the ends of FP64's range take the FP64 form (hop_site_fp64).
+// an infinity or exponents near the ends of FP64's range take the FP64 form (hop_dir_fp64).
 #pragma once
 
 #include "wf_line.cuh"
@@ -178,5 +178,136 @@ __device__ __forceinline__ void fx_multiply(FxAcc& f, const FxHalf& q, int d, co
 
 // 2^(E - 1023 - 58): a unit of the accumulators times the projectors' factor 1/2 (E >= kFxMinExp)
 __device__ __forceinline__ double fx_unit(const FxAcc& f) { return __hiloint2double((f.E - 58) << 20, 0); }
+
+// ----------------------------------------------------------------------------
+// D_s at one site. dir(d) names direction d's operands (HopDir).
+// ----------------------------------------------------------------------------
+struct HopDir {
+  const Cx<double>* up;  // the neighbour's components that supply spins 0-1, and
+  const Cx<double>* lo;  // spins 2-3, cs elements apart
+  const int4* fx;        // the link in fixed point and in FP64, entries ls elements apart
+  const Cx<double>* u;
+};
+
+// one direction in FP64, added to acc (out of line: sites whose neighbours are out of the
+// fixed-point range)
+static __device__ __noinline__ void hop_dir_fp64(int d, HopDir q, int cs, int ls, double* acc) {
+  const int k = d >> 1, dir = d & 1;
+  Mat3<double> U = ldmat(q.u, ls, 0);
+  if (dir) U = dagger(U);
+  Vec3<double> s[2], w[2];
+  isigma(k, ldvec(q.lo, cs, 0), ldvec(q.lo + 3 * cs, cs, 0), s[0], s[1]);
+  for (int i = 0; i < 2; ++i) w[i] = matvec(U, vaxpy(dir ? -1.0 : 1.0, s[i], ldvec(q.up + 3 * i * cs, cs, 0)));
+  isigma(k, w[0], w[1], s[0], s[1]);
+  for (int i = 0; i < 2; ++i)
+    for (int c = 0; c < 3; ++c) {
+      acc[6 * i + 2 * c] += w[i].c[c].re;
+      acc[6 * i + 2 * c + 1] += w[i].c[c].im;
+      acc[12 + 6 * i + 2 * c] += dir ? s[i].c[c].re : -s[i].c[c].re;
+      acc[12 + 6 * i + 2 * c + 1] += dir ? s[i].c[c].im : -s[i].c[c].im;
+    }
+}
+
+// 16 bytes of device memory into shared memory, asynchronously
+__device__ __forceinline__ void fx_copy(int4* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+               "l"(__cvta_generic_to_global(src))
+               : "memory");
+}
+// dynamic shared memory of a warp: 12 spinor and 9 link entries per lane. A lane reads only what it
+// copied, so the copies need no barrier: a direction's spinor arrives while the one before multiplies its
+// link, its link while it is projected.
+constexpr int kFxStage = 21 * 32;
+inline size_t fx_smem(int threads) { return (size_t)threads / 32 * kFxStage * sizeof(int4); }
+
+// returns unit, with unit h = D_s (so that the scale joins the next multiply-add)
+template <class Dir>
+__device__ __forceinline__ double hop_fx(const Dir& dir, int cs, int ls, Vec3<double> (&h)[4]) {
+  extern __shared__ int4 fx_shared[];
+  int4* stage = fx_shared + (threadIdx.x >> 5) * kFxStage + (threadIdx.x & 31);
+  FxAcc f;
+  fx_clear(f);
+  auto fetch_spinor = [&](const HopDir& q) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      fx_copy(stage + 32 * c, q.up + (size_t)c * cs);
+      fx_copy(stage + 32 * (6 + c), q.lo + (size_t)c * cs);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto fetch_link = [&](const HopDir& q) {
+#pragma unroll
+    for (int e = 0; e < 9; ++e) fx_copy(stage + 32 * (12 + e), q.fx + (size_t)e * ls);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  HopDir next = dir(0);
+  fetch_spinor(next);
+  fetch_link(next);
+#pragma unroll 1
+  for (int d = 0; d < 6; ++d) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    FxHalf q;
+    {
+      Vec3<double> v[4];
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[s].c[c] = *reinterpret_cast<const Cx<double>*>(stage + 32 * (3 * s + c));
+      fx_project(f, q, d, v);
+    }
+    if (d < 5) {
+      next = dir(d + 1);
+      fetch_spinor(next);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    fx_multiply(f, q, d, stage + 32 * 12, 32);
+    if (d < 5) fetch_link(next);
+  }
+  if (f.wide) {
+    double o[24];
+    for (int i = 0; i < 24; ++i) o[i] = 0.0;
+#pragma unroll 1
+    for (int d = 0; d < 6; ++d) hop_dir_fp64(d, dir(d), cs, ls, o);
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) h[s].c[c] = mk<double>(o[2 * (3 * s + c)], o[2 * (3 * s + c) + 1]);
+    return 0.5;
+  }
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) h[s].c[c] = mk<double>((double)f.a[s][c][0], (double)f.a[s][c][1]);
+  return fx_unit(f);
+}
+
+// For the lanes with flag set: out = P x (dag: P^dag x) of two colour vectors, x's six components cs elements
+// apart. Six lanes of the warp form one component each: as one lane's two products, the wrap of the
+// axial frame would hold the FP64 pipe for the whole warp as long as the rest of a site's FP64
+// operations. Warp-collective.
+__device__ __forceinline__ void warp_link_product(bool flag, const Cx<double>* P, const Cx<double>* x, int cs, bool dag,
+                                                  Vec3<double> (&out)[2]) {
+  const int lane = threadIdx.x & 31;
+  const int q = lane < 6 ? lane : 0, row = q % 3;
+  unsigned m = __ballot_sync(0xffffffffu, flag);
+  while (m) {
+    const int w = __ffs(m) - 1;
+    m &= m - 1;
+    const Cx<double>* Pw = reinterpret_cast<const Cx<double>*>(__shfl_sync(0xffffffffu, (unsigned long long)P, w));
+    const Cx<double>* xw = reinterpret_cast<const Cx<double>*>(__shfl_sync(0xffffffffu, (unsigned long long)x, w));
+    xw += (size_t)(q - row) * cs;
+    Cx<double> v = czero<double>();
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+      v = dag ? cfmaconj(v, Pw[3 * b + row], xw[(size_t)b * cs]) : cfma(v, Pw[3 * row + b], xw[(size_t)b * cs]);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const Cx<double> u = shfl_idx(v, i, 32);
+      if (lane == w) out[i / 3].c[i % 3] = u;
+    }
+  }
+}
 
 }  // namespace wf

@@ -228,6 +228,7 @@ struct EoArgs {
   const Cx<R>* ut[2];     // general frame: U_t per 3-D parity, line layout
   const Cx<R>* pl[2];     // axial frame: boundary link P per line
   const Cx<R>* us[2];     // spatial forward links per 3-D parity, line layout
+  const int4* fx[2];      // R = double: the same in fixed point (wf_fixed.cuh)
   R inv_gf, bc;
 };
 template <typename R>

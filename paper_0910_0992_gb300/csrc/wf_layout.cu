@@ -216,18 +216,19 @@ __device__ __forceinline__ void rotate3_split(const SplitMat& G, const float (&f
 }
 
 // One spin of a site on import: in (shared memory, 3 FP64 elements, negated for gamma_5) rotated by G
-// into out (components tp elements apart). The _wide forms are the rotation in FP64, out of line, for
+// into out (components os elements apart). The _wide forms are the rotation in FP64, out of line, for
 // extreme magnitudes, infinities and NaN.
 template <typename R>
-__device__ __noinline__ void import_spin_wide(const Cx<double>* gl, const Cx<double>* in, bool neg, Cx<R>* out, int tp) {
+__device__ __noinline__ void import_spin_wide(const Cx<double>* gl, int tp, const Cx<double>* in, bool neg, Cx<R>* out,
+                                              int os) {
   for (int a = 0; a < 3; ++a) {
     Cx<double> w = czero<double>();
     for (int b = 0; b < 3; ++b) w = cfma(w, gl[(size_t)(3 * a + b) * tp], neg ? mk<double>(-in[b].re, -in[b].im) : in[b]);
-    out[(size_t)a * tp] = mk<R>((R)w.re, (R)w.im);
+    out[(size_t)a * os] = mk<R>((R)w.re, (R)w.im);
   }
 }
-__device__ __forceinline__ void import_spin(const FxMat& G, const Cx<double>* gl, int sl, const Cx<double>* in, bool neg,
-                                            Cx<double>* out, int tp) {
+__device__ __forceinline__ void import_spin(const FxMat& G, const Cx<double>* gl, int tp, int sl, const Cx<double>* in,
+                                            bool neg, Cx<double>* out, int os) {
   double v[6], w[6];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -235,14 +236,14 @@ __device__ __forceinline__ void import_spin(const FxMat& G, const Cx<double>* gl
     v[2 * c + 1] = neg ? -in[c].im : in[c].im;
   }
   if (!rotate3_fx<false>(G, v, w)) {
-    import_spin_wide<double>(gl + sl, in, neg, out, tp);
+    import_spin_wide<double>(gl + sl, tp, in, neg, out, os);
     return;
   }
 #pragma unroll
-  for (int c = 0; c < 3; ++c) out[(size_t)c * tp] = mk<double>(w[2 * c], w[2 * c + 1]);
+  for (int c = 0; c < 3; ++c) out[(size_t)c * os] = mk<double>(w[2 * c], w[2 * c + 1]);
 }
-__device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>* gl, int sl, const Cx<double>* in,
-                                            bool neg, Cx<float>* out, int tp) {
+__device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>* gl, int tp, int sl,
+                                            const Cx<double>* in, bool neg, Cx<float>* out, int os) {
   float f[6], lo[6];
   bool ok = true;
 #pragma unroll
@@ -252,13 +253,13 @@ __device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>*
     ok &= split_double(neg ? -v.im : v.im, f[2 * k + 1], lo[2 * k + 1]);
   }
   if (!ok) {
-    import_spin_wide<float>(gl + sl, in, neg, out, tp);
+    import_spin_wide<float>(gl + sl, tp, in, neg, out, os);
     return;
   }
   float s[6], c[6];
   rotate3_split<false>(G, f, lo, s, c);
 #pragma unroll
-  for (int k = 0; k < 3; ++k) out[(size_t)k * tp] = mk<float>(s[2 * k] + c[2 * k], s[2 * k + 1] + c[2 * k + 1]);
+  for (int k = 0; k < 3; ++k) out[(size_t)k * os] = mk<float>(s[2 * k] + c[2 * k], s[2 * k + 1] + c[2 * k + 1]);
 }
 // One spin of a site on export: v rotated by G^dag into out (shared memory, 3 FP64 elements)
 template <typename R>
@@ -326,11 +327,13 @@ struct RotationOf<double> {
 // thread k + (128 / SPL) h holds spins h, h + SPL, .. of row k: line li = k / nJ, slot m lpl + j0 + jj with
 // (m, jj) = (k % nJ) / J, % J. SPL = 1 (a thread holds the site), or 4 where the lattice is so small
 // that the rotation's serial chain, not the memory, is what a launch waits for.
+// EO: the 4-D even-odd fields [rhs][L^3][12][T/2] of wf_eo4d.cu instead of the line layout; "lines" are
+// then all L^3 spatial sites, p the 4-D parity, m = 0 and slot h holds t = 2 h + t0.
 struct TileAt {
   int p, l0, j0, r0, r1;
-  __device__ __forceinline__ TileAt(const Geom& g, const SpinorTile& t, int npar, int nrhs) {
+  __device__ __forceinline__ TileAt(const SpinorTile& t, int npar, int par, int nrhs) {
     int b = blockIdx.x;
-    p = npar == 2 ? b & 1 : 0;
+    p = npar == 2 ? b & 1 : par;
     b /= npar;
     l0 = (b % t.ntl) * t.tl;
     j0 = (b / t.ntl) * t.J;
@@ -338,67 +341,102 @@ struct TileAt {
     r1 = min(nrhs, r0 + t.rper);
   }
 };
-// element offset of line l's site at t = 0 in the caller's array (add t * stride)
-__device__ __forceinline__ size_t caller_site(const Geom& g, int compact, int p, int l) {
-  if (compact) return (size_t)l;
-  int x, y, z;
-  line_coords(g, p, l, x, y, z);
-  return (size_t)x + g.L * ((size_t)y + (size_t)g.L * z);
+// one line's places: the caller's site at time t is (origin + t stride) / div
+template <bool EO>
+struct TileLine {
+  size_t origin, stride;
+  int t0;             // EO: first time
+  int p3, l3;         // 3-D parity and line of the line layout (rotation)
+  __device__ __forceinline__ TileLine(const Geom& g, int compact, int p, int l) {
+    int x, y, z;
+    if (EO) {
+      x = l % g.L;
+      y = (l / g.L) % g.L;
+      z = l / (g.L * g.L);
+      t0 = (p + x + y + z) & 1;
+      p3 = (x + y + z) & 1;
+      l3 = line_of(g, x, y, z);
+    } else {
+      line_coords(g, p, l, x, y, z);
+      t0 = 0;
+      p3 = p;
+      l3 = l;
+    }
+    if (!EO && compact) {
+      origin = (size_t)l;
+      stride = (size_t)g.Nl;
+    } else {
+      origin = (size_t)x + g.L * ((size_t)y + (size_t)g.L * z);
+      stride = (size_t)g.L * g.L * g.L;
+    }
+  }
+  __device__ __forceinline__ size_t site(int compact, int t) const {
+    const size_t i = origin + stride * t;
+    return EO && compact ? i / 2 : i;
+  }
+};
+template <bool EO>
+__device__ __forceinline__ size_t caller_sites(const Geom& g, int compact) {
+  const size_t V = (size_t)g.L * g.L * g.L * g.T;
+  return compact ? V / 2 : V;
 }
 
-template <typename R, int SPL>
-__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_import_spinor(const Geom g, const SpinorTile t, int compact,
-                                                                const Cx<double>* __restrict__ lex, Cx<R>* even,
-                                                                Cx<R>* odd, int nrhs, int g5, const Cx<double>* g_e,
-                                                                const Cx<double>* g_o) {
+// compact: 0 full arrays, 1 arrays of one parity (par: which)
+template <typename R, int SPL, bool EO>
+__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks)
+    k_import_spinor(const Geom g, const SpinorTile t, int compact, int par, const Cx<double>* __restrict__ lex, Cx<R>* even,
+                    Cx<R>* odd, int nrhs, int g5, const Cx<double>* g_e, const Cx<double>* g_o) {
   __shared__ __align__(16) Cx<double> buf[kTileThreads / SPL * kTileRow];
-  const TileAt at(g, t, compact ? 1 : 2, nrhs);
+  const TileAt at(t, compact ? 1 : 2, par, nrhs);
   Cx<R>* dst = at.p ? odd : even;
   if (!dst) return;
-  const Cx<double>* gr = at.p ? g_o : g_e;
-  const int q = threadIdx.x;
-  const size_t ts = compact ? (size_t)g.Nl : (size_t)g.L * g.L * g.L;  // sites per time slice of the caller's array
+  const int q = threadIdx.x, nl = EO ? 2 * g.Nl : g.Nl, os = EO ? g.T / 2 : g.tp;
+  const size_t ns = caller_sites<EO>(g, compact);
   // layout's side
   const int row = q % (kTileThreads / SPL), sp0 = q / (kTileThreads / SPL);
   const int li = row / t.nJ, mj = row - li * t.nJ, m = mj / t.J, jj = mj - m * t.J;
-  const int l = at.l0 + li, sl = m * g.lpl + at.j0 + jj;
-  const bool mine = li < t.tl && l < g.Nl;
-  const bool valid = mine && (at.j0 + jj) * g.n + m < g.T;
+  const int l = at.l0 + li, sl = EO ? at.j0 + jj : m * g.lpl + at.j0 + jj;
+  const TileLine<EO> mine_at(g, compact, at.p, l < nl ? l : 0);
+  const int time = EO ? 2 * sl + mine_at.t0 : (at.j0 + jj) * g.n + m;
+  const bool mine = li < t.tl && l < nl && (!EO || sl < os);
+  const bool valid = mine && time < g.T;
+  const Cx<double>* gr = mine_at.p3 ? g_o : g_e;
+  const Cx<double>* gl = gr ? gr + (size_t)mine_at.l3 * 9 * g.tp : nullptr;
+  const int gsl = EO ? slot_of(g, valid ? time : 0) : sl;
   typename RotationOf<R>::type G;
-  const Cx<double>* gl = gr ? gr + (size_t)l * 9 * g.tp : nullptr;
-  if (valid && gr) load_rotation(gl, g.tp, sl, G);
+  if (valid && gr) load_rotation(gl, g.tp, gsl, G);
   // caller's side
   const int cc = q % 12, cs = q / 12, cli = cs & (t.tl - 1), step = 8 / t.tl;
-  const bool mover = q < 96 && at.l0 + cli < g.Nl;
-  const size_t csite = mover ? caller_site(g, compact, at.p, at.l0 + cli) : 0;
+  const bool mover = q < 96 && at.l0 + cli < nl;
+  const TileLine<EO> from(g, compact, at.p, mover ? at.l0 + cli : 0);
 
   for (int rhs = at.r0; rhs < at.r1; ++rhs) {
     if (mover) {
-      const Cx<double>* src = lex + ((size_t)rhs * g.T * ts + csite) * NSPIN_C + cc;
+      const Cx<double>* src = lex + (size_t)rhs * ns * NSPIN_C + cc;
       for (int tt = cs / t.tl; tt < t.nJ; tt += step) {
-        const int time = at.j0 * g.n + tt;
-        if (time >= g.T) break;
-        const int j = tt / g.n;
-        const int to = (cli * g.n + (tt - j * g.n)) * t.J + j;  // its row
-        cp_async16(&buf[to * kTileRow + cc], src + (size_t)time * ts * NSPIN_C);
+        const int tm = EO ? 2 * (at.j0 + tt) + from.t0 : at.j0 * g.n + tt;
+        if (tm >= g.T) break;
+        const int j = EO ? tt : tt / g.n;
+        const int to = EO ? cli * t.J + tt : (cli * g.n + (tt - j * g.n)) * t.J + j;  // its row
+        cp_async16(&buf[to * kTileRow + cc], src + from.site(compact, tm) * NSPIN_C);
       }
     }
     cp_async_wait_all();
     __syncthreads();
     if (mine) {
-      Cx<R>* out = dst + ((size_t)rhs * g.Nl + l) * NSPIN_C * g.tp + sl;
+      Cx<R>* out = dst + ((size_t)rhs * nl + l) * NSPIN_C * os + sl;
 #pragma unroll 1
       for (int i = 0; i < 4 / SPL; ++i) {
         const int sp = sp0 + i * SPL;
-        Cx<R>* o = out + (size_t)sp * 3 * g.tp;
+        Cx<R>* o = out + (size_t)sp * 3 * os;
         const Cx<double>* in = buf + row * kTileRow + (g5 ? (sp + 2) % 4 : sp) * 3;
         if (valid && gr) {
-          import_spin(G, gl, sl, in, g5 != 0, o, g.tp);
+          import_spin(G, gl, g.tp, gsl, in, g5 != 0, o, os);
         } else {  // the caller's gauge, or padding slots: zero
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
             const Cx<double> v = valid ? in[c] : czero<double>();
-            o[(size_t)c * g.tp] = g5 ? mk<R>((R)-v.re, (R)-v.im) : mk<R>((R)v.re, (R)v.im);
+            o[(size_t)c * os] = g5 ? mk<R>((R)-v.re, (R)-v.im) : mk<R>((R)v.re, (R)v.im);
           }
         }
       }
@@ -407,31 +445,33 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_import_spinor(
   }
 }
 
-template <typename R, int SPL>
-__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_export_spinor(const Geom g, const SpinorTile t, int compact,
-                                                                const Cx<R>* even, const Cx<R>* odd,
-                                                                Cx<double>* __restrict__ lex, int nrhs, int g5,
-                                                                const Cx<double>* g_e, const Cx<double>* g_o) {
+template <typename R, int SPL, bool EO>
+__global__ void __launch_bounds__(kTileThreads, kTileMinBlocks)
+    k_export_spinor(const Geom g, const SpinorTile t, int compact, int par, const Cx<R>* even, const Cx<R>* odd,
+                    Cx<double>* __restrict__ lex, int nrhs, int g5, const Cx<double>* g_e, const Cx<double>* g_o) {
   __shared__ __align__(16) Cx<double> buf[kTileThreads / SPL * kTileRow];
-  const TileAt at(g, t, compact ? 1 : 2, nrhs);
+  const TileAt at(t, compact ? 1 : 2, par, nrhs);
   const Cx<R>* src = at.p ? odd : even;  // null: that parity's sites are zero
-  const Cx<double>* gr = at.p ? g_o : g_e;
-  const int q = threadIdx.x;
-  const size_t ts = compact ? (size_t)g.Nl : (size_t)g.L * g.L * g.L;
+  const int q = threadIdx.x, nl = EO ? 2 * g.Nl : g.Nl, os = EO ? g.T / 2 : g.tp;
+  const size_t ns = caller_sites<EO>(g, compact);
   const int row = q % (kTileThreads / SPL), sp0 = q / (kTileThreads / SPL);
   const int li = row / t.nJ, mj = row - li * t.nJ, m = mj / t.J, jj = mj - m * t.J;
-  const int l = at.l0 + li, sl = m * g.lpl + at.j0 + jj;
-  const bool valid = li < t.tl && l < g.Nl && (at.j0 + jj) * g.n + m < g.T;
+  const int l = at.l0 + li, sl = EO ? at.j0 + jj : m * g.lpl + at.j0 + jj;
+  const TileLine<EO> mine_at(g, compact, at.p, l < nl ? l : 0);
+  const int time = EO ? 2 * sl + mine_at.t0 : (at.j0 + jj) * g.n + m;
+  const bool valid = li < t.tl && l < nl && (!EO || sl < os) && time < g.T;
+  const Cx<double>* gr = mine_at.p3 ? g_o : g_e;
+  const Cx<double>* gl = gr ? gr + (size_t)mine_at.l3 * 9 * g.tp : nullptr;
+  const int gsl = EO ? slot_of(g, valid ? time : 0) : sl;
   typename RotationOf<R>::type G;
-  const Cx<double>* gl = gr ? gr + (size_t)l * 9 * g.tp : nullptr;
-  if (valid && gr && src) load_rotation(gl, g.tp, sl, G);
+  if (valid && gr && src) load_rotation(gl, g.tp, gsl, G);
   const int cc = q % 12, cs = q / 12, cli = cs & (t.tl - 1), step = 8 / t.tl;
-  const bool mover = q < 96 && at.l0 + cli < g.Nl;
-  const size_t csite = mover ? caller_site(g, compact, at.p, at.l0 + cli) : 0;
+  const bool mover = q < 96 && at.l0 + cli < nl;
+  const TileLine<EO> to(g, compact, at.p, mover ? at.l0 + cli : 0);
 
   for (int rhs = at.r0; rhs < at.r1; ++rhs) {
     if (valid) {
-      const Cx<R>* in = src ? src + ((size_t)rhs * g.Nl + l) * NSPIN_C * g.tp + sl : nullptr;
+      const Cx<R>* in = src ? src + ((size_t)rhs * nl + l) * NSPIN_C * os + sl : nullptr;
 #pragma unroll 1
       for (int i = 0; i < 4 / SPL; ++i) {
         const int sp = sp0 + i * SPL, ss = g5 ? (sp + 2) % 4 : sp;
@@ -439,10 +479,10 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_export_spinor(
         Vec3<R> v = {};
         if (src) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c) v.c[c] = in[(size_t)(ss * 3 + c) * g.tp];
+          for (int c = 0; c < 3; ++c) v.c[c] = in[(size_t)(ss * 3 + c) * os];
         }
         if (src && gr) {
-          export_spin(G, gl, g.tp, sl, v, g5 != 0, out);
+          export_spin(G, gl, g.tp, gsl, v, g5 != 0, out);
         } else {
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
@@ -454,13 +494,13 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_export_spinor(
     }
     __syncthreads();
     if (mover) {
-      Cx<double>* dst = lex + ((size_t)rhs * g.T * ts + csite) * NSPIN_C + cc;
+      Cx<double>* dst = lex + (size_t)rhs * ns * NSPIN_C + cc;
       for (int tt = cs / t.tl; tt < t.nJ; tt += step) {
-        const int time = at.j0 * g.n + tt;
-        if (time >= g.T) break;
-        const int j = tt / g.n;
-        const int from = (cli * g.n + (tt - j * g.n)) * t.J + j;
-        dst[(size_t)time * ts * NSPIN_C] = buf[from * kTileRow + cc];
+        const int tm = EO ? 2 * (at.j0 + tt) + to.t0 : at.j0 * g.n + tt;
+        if (tm >= g.T) break;
+        const int j = EO ? tt : tt / g.n;
+        const int from = EO ? cli * t.J + tt : (cli * g.n + (tt - j * g.n)) * t.J + j;
+        dst[to.site(compact, tm) * NSPIN_C] = buf[from * kTileRow + cc];
       }
     }
     __syncthreads();
@@ -620,16 +660,23 @@ static int grid_for(size_t n) {
 // lines, 128 sites at most; 32 sites with four threads each where that leaves fewer than two CTAs per
 // SM (then as few as one line), and all sources of a tile in one CTA (its rotation is then read
 // once) only where the tiles alone fill the chip
-static SpinorTile tile_of(const Geom& g, int npar, int nrhs, dim3& grid, bool& split) {
+static SpinorTile tile_of(const Geom& g, int npar, int nrhs, bool eo, dim3& grid, bool& split) {
   SpinorTile t;
-  t.J = g.n == 1 ? 32 : g.n == 2 ? 16 : g.n <= 4 ? 8 : 4;
-  if (t.J > g.lpl) t.J = g.lpl;
-  t.nJ = g.n * t.J;
-  t.nch = g.lpl / t.J;
+  if (eo) {
+    t.J = std::min(32, g.T / 2);
+    t.nJ = t.J;
+    t.nch = (g.T / 2 + t.J - 1) / t.J;
+  } else {
+    t.J = g.n == 1 ? 32 : g.n == 2 ? 16 : g.n <= 4 ? 8 : 4;
+    if (t.J > g.lpl) t.J = g.lpl;
+    t.nJ = g.n * t.J;
+    t.nch = g.lpl / t.J;
+  }
+  const int nl = eo ? 2 * g.Nl : g.Nl;
   auto lines = [&](int sites) {
     t.tl = 8;
     while (t.tl > 1 && t.tl * t.nJ > sites) t.tl >>= 1;
-    t.ntl = (g.Nl + t.tl - 1) / t.tl;
+    t.ntl = (nl + t.tl - 1) / t.tl;
     return (long long)npar * t.ntl * t.nch;
   };
   long long blocks = lines(kTileThreads);
@@ -641,50 +688,64 @@ static SpinorTile tile_of(const Geom& g, int npar, int nrhs, dim3& grid, bool& s
   return t;
 }
 
-template <typename R>
-static void launch_import_tiles(const Geom& g, int compact, const Cx<double>* in, Cx<R>* even, Cx<R>* odd, int nrhs,
+// par: -1 full arrays, else arrays of that parity (line layout: the caller's pointers choose it)
+template <typename R, bool EO>
+static void launch_import_tiles(const Geom& g, int par, const Cx<double>* in, Cx<R>* even, Cx<R>* odd, int nrhs, int g5,
+                                const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
+  dim3 grid;
+  bool split;
+  const int compact = par >= 0;
+  const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, EO, grid, split);
+  if (split)
+    k_import_spinor<R, 4, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, in, even, odd, nrhs, g5, g_e, g_o);
+  else
+    k_import_spinor<R, 1, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, in, even, odd, nrhs, g5, g_e, g_o);
+  WF_CUDA(cudaGetLastError());
+}
+template <typename R, bool EO>
+static void launch_export_tiles(const Geom& g, int par, const Cx<R>* even, const Cx<R>* odd, Cx<double>* out, int nrhs,
                                 int g5, const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
   dim3 grid;
   bool split;
-  const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, grid, split);
+  const int compact = par >= 0;
+  const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, EO, grid, split);
   if (split)
-    k_import_spinor<R, 4><<<grid, kTileThreads, 0, s>>>(g, t, compact, in, even, odd, nrhs, g5, g_e, g_o);
+    k_export_spinor<R, 4, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, even, odd, out, nrhs, g5, g_e, g_o);
   else
-    k_import_spinor<R, 1><<<grid, kTileThreads, 0, s>>>(g, t, compact, in, even, odd, nrhs, g5, g_e, g_o);
-  WF_CUDA(cudaGetLastError());
-}
-template <typename R>
-static void launch_export_tiles(const Geom& g, int compact, const Cx<R>* even, const Cx<R>* odd, Cx<double>* out,
-                                int nrhs, int g5, const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
-  dim3 grid;
-  bool split;
-  const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, grid, split);
-  if (split)
-    k_export_spinor<R, 4><<<grid, kTileThreads, 0, s>>>(g, t, compact, even, odd, out, nrhs, g5, g_e, g_o);
-  else
-    k_export_spinor<R, 1><<<grid, kTileThreads, 0, s>>>(g, t, compact, even, odd, out, nrhs, g5, g_e, g_o);
+    k_export_spinor<R, 1, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, even, odd, out, nrhs, g5, g_e, g_o);
   WF_CUDA(cudaGetLastError());
 }
 
 template <typename R>
 void launch_import_spinor(const Geom& g, const Cx<double>* lex, Cx<R>* even, Cx<R>* odd, int nrhs, int g5,
                           const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
-  launch_import_tiles<R>(g, 0, lex, even, odd, nrhs, g5, g_e, g_o, s);
+  launch_import_tiles<R, false>(g, -1, lex, even, odd, nrhs, g5, g_e, g_o, s);
 }
 template <typename R>
 void launch_export_spinor(const Geom& g, const Cx<R>* even, const Cx<R>* odd, Cx<double>* lex, int nrhs, int g5,
                           const Cx<double>* g_e, const Cx<double>* g_o, cudaStream_t s) {
-  launch_export_tiles<R>(g, 0, even, odd, lex, nrhs, g5, g_e, g_o, s);
+  launch_export_tiles<R, false>(g, -1, even, odd, lex, nrhs, g5, g_e, g_o, s);
 }
 template <typename R>
 void launch_import_compact(const Geom& g, const Cx<double>* cmp, Cx<R>* half, int nrhs, int g5,
                            const Cx<double>* gr, cudaStream_t s) {
-  launch_import_tiles<R>(g, 1, cmp, half, nullptr, nrhs, g5, gr, nullptr, s);
+  launch_import_tiles<R, false>(g, 0, cmp, half, nullptr, nrhs, g5, gr, nullptr, s);
 }
 template <typename R>
 void launch_export_compact(const Geom& g, const Cx<R>* half, Cx<double>* cmp, int nrhs, int g5,
                            const Cx<double>* gr, cudaStream_t s) {
-  launch_export_tiles<R>(g, 1, half, nullptr, cmp, nrhs, g5, gr, nullptr, s);
+  launch_export_tiles<R, false>(g, 0, half, nullptr, cmp, nrhs, g5, gr, nullptr, s);
+}
+// 4-D even-odd fields; compact_par < 0: full lexicographic arrays
+template <typename R>
+void launch_import_eo(const Geom& g, const Cx<double>* lex, Cx<R>* even, Cx<R>* odd, int nrhs, const Cx<double>* g0,
+                      const Cx<double>* g1, int compact_par, cudaStream_t s) {
+  launch_import_tiles<R, true>(g, compact_par, lex, even, odd, nrhs, 0, g0, g1, s);
+}
+template <typename R>
+void launch_export_eo(const Geom& g, const Cx<R>* even, const Cx<R>* odd, Cx<double>* lex, int nrhs,
+                      const Cx<double>* g0, const Cx<double>* g1, int compact_par, cudaStream_t s) {
+  launch_export_tiles<R, true>(g, compact_par, even, odd, lex, nrhs, 0, g0, g1, s);
 }
 #define WF_INST(R)                                                                                          \
   template void launch_import_spinor<R>(const Geom&, const Cx<double>*, Cx<R>*, Cx<R>*, int, int,             \
@@ -694,7 +755,11 @@ void launch_export_compact(const Geom& g, const Cx<R>* half, Cx<double>* cmp, in
   template void launch_import_compact<R>(const Geom&, const Cx<double>*, Cx<R>*, int, int, const Cx<double>*, \
                                          cudaStream_t);                                                     \
   template void launch_export_compact<R>(const Geom&, const Cx<R>*, Cx<double>*, int, int, const Cx<double>*, \
-                                         cudaStream_t);
+                                         cudaStream_t);                                                     \
+  template void launch_import_eo<R>(const Geom&, const Cx<double>*, Cx<R>*, Cx<R>*, int, const Cx<double>*,   \
+                                    const Cx<double>*, int, cudaStream_t);                                  \
+  template void launch_export_eo<R>(const Geom&, const Cx<R>*, const Cx<R>*, Cx<double>*, int,               \
+                                    const Cx<double>*, const Cx<double>*, int, cudaStream_t);
 WF_INST(float)
 WF_INST(double)
 #undef WF_INST
