@@ -2234,16 +2234,22 @@ void clover_on(wf_handle* h, int p, const Cx<R>* in, Cx<R>* out, const Cx<R>* ac
 
 // out = xpost + apost C[xpre + apre S(in)] on the lines of `parity` for one right-hand side: S the
 // site's own spinor (SRC_LOAD) or D_s of the other parity (SRC_HOP), C the line operation opu /
-// opl per spin half; xpre / xpost null: no pre- / post-axpy
+// opl per spin half; xpre / xpost null: no pre- / post-axpy; norm2: add |out|^2 there. With dagger
+// gamma_5 C S gamma_5 takes the place of C S: the operations change halves, and a hop reads and
+// stores the halves exchanged, so no field has to be
 template <typename R>
 void line_step(wf_handle* h, int parity, int src, const Cx<R>* in, Cx<R>* out, int opu, int opl, const Cx<R>* xpre,
-               double apre, const Cx<R>* xpost, double apost, const char* name) {
+               double apre, const Cx<R>* xpost, double apost, const char* name, int dagger = 0,
+               double* norm2 = nullptr) {
   LineArgs<R> a = line_args<R>(h, parity, 1);
+  const bool swap = dagger && src == SRC_HOP;
   a.src = src;
-  a.src_up = in;
-  a.src_lo = in + 6 * h->g.tp;
-  a.opu = opu;
-  a.opl = opl;
+  a.src_up = in + (swap ? 6 * h->g.tp : 0);
+  a.src_lo = in + (swap ? 0 : 6 * h->g.tp);
+  a.swap_out = swap ? 1 : 0;
+  a.opu = dagger && !swap ? opl : opu;
+  a.opl = dagger && !swap ? opu : opl;
+  a.norm2 = norm2;
   a.xpre = xpre;
   a.apre = (R)apre;
   a.xpost = xpost;
@@ -2265,11 +2271,20 @@ void line_step(wf_handle* h, int parity, int src, const Cx<R>* in, Cx<R>* out, i
 // into its kernel: with a = C_R^o psi_o and u = C_L^e D_s^eo a (so t1 = g u),
 //   t2 = C_L^e A^ee C_R^e (psi_e + g u),  chi_e = psi_e + t2,
 //   chi_o = [psi_o + C_L^o A^oo a] + g C_L^o D_s^oe C_R^e (t2 - g u);
-// without a clover term t2 = 0 and chi_o = psi_o - g^2 C_L^o D_s^oe C_R^e u.
+// without a clover term t2 = 0 and chi_o = psi_o - g^2 C_L^o D_s^oe C_R^e u. The adjoint (dagger) is
+// gamma_5 M-tilde_ILU gamma_5 (S_R^dag = gamma_5 S_L gamma_5, M_SW gamma_5-hermitian; A commutes with
+// gamma_5): the same sequence of line_step with dagger. norm2 (if set): |chi|^2, added up by the two
+// kernels that store chi (16^3 x 128 in FP32: the exchanges of halves took 52 us per adjoint and the
+// norm's own pass 21 us per apply).
 template <typename R>
-void ilu_apply(wf_handle* h, const Cx<R>* pe, const Cx<R>* po, Cx<R>* ce, Cx<R>* co) {
+void ilu_apply(wf_handle* h, const Cx<R>* pe, const Cx<R>* po, Cx<R>* ce, Cx<R>* co, int dagger, double* norm2) {
   const size_t hn = h->half_int();
   cudaStream_t s = h->stream;
+  auto step = [&](int parity, int src, const Cx<R>* in, Cx<R>* out, int opu, int opl, const Cx<R>* xpre, double apre,
+                  const Cx<R>* xpost, double apost, const char* name, double* nrm = nullptr) {
+    line_step<R>(h, parity, src, in, out, opu, opl, xpre, apre, xpost, apost, name, dagger, nrm);
+  };
+  if (norm2 && !h->norm_cleared) WF_CUDA(cudaMemsetAsync(norm2, 0, sizeof(double), s));
   const double g = 1.0 / h->g.gamma_f;
   Cx<R>* a = h->buf<Cx<R>>(pname<R>("il_a"), hn);
   Cx<R>* u = h->buf<Cx<R>>(pname<R>("il_u"), hn);
@@ -2277,50 +2292,30 @@ void ilu_apply(wf_handle* h, const Cx<R>* pe, const Cx<R>* po, Cx<R>* ce, Cx<R>*
   Cx<R>* d = h->buf<Cx<R>>(pname<R>("il_d"), hn);
   Cx<R>* t2 = h->buf<Cx<R>>(pname<R>("il_t2"), hn);
   Cx<R>* e = h->buf<Cx<R>>(pname<R>("il_e"), hn);
-  line_step<R>(h, 1, SRC_LOAD, po, a, OP_FWD, OP_COPY, nullptr, 0.0, nullptr, 0.0, "il_c_right");  // a = C_R^o psi_o
-  line_step<R>(h, 0, SRC_HOP, a, u, OP_COPY, OP_BWD, nullptr, 0.0, nullptr, 0.0, "il_hop_c_left");  // u = C_L^e D a
+  step(1, SRC_LOAD, po, a, OP_FWD, OP_COPY, nullptr, 0.0, nullptr, 0.0, "il_c_right");  // a = C_R^o psi_o
+  step(0, SRC_HOP, a, u, OP_COPY, OP_BWD, nullptr, 0.0, nullptr, 0.0, "il_hop_c_left");  // u = C_L^e D a
   if (h->clover) {
-    line_step<R>(h, 0, SRC_LOAD, u, c, OP_FWD, OP_COPY, pe, g, nullptr, 0.0, "il_c_right");  // C_R^e (psi_e + g u)
+    step(0, SRC_LOAD, u, c, OP_FWD, OP_COPY, pe, g, nullptr, 0.0, "il_c_right");  // C_R^e (psi_e + g u)
     clover_on<R>(h, 0, c, d, nullptr, 1.0, 1);
-    line_step<R>(h, 0, SRC_LOAD, d, t2, OP_COPY, OP_BWD, nullptr, 0.0, nullptr, 0.0, "il_c_left");  // t2
-    line_step<R>(h, 0, SRC_LOAD, t2, ce, OP_COPY, OP_COPY, pe, 1.0, nullptr, 0.0, "il_axpy");  // chi_e = psi_e + t2
-    line_step<R>(h, 0, SRC_LOAD, u, c, OP_FWD, OP_COPY, t2, -g, nullptr, 0.0, "il_c_right");  // C_R^e (t2 - g u)
+    step(0, SRC_LOAD, d, t2, OP_COPY, OP_BWD, nullptr, 0.0, nullptr, 0.0, "il_c_left");  // t2
+    step(0, SRC_LOAD, t2, ce, OP_COPY, OP_COPY, pe, 1.0, nullptr, 0.0, "il_axpy", norm2);  // chi_e = psi_e + t2
+    step(0, SRC_LOAD, u, c, OP_FWD, OP_COPY, t2, -g, nullptr, 0.0, "il_c_right");  // C_R^e (t2 - g u)
     clover_on<R>(h, 1, a, d, nullptr, 1.0, 1);  // d = A^oo C_R^o psi_o
-    line_step<R>(h, 1, SRC_LOAD, d, e, OP_COPY, OP_BWD, nullptr, 0.0, po, 1.0, "il_c_left");  // psi_o + Abar^oo psi_o
-    line_step<R>(h, 1, SRC_HOP, c, co, OP_COPY, OP_BWD, nullptr, 0.0, e, g, "il_hop_c_left");
+    step(1, SRC_LOAD, d, e, OP_COPY, OP_BWD, nullptr, 0.0, po, 1.0, "il_c_left");  // psi_o + Abar^oo psi_o
+    step(1, SRC_HOP, c, co, OP_COPY, OP_BWD, nullptr, 0.0, e, g, "il_hop_c_left", norm2);
   } else {
-    WF_CUDA(cudaMemcpyAsync(ce, pe, hn * sizeof(Cx<R>), cudaMemcpyDeviceToDevice, s));
-    line_step<R>(h, 0, SRC_LOAD, u, c, OP_FWD, OP_COPY, nullptr, 0.0, nullptr, 0.0, "il_c_right");  // C_R^e u
-    line_step<R>(h, 1, SRC_HOP, c, co, OP_COPY, OP_BWD, nullptr, 0.0, po, -g * g, "il_hop_c_left");
+    step(0, SRC_LOAD, pe, ce, OP_COPY, OP_COPY, nullptr, 0.0, nullptr, 0.0, "il_copy", norm2);
+    step(0, SRC_LOAD, u, c, OP_FWD, OP_COPY, nullptr, 0.0, nullptr, 0.0, "il_c_right");  // C_R^e u
+    step(1, SRC_HOP, c, co, OP_COPY, OP_BWD, nullptr, 0.0, po, -g * g, "il_hop_c_left", norm2);
   }
 }
 
-// M-tilde_ILU on [even | odd] internal vectors (one right-hand side); the adjoint is
-// gamma_5 M-tilde_ILU gamma_5 (S_R^dag = gamma_5 S_L gamma_5, M_SW gamma_5-hermitian), applied
-// with the spin halves exchanged on both sides
+// M-tilde_ILU on [even | odd] internal vectors (one right-hand side)
 template <typename R>
 OpFn<R> ilu_op(wf_handle* h) {
   return [=](const Cx<R>* x, Cx<R>* y, int dagger, double* norm2) {
     const size_t hn = h->half_int();
-    cudaStream_t s = h->stream;
-    if (dagger) {
-      Cx<R>* xs = h->buf<Cx<R>>(pname<R>("il_xs"), 2 * hn);
-      Cx<R>* ys = h->buf<Cx<R>>(pname<R>("il_ys"), 2 * hn);
-      {
-        Prof P(h, pname<R>("il_swap"));
-        launch_swap_halves<R>(x, xs, 2 * hn, h->g.tp, s);
-      }
-      ilu_apply<R>(h, xs, xs + hn, ys, ys + hn);
-      Prof P(h, pname<R>("il_swap"));
-      launch_swap_halves<R>(ys, y, 2 * hn, h->g.tp, s);
-    } else {
-      ilu_apply<R>(h, x, x + hn, y, y + hn);
-    }
-    if (norm2) {
-      double* partial = h->buf<double>("op_partial", 1024);
-      Prof P(h, pname<R>("norm2"), 2);
-      launch_norm2<R>(y, 2 * hn, 1, partial, norm2, s);
-    }
+    ilu_apply<R>(h, x, x + hn, y, y + hn, dagger, norm2);
   };
 }
 
@@ -2754,7 +2749,7 @@ int apply_line_abi(wf_handle* h, const double* in, double* out, int opu, int opl
   return WF_OK;
 }
 
-// M-tilde_ILU (dagger: gamma_5 M-tilde_ILU gamma_5) on full fields
+// M-tilde_ILU or its adjoint on full fields
 template <typename R>
 int apply_ilu_abi(wf_handle* h, const double* in, double* out, int dagger, int nrhs) {
   if (!h->gauge) throw Error(WF_EINVAL, "no gauge field loaded");
@@ -2768,9 +2763,9 @@ int apply_ilu_abi(wf_handle* h, const double* in, double* out, int dagger, int n
   Cx<R>* io = h->buf<Cx<R>>(pname<R>("ap_io"), nt);
   Cx<R>* oe = h->buf<Cx<R>>(pname<R>("ap_oe"), nt);
   Cx<R>* oo = h->buf<Cx<R>>(pname<R>("ap_oo"), nt);
-  { Prof P(h, pname<R>("import_spinor")); launch_import_spinor<R>(h->g, din, ie, io, nrhs, dagger, frame_rot(h, 0), frame_rot(h, 1), h->stream); }
-  for (int k = 0; k < nrhs; ++k) ilu_apply<R>(h, ie + k * hn, io + k * hn, oe + k * hn, oo + k * hn);
-  { Prof P(h, pname<R>("export_spinor")); launch_export_spinor<R>(h->g, oe, oo, dout, nrhs, dagger, frame_rot(h, 0), frame_rot(h, 1), h->stream); }
+  { Prof P(h, pname<R>("import_spinor")); launch_import_spinor<R>(h->g, din, ie, io, nrhs, 0, frame_rot(h, 0), frame_rot(h, 1), h->stream); }
+  for (int k = 0; k < nrhs; ++k) ilu_apply<R>(h, ie + k * hn, io + k * hn, oe + k * hn, oo + k * hn, dagger, nullptr);
+  { Prof P(h, pname<R>("export_spinor")); launch_export_spinor<R>(h->g, oe, oo, dout, nrhs, 0, frame_rot(h, 0), frame_rot(h, 1), h->stream); }
   finish_out(h, out, dout, le, staged);
   return WF_OK;
 }
@@ -2956,7 +2951,7 @@ int wf_load_gauge_clover(wf_handle_t* h, const double* U, double c_s, double c_t
     const size_t nh = (size_t)g.Nl * 72 * g.tp;
     for (int p = 0; p < 2; ++p) {
       h->clov64[p].ensure(nh * sizeof(Cx<double>), s);
-      h->clov32[p].ensure(nh * sizeof(Cx<float>), s);
+      h->clov32[p].ensure(nh / 2 * sizeof(Cx<float>), s);
       WF_CUDA(cudaMemsetAsync(h->clov64[p].p, 0, nh * sizeof(Cx<double>), s));  // padding slots stay zero
     }
     Cx<double>* F = h->buf<Cx<double>>("clover_F", V * 54);
@@ -2965,15 +2960,15 @@ int wf_load_gauge_clover(wf_handle_t* h, const double* U, double c_s, double c_t
     {
       Prof P(h, "clover_build", 2 + 2);
       launch_clover_build(g, dU, h->axial ? rot : nullptr, c_s, c_t, F, H, s);
-      for (int p = 0; p < 2; ++p) launch_d2f(H[p], h->clov32[p].as<Cx<float>>(), nh, s);
+      for (int p = 0; p < 2; ++p) launch_clover_pack(H[p], h->clov32[p].as<Cx<float>>(), (size_t)g.Nl * 2, g.tp, s);
     }
     if (g.T % 2 == 0) {  // the 4-D Schur comparator: mu + A and its inverse, 4-D even-odd layout
       const size_t n4 = (size_t)g.L * g.L * g.L * 72 * (g.T / 2);
       for (int p = 0; p < 2; ++p) {
         h->clmu64[p].ensure(n4 * sizeof(Cx<double>), s);
         h->clinv64[p].ensure(n4 * sizeof(Cx<double>), s);
-        h->clmu32[p].ensure(n4 * sizeof(Cx<float>), s);
-        h->clinv32[p].ensure(n4 * sizeof(Cx<float>), s);
+        h->clmu32[p].ensure(n4 / 2 * sizeof(Cx<float>), s);
+        h->clinv32[p].ensure(n4 / 2 * sizeof(Cx<float>), s);
       }
       const Cx<double>* Hc[2] = {H[0], H[1]};
       Cx<double>* M4[2] = {h->clmu64[0].as<Cx<double>>(), h->clmu64[1].as<Cx<double>>()};
@@ -2982,8 +2977,8 @@ int wf_load_gauge_clover(wf_handle_t* h, const double* U, double c_s, double c_t
       Prof P(h, "clover_eo4_build", 1 + 4);
       launch_clover_eo4_build(g, Hc, M4, Mi4, h->iflag.as<int>(), s);
       for (int p = 0; p < 2; ++p) {
-        launch_d2f(M4[p], h->clmu32[p].as<Cx<float>>(), n4, s);
-        launch_d2f(Mi4[p], h->clinv32[p].as<Cx<float>>(), n4, s);
+        launch_clover_pack(M4[p], h->clmu32[p].as<Cx<float>>(), (size_t)g.L * g.L * g.L * 2, g.T / 2, s);
+        launch_clover_pack(Mi4[p], h->clinv32[p].as<Cx<float>>(), (size_t)g.L * g.L * g.L * 2, g.T / 2, s);
       }
       int flag = 0;
       WF_CUDA(cudaMemcpyAsync(&flag, h->iflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -186,7 +186,7 @@ template <typename R>
 struct SetupArgs {
   Geom g;
   int line0;            // first line of this launch
-  const Cx<R>* H;       // clover blocks of the parity [Nl][2][36][tp] (H_a, H_b = half the chiral
+  const Cx<R>* H;       // clover blocks of the parity [Nl][2][36 (FP32: 18)][tp] (H_a, H_b = half the chiral
                         // blocks of A), or null: A = 0
   const Cx<R>* ut;      // general frame: U_t of the parity [Nl][9][tp]
   const Cx<R>* pl;      // axial frame: the boundary link P of every line [Nl][9]
@@ -214,7 +214,8 @@ __global__ void __launch_bounds__(kSetupThreads) k_qinv_setup(const SetupArgs<R>
   const int T = g.T, tp = g.tp;
   Cx<R>* S = A.sinv + (size_t)l * T * kBlk;
   const Cx<R>* ut = AX ? nullptr : A.ut + (size_t)l * 9 * tp;
-  const Cx<R>* Hl = A.H ? A.H + (size_t)l * 72 * tp : nullptr;
+  constexpr int HP = herm_planes<R>();
+  const Cx<R>* Hl = A.H ? A.H + (size_t)l * 2 * HP * tp : nullptr;
   const R mu = (R)g.mu;
 
   // block LU of T_0
@@ -227,7 +228,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_qinv_setup(const SetupArgs<R>
       Cx<R> v = mk<R>(r == c ? mu : R(0), R(0));
       if (Hl) {  // A = [[H_a + H_b, H_a - H_b], [H_a - H_b, H_a + H_b]] on the (P_+, P_-) halves
         const int i = r % 6, j = c % 6;
-        const Cx<R> ha = Hl[(size_t)(6 * i + j) * tp + sl], hb = Hl[(size_t)(36 + 6 * i + j) * tp + sl];
+        const Cx<R> ha = herm_entry(Hl, i, j, tp, sl), hb = herm_entry(Hl + (size_t)HP * tp, i, j, tp, sl);
         v = (r < 6) == (c < 6) ? v + ha + hb : v + ha - hb;
       }
       if (t > 0 && r < 6 && c >= 6) {
@@ -739,7 +740,7 @@ bool qinv_current(wf_handle* h, unsigned long long* key) {
     WF_CUDA(cudaGetLastError());
   };
   for (int p = 0; p < 2; ++p) {
-    if (h->clover) add(clover_of<R>(h, p), (size_t)g.Nl * 72 * g.tp * sizeof(Cx<R>), 0x1000ull + p);
+    if (h->clover) add(clover_of<R>(h, p), (size_t)g.Nl * 2 * herm_planes<R>() * g.tp * sizeof(Cx<R>), 0x1000ull + p);
     if (h->axial)
       add(gauge_pl<R>(h, p), (size_t)g.Nl * 9 * sizeof(Cx<R>), 0x2000ull + p);
     else

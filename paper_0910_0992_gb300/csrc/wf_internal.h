@@ -271,6 +271,8 @@ void launch_force(const ForceArgs& a, cudaStream_t s);
 // null in the caller's gauge); F_scratch holds V x 6 matrices
 void launch_clover_build(const Geom& g, const Cx<double>* U_lex, const Cx<double>* rot[2], double c_s, double c_t,
                          Cx<double>* F_scratch, Cx<double>* H[2], cudaStream_t s);
+// the FP32 copy of hermitian 6x6 blocks: nb blocks [36][inner] in FP64 to [18][inner] (wf_clover.cu)
+void launch_clover_pack(const Cx<double>* H, Cx<float>* out, size_t nb, int inner, cudaStream_t s);
 // out = acc + alpha A in on one parity (acc may be null; padding slots get acc or zero)
 template <typename R>
 void launch_clover_apply(const Geom& g, const Cx<R>* H, const Cx<R>* in, Cx<R>* out, const Cx<R>* acc, double alpha,
@@ -283,8 +285,5 @@ void launch_clover_apply_eo(const Geom& g, const Cx<R>* H, const Cx<R>* in, Cx<R
 // the line-layout blocks H; *singular set where mu + A has no inverse
 void launch_clover_eo4_build(const Geom& g, const Cx<double>* H[2], Cx<double>* M[2], Cx<double>* Minv[2],
                              int* singular, cudaStream_t s);
-// out = in with the spin halves exchanged, n elements of [..][12][tp] fields
-template <typename R>
-void launch_swap_halves(const Cx<R>* in, Cx<R>* out, size_t n, int tp, cudaStream_t s);
 
 }  // namespace wf

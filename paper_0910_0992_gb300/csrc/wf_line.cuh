@@ -351,6 +351,27 @@ __device__ __forceinline__ Vec3<R> vadd(const Vec3<R>& x, const Vec3<R>& y) {
 
 // |x|^2 in the field's own precision (GB300's FP64 rate is far below its FP32 rate, so FP32
 // kernels keep FP64 for the final cross-thread sums only)
+// Hermitian 6x6 blocks over slots (the clover term): FP64 whole, [36][stride]; FP32 the diagonal in
+// pairs, then the entries below it, (r, c) at plane 3 + r (r - 1) / 2 + c: [18][stride]
+template <typename R>
+__host__ __device__ constexpr int herm_planes() {
+  return sizeof(R) == 8 ? 36 : 18;
+}
+template <typename R>
+__device__ __forceinline__ Cx<R> herm_entry(const Cx<R>* H, int r, int c, size_t stride, int sl) {
+  if constexpr (sizeof(R) == 8) {
+    return H[(6 * r + c) * stride + sl];
+  } else {
+    if (r == c) {
+      const Cx<R> d = H[(r / 2) * stride + sl];
+      return mk<R>(r % 2 ? d.im : d.re, R(0));
+    }
+    const int hi = r > c ? r : c, lo = r > c ? c : r;
+    const Cx<R> e = H[(3 + hi * (hi - 1) / 2 + lo) * stride + sl];
+    return mk<R>(e.re, r > c ? e.im : -e.im);
+  }
+}
+
 template <typename R>
 __device__ __forceinline__ R vnorm2(const Vec3<R>& x) {
   R s = R(0);
