@@ -2292,6 +2292,30 @@ void ilu_apply(wf_handle* h, const Cx<R>* pe, const Cx<R>* po, Cx<R>* ce, Cx<R>*
   Cx<R>* d = h->buf<Cx<R>>(pname<R>("il_d"), hn);
   Cx<R>* t2 = h->buf<Cx<R>>(pname<R>("il_t2"), hn);
   Cx<R>* e = h->buf<Cx<R>>(pname<R>("il_e"), hn);
+  if constexpr (sizeof(R) == 4) {
+    if (h->clover && h->g.n <= NMAX) {  // C_R, A, C_L and the axpys around them in one kernel per parity
+      auto abar = [&](int p, const Cx<R>* x, const Cx<R>* y, Cx<R>* out, Cx<R>* out2, double* nrm, const char* name) {
+        AbarArgs b;
+        std::memset(&b, 0, sizeof(b));
+        b.line = line_args<R>(h, p, 1);
+        b.H = clover_blocks<R>(h, p);
+        b.x = x;
+        b.y = y;
+        b.f = (R)g;
+        b.dagger = dagger;
+        b.out = out;
+        b.out2 = out2;
+        b.norm2 = nrm;
+        Prof P(h, pname<R>(name));
+        launch_abar(b, h->axial, p == 1, s);
+      };
+      abar(1, po, nullptr, a, e, nullptr, "il_abar_odd");
+      step(0, SRC_HOP, a, u, OP_COPY, OP_BWD, nullptr, 0.0, nullptr, 0.0, "il_hop_c_left");
+      abar(0, pe, u, c, ce, norm2, "il_abar_even");
+      step(1, SRC_HOP, c, co, OP_COPY, OP_BWD, nullptr, 0.0, e, g, "il_hop_c_left", norm2);
+      return;
+    }
+  }
   step(1, SRC_LOAD, po, a, OP_FWD, OP_COPY, nullptr, 0.0, nullptr, 0.0, "il_c_right");  // a = C_R^o psi_o
   step(0, SRC_HOP, a, u, OP_COPY, OP_BWD, nullptr, 0.0, nullptr, 0.0, "il_hop_c_left");  // u = C_L^e D a
   if (h->clover) {

@@ -27,6 +27,7 @@
 #include "../../include/wf.h"
 #include "wf_internal.h"
 #include "wf_line.cuh"
+#include "wf_line_kernels.cuh"
 
 namespace wf {
 
@@ -219,6 +220,103 @@ __global__ void __launch_bounds__(kBlock) k_clover_apply(const Geom g, const Cx<
   }
 }
 
+// One line of Abar = C_L A C_R and the steps around it in M-tilde_ILU (ilu_apply), FP32: a warp (or
+// part of one) holds the line's spinors in registers through the time-line operations on one spin
+// half, the clover blocks and the operation on the other half, n sites per lane as in k_line.
+//   ODD:   a = C_R x, e = x + C_L A a                                       (out = a, out2 = e)
+//   else:  t = C_L A C_R (x + f y), chi = x + t, c = C_R (t - f y)          (out = c, out2 = chi, |chi|^2)
+// The adjoint exchanges the roles of the halves (C_R acts on `up`). The separate
+// kernels passed the spinors through L2 five times per line. Bound by the latency of its three solves
+// and of the blocks' loads (the register file holds 8 warps an SM; at 12 and 16 the spinors spill: 81, 75
+// against 69 us for the even parity of 16^3 x 128): 155 -> 113 us for both parities kernel by kernel, the
+// solve 19.3 -> 18.9 ms, its first pass 22.0 -> 20.9 ms
+template <bool AX, bool ODD>
+__global__ void __launch_bounds__(32, 8) k_abar(const AbarArgs B) {
+  using R = float;
+  const LineArgs<R>& A = B.line;
+  const Geom& g = A.g;
+  const int lane = threadIdx.x;
+  const int lg_raw = blockIdx.x * g.lpw + lane / g.lpl;
+  const bool active = lg_raw < g.Nl;
+  const int l = active ? lg_raw : 0;  // idle lanes still join the warp shuffles
+  const int jj = lane % g.lpl;
+  const int tp = g.tp, n = g.n;
+  const size_t base = (size_t)l * NSPIN_C * tp;
+  const int up = B.dagger ? 6 * tp : 0;
+  // element offset of spin s (0, 1: the half of C_R) at site m
+  auto at = [&](int s, int m) { return base + (s < 2 ? up : 6 * tp - up) + 3 * (s & 1) * tp + m * g.lpl + jj; };
+  auto valid = [&](int m) { return m < n && jj * n + m < g.T; };
+  const Cx<R>* H = B.H + (size_t)l * 2 * herm_planes<R>() * tp;
+  Vec3<R> v[NMAX][4];
+#pragma unroll
+  for (int m = 0; m < NMAX; ++m)
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      v[m][s] = vzero<R>();
+      if (!valid(m)) continue;
+      if (ODD)
+        v[m][s] = ldvec(B.x + at(s, m), tp, 0);
+      else
+        v[m][s] = vaxpy(B.f, ldvec(B.y + at(s, m), tp, 0), ldvec(B.x + at(s, m), tp, 0));
+    }
+  solve_half<R, AX, true>(v, 0, A, l, jj);
+#pragma unroll
+  for (int m = 0; m < NMAX; ++m) {
+    if (!valid(m)) continue;
+    if (ODD && active) {
+#pragma unroll
+      for (int s = 0; s < 4; ++s) stvec(B.out + at(s, m), tp, 0, v[m][s]);
+    }
+    Cx<R> sv[6], dv[6], ya[6], yb[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const Cx<R> u = v[m][i / 3].c[i % 3], lo = v[m][2 + i / 3].c[i % 3];
+      sv[i] = u + lo;
+      dv[i] = u - lo;
+    }
+    const Cx<R>* Hm = H + m * g.lpl + jj;
+    herm_times<R>(Hm, Hm + (size_t)herm_planes<R>() * tp, tp, sv, dv, ya, yb);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      v[m][i / 3].c[i % 3] = ya[i] + yb[i];
+      v[m][2 + i / 3].c[i % 3] = ya[i] - yb[i];
+    }
+  }
+  solve_half<R, AX, false>(v, 2, A, l, jj);
+  R nrm = R(0);
+#pragma unroll
+  for (int m = 0; m < NMAX; ++m) {
+    if (m >= n) continue;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const bool ok = valid(m);
+      const Vec3<R> sum = ok ? vaxpy(R(1), v[m][s], ldvec(B.x + at(s, m), tp, 0)) : vzero<R>();
+      if (active) {
+        stvec(B.out2 + at(s, m), tp, 0, sum);
+        if (ODD && !ok) stvec(B.out + at(s, m), tp, 0, sum);  // padding: zero
+      }
+      if (!ODD) {
+        nrm += vnorm2(sum);
+        v[m][s] = ok ? vaxpy(-B.f, ldvec(B.y + at(s, m), tp, 0), v[m][s]) : vzero<R>();
+      }
+    }
+  }
+  if (ODD) return;
+  solve_half<R, AX, true>(v, 0, A, l, jj);
+#pragma unroll
+  for (int m = 0; m < NMAX; ++m) {
+    if (m >= n || !active) continue;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) stvec(B.out + at(s, m), tp, 0, valid(m) ? v[m][s] : vzero<R>());
+  }
+  if (B.norm2) {
+    double dn = active ? (double)nrm : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dn += __shfl_down_sync(0xffffffffu, dn, o);
+    if (lane == 0) atomicAdd(B.norm2, dn);
+  }
+}
+
 // The 4-D even-odd blocks of mu + A and of its inverse, from the line-layout blocks H = A_k / 2:
 // one thread per site and chiral block; B = mu 1 + A_k (6x6), B^-1 by Gauss-Jordan elimination
 // with partial pivoting; stored halved like H. Sets *singular when a pivot vanishes.
@@ -398,6 +496,17 @@ void launch_clover_eo4_build(const Geom& g, const Cx<double>* H[2], Cx<double>* 
 void launch_clover_pack(const Cx<double>* H, Cx<float>* out, size_t nb, int inner, cudaStream_t s) {
   const size_t n = nb * 18 * inner;
   k_clover_pack<<<grid_of(n), kBlock, 0, s>>>(H, out, n, inner);
+  WF_CUDA(cudaGetLastError());
+}
+
+void launch_abar(const AbarArgs& a, bool axial, bool odd, cudaStream_t s) {
+  const Geom& g = a.line.g;
+  if (g.n < 1 || g.n > NMAX) throw Error(WF_EINVAL, "Abar kernel: unsupported sites per lane");
+  const unsigned blocks = (unsigned)((g.Nl + g.lpw - 1) / g.lpw);
+  if (axial)
+    odd ? k_abar<true, true><<<blocks, 32, 0, s>>>(a) : k_abar<true, false><<<blocks, 32, 0, s>>>(a);
+  else
+    odd ? k_abar<false, true><<<blocks, 32, 0, s>>>(a) : k_abar<false, false><<<blocks, 32, 0, s>>>(a);
   WF_CUDA(cudaGetLastError());
 }
 

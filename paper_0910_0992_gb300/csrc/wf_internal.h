@@ -277,6 +277,9 @@ void launch_clover_pack(const Cx<double>* H, Cx<float>* out, size_t nb, int inne
 template <typename R>
 void launch_clover_apply(const Geom& g, const Cx<R>* H, const Cx<R>* in, Cx<R>* out, const Cx<R>* acc, double alpha,
                          int nrhs, cudaStream_t s);
+struct AbarArgs;
+// C_L A C_R with the steps around it in M-tilde_ILU, on one parity (FP32, lines of up to 128 slots)
+void launch_abar(const AbarArgs& a, bool axial, bool odd, cudaStream_t s);
 // the same on a 4-D even-odd field [rhs][L^3][12][T/2] with blocks [L^3][2][36][T/2]
 template <typename R>
 void launch_clover_apply_eo(const Geom& g, const Cx<R>* H, const Cx<R>* in, Cx<R>* out, const Cx<R>* acc,

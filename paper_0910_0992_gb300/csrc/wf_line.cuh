@@ -88,6 +88,20 @@ struct LineArgs {
   const int* active;
 };
 
+// Arguments of the clover ILU's fused line kernel (k_abar, wf_clover.cu; one right-hand side). x is
+// psi_o (odd) or psi_e with y = u, f = 1 / gamma_f; H the parity's packed clover blocks
+struct AbarArgs {
+  LineArgs<float> line;
+  const Cx<float>* H;
+  const Cx<float>* x;
+  const Cx<float>* y;
+  float f;
+  int dagger;
+  Cx<float>* out;
+  Cx<float>* out2;
+  double* norm2;
+};
+
 // Arguments of one launch over a ragged batch of lattices (kMaxLattices at most per launch): the
 // per-lattice arguments and the first block of each lattice (blk0[n] = total blocks).
 constexpr int kMaxLattices = 8;
