@@ -68,6 +68,19 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
     return;
   }
   // FP64 kernels only load their own site: their hops have run in fixed point (launch_line)
+  if constexpr (std::is_same<R, double>::value) {
+    if (few_lines(a.g, a.nrhs)) {
+      LineArgs<R> q = a;
+      if (kind == LK_SCHUR_A) {
+        q.opu = OP_FWD;
+        q.opl = OP_SKIP;
+      }
+      const dim3 grid(line_warps(a.g, a.nrhs), 4);
+      axial ? k_line_spin<true><<<grid, 32, 0, s>>>(q) : k_line_spin<false><<<grid, 32, 0, s>>>(q);
+      WF_CUDA(cudaGetLastError());
+      return;
+    }
+  }
   constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;
   constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
 #define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV><<<b, th, 0, s>>>(a)

@@ -19,10 +19,10 @@ constexpr int kLineThreads = 128;
 // on GB300 against 1 and 4, where 4 spills)
 template <typename R, bool AX, bool FWD, int NM, int W>
 __device__ __forceinline__ void solve_half(Vec3<R> (&v)[NM][W], int s0, const LineArgs<R>& A, int l, int jj) {
-  constexpr int NS = sizeof(R) == 4 ? 2 : 1;
+  constexpr int NS = sizeof(R) == 4 && W > 1 ? 2 : 1;
   const Geom& g = A.g;
 #pragma unroll
-  for (int sp = 0; sp < 2; sp += NS) {
+  for (int sp = 0; sp < (W < 2 ? W : 2); sp += NS) {
     Vec3<R> w[NM][NS];
 #pragma unroll
     for (int m = 0; m < NM; ++m)
@@ -60,21 +60,22 @@ __device__ __forceinline__ void store_spin(const LineArgs<R>& A, size_t base, in
   if (A.norm2) nrm += vnorm2(val);
 }
 
-// One spin half of a line kernel that loads its own site: load, pre-axpy, time-line operation, store
-template <typename R, bool AX, bool H, int NM>
+// One spin half of a line kernel that loads its own site, or with W = 1 spin s0 of it: load, pre-axpy,
+// time-line operation, store
+template <typename R, bool AX, bool H, int NM, int W = 2>
 __device__ __forceinline__ void load_half(const LineArgs<R>& A, int h, int op, size_t base, int l, int jj, bool active,
-                                          R& nrm) {
+                                          R& nrm, int s0 = 0) {
   const Geom& g = A.g;
   const int tp = g.tp, n = g.n;
   const Cx<R>* src = h ? A.src_lo : A.src_up;
-  Vec3<R> v[NM][2];
+  Vec3<R> v[NM][W];
 #pragma unroll
   for (int m = 0; m < NM; ++m)
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < W; ++s) {
       const int sl = m * g.lpl + jj;
-      v[m][s] = m < n ? ldv<R, H>(src, base + 3 * s * tp, tp, sl) : vzero<R>();
-      if (A.xpre && m < n) v[m][s] = vaxpy(A.apre, v[m][s], ldv<R, H>(A.xpre, base + (6 * h + 3 * s) * tp, tp, sl));
+      v[m][s] = m < n ? ldv<R, H>(src, base + 3 * (s0 + s) * tp, tp, sl) : vzero<R>();
+      if (A.xpre && m < n) v[m][s] = vaxpy(A.apre, v[m][s], ldv<R, H>(A.xpre, base + (6 * h + 3 * (s0 + s)) * tp, tp, sl));
     }
   apply_op<R, AX>(op, v, 0, A, l, jj);
   if (!active) return;
@@ -82,8 +83,21 @@ __device__ __forceinline__ void load_half(const LineArgs<R>& A, int h, int op, s
   for (int m = 0; m < NM; ++m) {
     if (m >= n) continue;
 #pragma unroll
-    for (int s = 0; s < 2; ++s) store_spin<R, H>(A, base, h, s, m * g.lpl + jj, jj * n + m < g.T, v[m][s], nrm);
+    for (int s = 0; s < W; ++s) store_spin<R, H>(A, base, h, s0 + s, m * g.lpl + jj, jj * n + m < g.T, v[m][s], nrm);
   }
+}
+
+// *norm2 += the lanes' nrm; lanes of one line share rhs: reduced over the warp per line group, one
+// atomic per line
+template <typename R>
+__device__ __forceinline__ void line_norm(const LineArgs<R>& A, R nrm, int rhs, int jj, bool active) {
+  double dn = (double)nrm;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double other = __shfl_down_sync(0xffffffffu, dn, o);
+    if (o < A.g.lpl) dn += other;
+  }
+  if (active && jj == 0) atomicAdd(A.norm2 + rhs, dn);
 }
 
 // SRC, OPU, OPL < 0: taken from the arguments at run time
@@ -173,21 +187,34 @@ __device__ __forceinline__ void line_body(const LineArgs<R>& A, int blk) {
     }
   }
   }
-  if (want_norm) {
-    // lanes of one line share rhs; reduce over the warp per line group, one atomic per line
-    double dn = (double)nrm;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double other = __shfl_down_sync(0xffffffffu, dn, o);
-      if (o < g.lpl) dn += other;
-    }
-    if (active && jj == 0) atomicAdd(A.norm2 + rhs, dn);
-  }
+  if (want_norm) line_norm(A, nrm, rhs, jj, active);
 }
 
 template <typename R, bool AX, int SRC, int OPU, int OPL, bool H = false, int NM = NMAX>
 __global__ void __launch_bounds__(kLineThreads, LineMinBlocks<R>::value) k_line(const LineArgs<R> A) {
   line_body<R, AX, SRC, OPU, OPL, H, NM>(A, blockIdx.x);
+}
+
+// A line operation without a hop on a small lattice, bound by the latency of its chain of loads, scan
+// and wrap: a warp takes one of the line's four spins (blockIdx.y) instead of all of them in turn, so
+// that four times the warps share the chain. FP64, us
+// (4^3 x 16; 8^3 x 32; 8^3 x 32 with two sources): hop and K-b 41 -> 31; 43 -> 33; 46 -> 42, T^-1 22 -> 12;
+// 24 -> 14; 25 -> 22. FP32 (K-a 7.5 us of which most is the launch) gains nothing.
+template <bool AX>
+__global__ void __launch_bounds__(32) k_line_spin(const LineArgs<double> A) {
+  using R = double;
+  const Geom& g = A.g;
+  const int h = blockIdx.y >> 1, op = h ? A.opl : A.opu;
+  if (op == OP_SKIP) return;
+  const int lane = threadIdx.x, jj = lane % g.lpl;
+  const int lg_raw = (int)blockIdx.x * g.lpw + lane / g.lpl;
+  const bool active = lg_raw < A.nrhs * g.Nl;
+  int rhs, l;
+  line_rhs(active ? lg_raw : 0, A.nrhs, g, rhs, l);
+  if (A.active && g.lpw == 1 && !A.active[rhs]) return;
+  R nrm = R(0);
+  load_half<R, AX, false, NMAX, 1>(A, h, op, ((size_t)rhs * g.Nl + l) * NSPIN_C * g.tp, l, jj, active, nrm, blockIdx.y & 1);
+  if (A.norm2) line_norm(A, nrm, rhs, jj, active);
 }
 
 // one launch over a ragged batch of lattices (MultiLineArgs, wf_line.cuh)
@@ -204,12 +231,13 @@ inline int line_blocks(const LineArgs<R>& a, int threads = kLineThreads) {
   return (line_warps(a.g, a.nrhs) * 32 + threads - 1) / threads;
 }
 // CTA size: one warp where the lattice has fewer than four per SM, so that they spread over all SMs
-// (an FP64 warp then shares an SM's FP64 pipe with no other; K-a in FP64 on 4^3 x 16: 17 -> 14 us)
+// (FP64 then also splits a line's spins, k_line_spin: with 1024 warps that is slower, K-a 19 -> 22 us on
+// 8^3 x 32 with four sources)
+inline bool few_lines(const Geom& g, int nrhs) { return line_warps(g, nrhs) < 4 * 152; }
 template <typename R>
 inline int line_threads(const LineArgs<R>& a) {
-  return line_warps(a.g, a.nrhs) < 4 * 152 ? 32 : kLineThreads;
+  return few_lines(a.g, a.nrhs) ? 32 : kLineThreads;
 }
-
 // ----------------------------------------------------------------------------
 // Wilson matrix M = mu - D_t - D_s / gamma_f (§II, Eq. for M) on the output parity:
 // out_p = mu psi_p - D_t psi_p - D_s psi_q / gamma_f   (or x + a * that).
