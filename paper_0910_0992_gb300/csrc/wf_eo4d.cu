@@ -209,13 +209,13 @@ struct EoDir {
 
 // The dslash in FP64, spatial hops in block fixed point (wf_fixed.cuh); sites, arguments and results of
 // k_dslash4. 16^3 x 96, 4 sources: 1.16 ms with every operation in FP64, 0.42 ms so.
-template <bool AX>
-__global__ void __launch_bounds__(kEoThreads, 4) k_dslash4_fx(const EoArgs<double> A) {
+template <bool AX, int S>
+__global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_dslash4_fx(const EoArgs<double> A) {
   const Geom& g = A.g;
   const int Th = g.T / 2, L = g.L;
   const size_t V3 = (size_t)L * L * L;
   const size_t total = (size_t)A.nrhs * V3 * Th;
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const size_t i = fx_site<S>();
   const bool active = i < total;
   const size_t ii = active ? i : 0;
   const int h = (int)(ii % Th);
@@ -233,11 +233,9 @@ __global__ void __launch_bounds__(kEoThreads, 4) k_dslash4_fx(const EoArgs<doubl
   const int cu = A.swap_in ? 6 : 0, cl = A.swap_in ? 0 : 6;
 
   Vec3<double> acc[4];
-  double unit = 0.0;
-  if (active) {
-    const EoDir dir{A, x, y, z, p3, l, sl, h, A.in + (size_t)rhs * V3 * fstride, cu, cl};
-    unit = hop_fx(dir, Th, tp, acc) * A.inv_gf;
-  }
+  const EoDir dir{A, x, y, z, p3, l, sl, h, A.in + (size_t)rhs * V3 * fstride, cu, cl};
+  const double unit = hop_fx<S>(dir, Th, tp, active, acc) * A.inv_gf;
+  if (S > 1 && threadIdx.x >= 32) return;
   // temporal hops: P_- U_t(t) psi(t+1) on spins 2-3, P_+ U_t^dag(t-1) psi(t-1) on spins 0-1
   const Cx<double>* own = A.in + ((size_t)rhs * V3 + s3) * fstride;
   const int hf = (t == g.T - 1) ? 0 : (t + 1) / 2;  // other-parity index of t + 1
@@ -337,12 +335,11 @@ void launch_dslash4(const EoArgs<R>& a, bool axial, cudaStream_t s) {
   if constexpr (std::is_same<R, double>::value) {
     if (!a.fx[0] || !a.fx[1]) throw Error(1, "FP64 dslash: no fixed-point links");
     const size_t total = (size_t)a.nrhs * a.g.L * a.g.L * a.g.L * (a.g.T / 2);
-    const int th = total < (size_t)152 * kEoThreads ? 32 : kEoThreads;  // one warp per CTA on small lattices
-    const unsigned blocks = (unsigned)((total + th - 1) / th);
-    if (axial)
-      k_dslash4_fx<true><<<blocks, th, fx_smem(th), s>>>(a);
-    else
-      k_dslash4_fx<false><<<blocks, th, fx_smem(th), s>>>(a);
+    fx_launch(total, [&](auto S, unsigned b, int th, size_t smem) {
+      auto* k = axial ? k_dslash4_fx<true, S.value> : k_dslash4_fx<false, S.value>;
+      fx_allow(k, smem);
+      k<<<b, th, smem, s>>>(a);
+    });
     WF_CUDA(cudaGetLastError());
   } else {
     launch_dslash4_impl<R>(a, axial, s);

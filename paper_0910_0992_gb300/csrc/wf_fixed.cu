@@ -10,9 +10,6 @@ namespace wf {
 
 namespace {
 
-constexpr int kFxThreads = 128;
-constexpr int kFxMinBlocks = 4;  // CTAs per SM (3, without spills: 4 % slower; 24^3 x 128, 12 sources)
-
 // direction d of line l's site (parity, source rhs, slot sl) in the line layout
 struct LineDir {
   const Geom& g;
@@ -43,9 +40,8 @@ struct LineDir {
   }
 };
 
-// thread -> (source, line, slot), slots fastest, in the line kernels' traversal
-__device__ __forceinline__ bool site_at(const Geom& g, int nrhs, int& rhs, int& l, int& sl, int& t) {
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+// site -> (source, line, slot), slots fastest, in the line kernels' traversal
+__device__ __forceinline__ bool site_at(const Geom& g, size_t i, int nrhs, int& rhs, int& l, int& sl, int& t) {
   const int lg = (int)(i / g.tp);
   sl = (int)(i - (size_t)lg * g.tp);
   const bool in = lg < nrhs * g.Nl;
@@ -56,18 +52,22 @@ __device__ __forceinline__ bool site_at(const Geom& g, int nrhs, int& rhs, int& 
 
 // out = v, v = xpre + apre D_s src (xpre null: D_s src), with the spin halves exchanged if swap_out;
 // post: out = xpost + apost v. Padding slots zero (post: xpost).
-__global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_hop_fx(const LineArgs<double> A, int post) {
+// (3 CTAs per SM, without spills: 4 % slower; 24^3 x 128, 12 sources)
+template <int S>
+__global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks)
+    k_hop_fx(const LineArgs<double> A, int post) {
   const Geom& g = A.g;
   int rhs, l, sl, t;
-  if (!site_at(g, A.nrhs, rhs, l, sl, t)) return;
-  if (A.active && g.lpw == 1 && !A.active[rhs]) return;  // as the line kernels skip them
+  bool in = site_at(g, fx_site<S>(), A.nrhs, rhs, l, sl, t);
+  if (A.active && g.lpw == 1 && !A.active[rhs]) in = false;  // as the line kernels skip them
   const int tp = g.tp;
   const size_t base = ((size_t)rhs * g.Nl + l) * NSPIN_C * tp;
   Vec3<double> h[4];
-  double unit = 0.0;
-  if (t < g.T) {
-    unit = hop_fx(LineDir(g, A.parity, rhs, l, sl, A.src_up, A.src_lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, h);
-  } else {
+  const bool site = in && t < g.T;
+  double unit = hop_fx<S>(
+      LineDir(g, A.parity, rhs, l, sl, A.src_up, A.src_lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site, h);
+  if (!in || (S > 1 && threadIdx.x >= 32)) return;
+  if (!site) {
 #pragma unroll
     for (int s = 0; s < 4; ++s) h[s] = vzero<double>();
   }
@@ -89,22 +89,21 @@ __global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_hop_fx(const LineA
 }
 
 // The Wilson matrix on the output parity (k_apply_M of wf_line_kernels.cuh), one thread per site
-template <bool AX>
-__global__ void __launch_bounds__(kFxThreads, kFxMinBlocks) k_apply_M_fx(const MArgs<double> A) {
+template <bool AX, int S>
+__global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_apply_M_fx(const MArgs<double> A) {
   const Geom& g = A.g;
   int rhs, l, sl, t;
-  const bool in = site_at(g, A.nrhs, rhs, l, sl, t);
+  const bool in = site_at(g, fx_site<S>(), A.nrhs, rhs, l, sl, t);
   const int tp = g.tp, T = g.T;
   const size_t base = ((size_t)rhs * g.Nl + l) * NSPIN_C * tp;
   const bool site = in && t < T;
   const Cx<double>* pp = A.psi_p + base;
   Vec3<double> h[4];
-  double unit = 0.0;
-  if (site) {
-    const Cx<double>* up = A.psi_q + (A.swap ? 6 * tp : 0);
-    const Cx<double>* lo = A.psi_q + (A.swap ? 0 : 6 * tp);
-    unit = hop_fx(LineDir(g, A.parity, rhs, l, sl, up, lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, h);
-  }
+  const Cx<double>* up = A.psi_q + (A.swap ? 6 * tp : 0);
+  const Cx<double>* lo = A.psi_q + (A.swap ? 0 : 6 * tp);
+  const double unit =
+      hop_fx<S>(LineDir(g, A.parity, rhs, l, sl, up, lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site, h);
+  if (S > 1 && threadIdx.x >= 32) return;
   // axial frame: spins 0-1 at t = 0 need P^dag psi(T - 1), spins 2-3 at t = T - 1 P psi(0)
   Vec3<double> wr[2];
   wr[0] = wr[1] = vzero<double>();
@@ -145,9 +144,6 @@ __global__ void k_links_fx(const Cx<double>* __restrict__ in, int4* __restrict__
   }
 }
 
-// CTA size: one warp where the lattice is too small to give every SM four
-int fx_threads(size_t sites) { return sites < (size_t)152 * kFxThreads ? 32 : kFxThreads; }
-
 }  // namespace
 
 void launch_links_fx(const Cx<double>* in, int4* out, size_t n, cudaStream_t s) {
@@ -158,21 +154,20 @@ void launch_links_fx(const Cx<double>* in, int4* out, size_t n, cudaStream_t s) 
 
 void launch_hop_fx(const LineArgs<double>& a, bool post, cudaStream_t s) {
   if (!a.fx_out || !a.fx_nbr) throw Error(1, "FP64 hop: no fixed-point links");
-  const size_t sites = (size_t)a.nrhs * a.g.Nl * a.g.tp;
-  const int th = fx_threads(sites);
-  k_hop_fx<<<(unsigned)((sites + th - 1) / th), th, fx_smem(th), s>>>(a, post ? 1 : 0);
+  fx_launch((size_t)a.nrhs * a.g.Nl * a.g.tp, [&](auto S, unsigned b, int th, size_t smem) {
+    fx_allow(k_hop_fx<S.value>, smem);
+    k_hop_fx<S.value><<<b, th, smem, s>>>(a, post ? 1 : 0);
+  });
   WF_CUDA(cudaGetLastError());
 }
 
 void launch_apply_M_fx(const MArgs<double>& a, bool axial, cudaStream_t s) {
   if (!a.fx_out || !a.fx_nbr) throw Error(1, "FP64 Wilson matrix: no fixed-point links");
-  const size_t sites = (size_t)a.nrhs * a.g.Nl * a.g.tp;
-  const int th = fx_threads(sites);
-  const unsigned b = (unsigned)((sites + th - 1) / th);
-  if (axial)
-    k_apply_M_fx<true><<<b, th, fx_smem(th), s>>>(a);
-  else
-    k_apply_M_fx<false><<<b, th, fx_smem(th), s>>>(a);
+  fx_launch((size_t)a.nrhs * a.g.Nl * a.g.tp, [&](auto S, unsigned b, int th, size_t smem) {
+    auto* k = axial ? k_apply_M_fx<true, S.value> : k_apply_M_fx<false, S.value>;
+    fx_allow(k, smem);
+    k<<<b, th, smem, s>>>(a);
+  });
   WF_CUDA(cudaGetLastError());
 }
 

@@ -19,6 +19,9 @@
 // an infinity or exponents near the ends of FP64's range take the FP64 form (hop_dir_fp64).
 #pragma once
 
+#include <type_traits>
+
+#include "wf_internal.h"
 #include "wf_line.cuh"
 
 namespace wf {
@@ -220,11 +223,27 @@ __device__ __forceinline__ void fx_copy(int4* dst, const void* src) {
 constexpr int kFxStage = 21 * 32;
 inline size_t fx_smem(int threads) { return (size_t)threads / 32 * kFxStage * sizeof(int4); }
 
-// returns unit, with unit h = D_s (so that the scale joins the next multiply-add)
-template <class Dir>
-__device__ __forceinline__ double hop_fx(const Dir& dir, int cs, int ls, Vec3<double> (&h)[4]) {
+// CTA size, resident CTAs per SM (128 registers a thread) and the thread's site for a hop split over S warps
+// (S = 1: one thread per site)
+template <int S>
+struct FxShape {
+  static constexpr int threads = S == 1 ? 128 : 32 * S, blocks = S == 1 ? 4 : 16 / S;
+};
+template <int S>
+__device__ __forceinline__ size_t fx_site() {
+  return S == 1 ? blockIdx.x * (size_t)blockDim.x + threadIdx.x : blockIdx.x * (size_t)32 + (threadIdx.x & 31);
+}
+
+// returns unit, with unit h = D_s (so that the scale joins the next multiply-add). With S > 1 the S warps
+// of a CTA take 6 / S directions each of the same 32 sites and warp 0 adds them up (integers: exactly,
+// but for the shift to a common exponent that the six directions of one thread see as well); the others
+// have no result. Called by every thread of the CTA; site: whether the thread has one.
+template <int S, class Dir>
+__device__ __forceinline__ double hop_fx(const Dir& dir, int cs, int ls, bool site, Vec3<double> (&h)[4]) {
   extern __shared__ int4 fx_shared[];
   int4* stage = fx_shared + (threadIdx.x >> 5) * kFxStage + (threadIdx.x & 31);
+  constexpr int N = 6 / S;
+  const int d0 = S == 1 ? 0 : (threadIdx.x >> 5) * N;
   FxAcc f;
   fx_clear(f);
   auto fetch_spinor = [&](const HopDir& q) {
@@ -240,31 +259,70 @@ __device__ __forceinline__ double hop_fx(const Dir& dir, int cs, int ls, Vec3<do
     for (int e = 0; e < 9; ++e) fx_copy(stage + 32 * (12 + e), q.fx + (size_t)e * ls);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  HopDir next = dir(0);
-  fetch_spinor(next);
-  fetch_link(next);
+  if (site) {
+    HopDir next = dir(d0);
+    fetch_spinor(next);
+    fetch_link(next);
 #pragma unroll 1
-  for (int d = 0; d < 6; ++d) {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    FxHalf q;
-    {
-      Vec3<double> v[4];
+    for (int d = d0; d < d0 + N; ++d) {
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      FxHalf q;
+      {
+        Vec3<double> v[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) v[s].c[c] = *reinterpret_cast<const Cx<double>*>(stage + 32 * (3 * s + c));
+        fx_project(f, q, d, v);
+      }
+      if (d < d0 + N - 1) {
+        next = dir(d + 1);
+        fetch_spinor(next);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      fx_multiply(f, q, d, stage + 32 * 12, 32);
+      if (d < d0 + N - 1) fetch_link(next);
+    }
+  }
+  if constexpr (S > 1) {  // the stage is free: each lane's sums there, then warp 0 collects them
+    longlong2* box = reinterpret_cast<longlong2*>(stage);
+    if (d0) {
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) v[s].c[c] = *reinterpret_cast<const Cx<double>*>(stage + 32 * (3 * s + c));
-      fx_project(f, q, d, v);
+        for (int c = 0; c < 3; ++c) box[32 * (3 * s + c)] = make_longlong2(f.a[s][c][0], f.a[s][c][1]);
+      stage[32 * 12] = make_int4(f.E, f.wide, 0, 0);
     }
-    if (d < 5) {
-      next = dir(d + 1);
-      fetch_spinor(next);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (d0) return 0.0;
+    int E[S];
+    E[0] = f.E;
+#pragma unroll
+    for (int p = 1; p < S; ++p) {
+      const int4 o = stage[p * kFxStage + 32 * 12];
+      E[p] = o.x;
+      f.E = max(f.E, o.x);
+      f.wide = f.wide || o.y;
     }
-    fx_multiply(f, q, d, stage + 32 * 12, 32);
-    if (d < 5) fetch_link(next);
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int s0 = min(f.E - E[0], 63);
+        f.a[s][c][0] >>= s0;
+        f.a[s][c][1] >>= s0;
+#pragma unroll
+        for (int p = 1; p < S; ++p) {
+          const longlong2 o = box[p * kFxStage + 32 * (3 * s + c)];
+          const int sp = min(f.E - E[p], 63);
+          f.a[s][c][0] += o.x >> sp;
+          f.a[s][c][1] += o.y >> sp;
+        }
+      }
   }
+  if (!site) return 0.0;
   if (f.wide) {
     double o[24];
     for (int i = 0; i < 24; ++i) o[i] = 0.0;
@@ -281,6 +339,33 @@ __device__ __forceinline__ double hop_fx(const Dir& dir, int cs, int ls, Vec3<do
 #pragma unroll
     for (int c = 0; c < 3; ++c) h[s].c[c] = mk<double>((double)f.a[s][c][0], (double)f.a[s][c][1]);
   return fx_unit(f);
+}
+
+// Launch shape of a hop over `sites`: run(S, blocks, threads, dynamic shared memory) with the directions
+// split over as many warps S (std::integral_constant) as still leaves every CTA resident at once; the
+// chain of six spinor and link fetches is what bounds few sites. The Wilson matrix on one parity, us with
+// S = 1, 2, 3, 6 (32-site warps): 16 warps 28, 22, 20, 17; 256 27, 21, 19, 17; 512 27, 23, 23, 29;
+// 768 34, 27, 34, 40; 1024 33, 32, 37, 49; 1536 42, 44, 49, 68.
+template <class Run>
+inline void fx_launch(size_t sites, Run&& run) {
+  const size_t warps = (sites + 31) / 32;
+  auto go = [&](auto S) {
+    constexpr int th = FxShape<S.value>::threads, per = S.value == 1 ? th : 32;
+    run(S, (unsigned)((sites + per - 1) / per), th, fx_smem(th));
+  };
+  if (warps <= 152 * FxShape<6>::blocks)
+    go(std::integral_constant<int, 6>{});
+  else if (warps <= 152 * FxShape<3>::blocks)
+    go(std::integral_constant<int, 3>{});
+  else if (warps <= 152 * FxShape<2>::blocks)
+    go(std::integral_constant<int, 2>{});
+  else
+    go(std::integral_constant<int, 1>{});
+}
+// lets kernel k have more dynamic shared memory than a launch may by default (48 KB)
+template <class K>
+inline void fx_allow(K* k, size_t smem) {
+  if (smem > 48 * 1024) WF_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
 }
 
 // For the lanes with flag set: out = P x (dag: P^dag x) of two colour vectors, x's six components cs elements
