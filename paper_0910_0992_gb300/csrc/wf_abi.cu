@@ -2922,35 +2922,36 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
     WF_CUDA(cudaMemsetAsync(h->iflag.p, 0, sizeof(int), s));
     Cx<double>* ut[2] = {h->ut64[0].as<Cx<double>>(), h->ut64[1].as<Cx<double>>()};
     Cx<double>* us[2] = {h->us64[0].as<Cx<double>>(), h->us64[1].as<Cx<double>>()};
-    Prof P(h, "gauge_ingest", 1 + 2 * 6);
-    launch_import_gauge(g, dU, ut, us, s);
-    if (h->axial) {
-      // axial frame: ut becomes the rotation g, spatial links rotated in place, P, Lambda and the
-      // wrap matrix P Lambda (held in lamf) per line
+    if (h->axial) {  // ut becomes the rotation g, lamf the wrap matrix P Lambda
+      AxialOut o;
       for (int p = 0; p < 2; ++p) {
         h->pl64[p].ensure(nlam * sizeof(Cx<double>), s);
         h->pl32[p].ensure(nlam * sizeof(Cx<float>), s);
-        launch_axial_frame(g, ut[p], h->pl64[p].as<Cx<double>>(), h->lamb64[p].as<Cx<double>>(),
-                           h->lamf64[p].as<Cx<double>>(), h->iflag.as<int>(), s);
+        o.g[p] = ut[p];
+        o.us[p] = us[p];
+        o.pl[p] = h->pl64[p].as<Cx<double>>();
+        o.lamb[p] = h->lamb64[p].as<Cx<double>>();
+        o.wrap[p] = h->lamf64[p].as<Cx<double>>();
+        o.pl32[p] = h->pl32[p].as<Cx<float>>();
+        o.lamb32[p] = h->lamb32[p].as<Cx<float>>();
+        o.wrap32[p] = h->lamf32[p].as<Cx<float>>();
+        o.us32[p] = h->us32[p].as<Cx<float>>();
+        o.usfx[p] = h->usfx[p].as<int4>();
       }
-      const Cx<double>* gg[2] = {ut[0], ut[1]};
-      launch_rotate_links(g, us, gg, s);
-      for (int p = 0; p < 2; ++p) {
-        launch_d2f_links(us[p], h->us32[p].as<Cx<float>>(), (size_t)3 * g.Nl, g.tp, s);
-        launch_d2f(h->pl64[p].as<Cx<double>>(), h->pl32[p].as<Cx<float>>(), nlam, s);
-        launch_d2f(h->lamb64[p].as<Cx<double>>(), h->lamb32[p].as<Cx<float>>(), nlam, s);
-        launch_d2f(h->lamf64[p].as<Cx<double>>(), h->lamf32[p].as<Cx<float>>(), nlam, s);
-      }
+      Prof P(h, "gauge_ingest", 2);
+      launch_axial_frame(g, dU, o, h->iflag.as<int>(), s);
     } else {
+      Prof P(h, "gauge_ingest", 1 + 2 * 6);
+      launch_import_gauge(g, dU, ut, us, s);
       for (int p = 0; p < 2; ++p) {
         launch_tline_init(g, ut[p], h->lamb64[p].as<Cx<double>>(), h->lamf64[p].as<Cx<double>>(), h->iflag.as<int>(), s);
         launch_d2f(ut[p], h->ut32[p].as<Cx<float>>(), nut, s);
         launch_d2f_links(us[p], h->us32[p].as<Cx<float>>(), (size_t)3 * g.Nl, g.tp, s);
         launch_d2f(h->lamb64[p].as<Cx<double>>(), h->lamb32[p].as<Cx<float>>(), nlam, s);
         launch_d2f(h->lamf64[p].as<Cx<double>>(), h->lamf32[p].as<Cx<float>>(), nlam, s);
+        launch_links_fx(us[p], h->usfx[p].as<int4>(), nus, s);
       }
     }
-    for (int p = 0; p < 2; ++p) launch_links_fx(us[p], h->usfx[p].as<int4>(), nus, s);
     int flag = 0;
     WF_CUDA(cudaMemcpyAsync(&flag, h->iflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     WF_CUDA(cudaStreamSynchronize(s));

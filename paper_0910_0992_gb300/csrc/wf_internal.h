@@ -142,9 +142,15 @@ void launch_import_gauge(const Geom& g, const Cx<double>* lex, Cx<double>* ut[2]
                          cudaStream_t s);
 void launch_tline_init(const Geom& g, const Cx<double>* ut, Cx<double>* lamb, Cx<double>* lamf, int* singular,
                        cudaStream_t s);
-void launch_axial_frame(const Geom& g, Cx<double>* ut_to_g, Cx<double>* pl, Cx<double>* lamb, Cx<double>* wrap,
-                        int* singular, cudaStream_t s);
-void launch_rotate_links(const Geom& g, Cx<double>* us[2], const Cx<double>* gg[2], cudaStream_t s);
+// the axial frame from the lexicographic links, per parity: the rotation g [Nl][9][tp], P, Lambda and
+// the wrap matrix P Lambda [Nl][9] in FP64 and FP32, the rotated spatial links [3][Nl][9][tp] in FP64 and
+// fixed point and [3][Nl][6][tp] in FP32
+struct AxialOut {
+  Cx<double>*g[2], *pl[2], *lamb[2], *wrap[2], *us[2];
+  Cx<float>*pl32[2], *lamb32[2], *wrap32[2], *us32[2];
+  int4* usfx[2];
+};
+void launch_axial_frame(const Geom& g, const Cx<double>* lex, const AxialOut& o, int* singular, cudaStream_t s);
 // flag |= 1 if a link of the lexicographic field U ([nlinks][3][3]) is not finite, |= 2 if one is
 // not SU(3) within tol (entries of U^dag U - 1 and det U - 1)
 void launch_check_links(const Cx<double>* U, size_t nlinks, double tol, int* flag, cudaStream_t s);

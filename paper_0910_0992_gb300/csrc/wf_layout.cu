@@ -593,52 +593,104 @@ __global__ void k_tline_init(const Geom g, const Cx<double>* __restrict__ ut, Cx
 
 // Axial (temporal) frame (§II.C; App. C): per line, g(t) = U_t(0) U_t(1) ... U_t(t-1), g(0) = 1,
 // so that U_t'(t) = g(t) U_t(t) g(t+1)^dag = 1 for t < N_t - 1 and U_t'(N_t - 1) = g(N_t - 1) U_t(N_t - 1)
-// = P, the Polyakov product. Written in place of U_t (ut becomes g); P,
-// Lambda = (1 - s mu^-N_t P)^-1 and the wrap matrix K = P Lambda per line. Lambda is a function
-// of P, so K = Lambda P as well and K^dag = Lambda^dag P^dag closes T^-dag.
-__global__ void k_axial_frame(const Geom g, Cx<double>* ut_to_g, Cx<double>* pl, Cx<double>* lamb, Cx<double>* wrap,
-                              int* singular) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= g.Nl) return;
-  Cx<double>* line = ut_to_g + (size_t)l * 9 * g.tp;
-  Mat3<double> run = ident<double>();
-  for (int t = 0; t < g.T; ++t) {
-    const int sl = slot_of(g, t);
-    const Mat3<double> u = ldmat_d(line, g.tp, sl);
-    for (int k = 0; k < 9; ++k) line[k * g.tp + sl] = run.e[k];
-    run = matmul(run, u);
+// = P, the Polyakov product; P, Lambda = (1 - s mu^-N_t P)^-1 and the wrap matrix K = P Lambda per
+// line, in FP64 and FP32. Lambda is a function of P, so K = Lambda P as well and K^dag = Lambda^dag P^dag
+// closes T^-dag. A line's lanes multiply their n sites and scan the products (one thread per
+// line took a chain of N_t loads and products, and the links six passes: with them a load of 8^3 x 32 took
+// 453 us instead of 135, of 24^3 x 128 8.2 ms instead of 6.1).
+__global__ void __launch_bounds__(32) k_axial_frame(const Geom g, const Cx<double>* __restrict__ lex, const AxialOut o,
+                                                    int* singular) {
+  const int p = blockIdx.y, lane = threadIdx.x, jj = lane % g.lpl, n = g.n, T = g.T;
+  const int l_raw = blockIdx.x * g.lpw + lane / g.lpl;
+  const bool in = l_raw < g.Nl;
+  const int l = in ? l_raw : 0;  // idle lanes still join the shuffles
+  int x, y, z;
+  line_coords(g, p, l, x, y, z);
+  const size_t V3 = (size_t)g.L * g.L * g.L;
+  const Cx<double>* u0 = lex + (((size_t)x + g.L * ((size_t)y + (size_t)g.L * z)) * 4 + 3) * 9;
+  auto link = [&](int t) {
+    Mat3<double> U;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) U.e[k] = u0[t * V3 * 36 + k];
+    return U;
+  };
+  Mat3<double> c = ident<double>();
+  for (int m = 0; m < n; ++m)
+    if (jj * n + m < T) c = matmul(c, link(jj * n + m));
+  for (int dd = 1; dd < g.lpl; dd <<= 1) {
+    Mat3<double> q;
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+      q.e[k] = mk<double>(shfl_up_r(c.e[k].re, dd, g.lpl), shfl_up_r(c.e[k].im, dd, g.lpl));
+    if (jj >= dd) c = matmul(q, c);
   }
-  const double f = g.bc * pow(g.mu, -(double)g.T);
+  Mat3<double> run;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    run.e[k] = mk<double>(shfl_up_r(c.e[k].re, 1, g.lpl), shfl_up_r(c.e[k].im, 1, g.lpl));
+    if (jj == 0) run.e[k] = mk<double>(k % 4 == 0 ? 1.0 : 0.0, 0.0);
+  }
+  if (!in) return;
+  Cx<double>* line = o.g[p] + (size_t)l * 9 * g.tp;
+  for (int m = 0; m < n; ++m) {
+    if (jj * n + m >= T) break;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) line[k * g.tp + m * g.lpl + jj] = run.e[k];
+    if (m + 1 < n && jj * n + m + 1 < T) run = matmul(run, link(jj * n + m));
+  }
+  if (jj != g.lpl - 1) return;  // the last lane has the product of the line
+  const double f = g.bc * pow(g.mu, -(double)T);
   Mat3<double> A, Ai;
+#pragma unroll
   for (int k = 0; k < 9; ++k) {
     const double id = (k % 4 == 0) ? 1.0 : 0.0;
-    A.e[k] = mk<double>(id - f * run.e[k].re, -f * run.e[k].im);
+    A.e[k] = mk<double>(id - f * c.e[k].re, -f * c.e[k].im);
   }
-  const double d = inv3(A, Ai);
-  if (!(d > 1e-12)) atomicExch(singular, 1);
-  const Mat3<double> K = matmul(run, Ai);
+  const double det = inv3(A, Ai);
+  if (!(det > 1e-12)) atomicExch(singular, 1);
+  const Mat3<double> K = matmul(c, Ai);
+#pragma unroll
   for (int k = 0; k < 9; ++k) {
-    pl[(size_t)l * 9 + k] = run.e[k];
-    lamb[(size_t)l * 9 + k] = Ai.e[k];
-    wrap[(size_t)l * 9 + k] = K.e[k];
+    const size_t at = (size_t)l * 9 + k;
+    o.pl[p][at] = c.e[k];
+    o.lamb[p][at] = Ai.e[k];
+    o.wrap[p][at] = K.e[k];
+    o.pl32[p][at] = mk<float>((float)c.e[k].re, (float)c.e[k].im);
+    o.lamb32[p][at] = mk<float>((float)Ai.e[k].re, (float)Ai.e[k].im);
+    o.wrap32[p][at] = mk<float>((float)K.e[k].re, (float)K.e[k].im);
   }
 }
 
-// spatial links into the axial frame, in place: U_k'(x) = g(x) U_k(x) g(x + k)^dag
-__global__ void k_rotate_links(const Geom g, int p, Cx<double>* us_p, const Cx<double>* g_p, const Cx<double>* g_q) {
-  const size_t total = (size_t)3 * g.Nl * g.T;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int t = (int)(i % g.T);
-    const int l = (int)((i / g.T) % g.Nl);
-    const int k = (int)(i / ((size_t)g.T * g.Nl));
-    int nb[6];
-    neighbour_lines(g, p, l, nb);
-    const int sl = slot_of(g, t);
-    Cx<double>* U = us_p + ((size_t)k * g.Nl + l) * 9 * g.tp;
-    const Mat3<double> gx = ldmat_d(g_p + (size_t)l * 9 * g.tp, g.tp, sl);
-    const Mat3<double> gy = ldmat_d(g_q + (size_t)nb[2 * k] * 9 * g.tp, g.tp, sl);
-    const Mat3<double> r = matmul(matmul(gx, ldmat_d(U, g.tp, sl)), dagger(gy));
-    for (int e = 0; e < 9; ++e) U[e * g.tp + sl] = r.e[e];
+// Spatial links in the axial frame, U_k'(x) = g(x) U_k(x) g(x + k)^dag, from the lexicographic field into the
+// three stored forms (FP64, FP32 rows 0 and 1, fixed point): one thread per link and slot, so that the stores
+// are contiguous; padding slots zero
+__global__ void __launch_bounds__(128) k_axial_links(const Geom g, const Cx<double>* __restrict__ lex, const AxialOut o) {
+  const int p = blockIdx.y;
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i >= (size_t)3 * g.Nl * g.tp) return;
+  const int sl = (int)(i % g.tp), l = (int)((i / g.tp) % g.Nl), k = (int)(i / g.tp / g.Nl);
+  const int t = (sl % g.lpl) * g.n + sl / g.lpl;
+  int x, y, z;
+  line_coords(g, p, l, x, y, z);
+  Mat3<double> r;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) r.e[e] = czero<double>();
+  if (t < g.T) {
+    const Cx<double>* u = lex + (((size_t)x + g.L * ((size_t)y + g.L * ((size_t)z + (size_t)g.L * t))) * 4 + k) * 9;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) r.e[e] = u[e];
+    const int ln = line_of(g, k == 0 ? (x + 1) % g.L : x, k == 1 ? (y + 1) % g.L : y, k == 2 ? (z + 1) % g.L : z);
+    r = matmul(ldmat_d(o.g[p] + (size_t)l * 9 * g.tp, g.tp, sl), r);
+    r = matmul(r, dagger(ldmat_d(o.g[1 - p] + (size_t)ln * 9 * g.tp, g.tp, sl)));
+  }
+  const size_t lk = (size_t)k * g.Nl + l;
+  constexpr int NC = SpatialLinkNC<float>::value;
+#pragma unroll
+  for (int e = 0; e < 9; ++e) {
+    o.us[p][(lk * 9 + e) * g.tp + sl] = r.e[e];
+    const int2 re = link_limbs(r.e[e].re), im = link_limbs(r.e[e].im);
+    o.usfx[p][(lk * 9 + e) * g.tp + sl] = make_int4(re.x, re.y, im.x, im.y);
+    if (e < NC) o.us32[p][(lk * NC + e) * g.tp + sl] = mk<float>((float)r.e[e].re, (float)r.e[e].im);
   }
 }
 
@@ -776,15 +828,11 @@ void launch_tline_init(const Geom& g, const Cx<double>* ut, Cx<double>* lamb, Cx
   WF_CUDA(cudaGetLastError());
 }
 
-void launch_axial_frame(const Geom& g, Cx<double>* ut_to_g, Cx<double>* pl, Cx<double>* lamb, Cx<double>* wrap,
-                        int* singular, cudaStream_t s) {
-  k_axial_frame<<<(g.Nl + 127) / 128, 128, 0, s>>>(g, ut_to_g, pl, lamb, wrap, singular);
+void launch_axial_frame(const Geom& g, const Cx<double>* lex, const AxialOut& o, int* singular, cudaStream_t s) {
+  k_axial_frame<<<dim3((g.Nl + g.lpw - 1) / g.lpw, 2), 32, 0, s>>>(g, lex, o, singular);
   WF_CUDA(cudaGetLastError());
-}
-
-void launch_rotate_links(const Geom& g, Cx<double>* us[2], const Cx<double>* gg[2], cudaStream_t s) {
-  size_t n = (size_t)3 * g.Nl * g.T;
-  for (int p = 0; p < 2; ++p) k_rotate_links<<<grid_for(n), kThreads, 0, s>>>(g, p, us[p], gg[p], gg[1 - p]);
+  const size_t n = (size_t)3 * g.Nl * g.tp;
+  k_axial_links<<<dim3((unsigned)((n + 127) / 128), 2), 128, 0, s>>>(g, lex, o);
   WF_CUDA(cudaGetLastError());
 }
 
