@@ -2619,8 +2619,9 @@ int force_abi(wf_handle* h, const double* phi_odd, double* F, int precision, dou
   hop(1, w4, w5, true);
   line(1, w5, w6, OP_BWD, OP_COPY);
   Gauge<double> G = gauge_of<double>(h);
+  ForceArgs fa[2];
   for (int p = 0; p < 2; ++p) {
-    ForceArgs a;
+    ForceArgs& a = fa[p];
     std::memset(&a, 0, sizeof(a));
     a.g = g;
     a.parity = p;
@@ -2639,8 +2640,10 @@ int force_abi(wf_handle* h, const double* phi_odd, double* F, int precision, dou
     a.coef = 2.0 / (g.gamma_f * g.gamma_f);
     a.bc = g.bc;
     a.F = dF;
-    Prof P(h, "force_outer_products_f64", 2);
-    launch_force(a, s);
+  }
+  {
+    Prof P(h, "force_outer_products_f64");
+    launch_force(fa, s);
   }
   if (staged) WF_CUDA(cudaMemcpyAsync(F, dF, V * 32 * sizeof(double), cudaMemcpyDeviceToHost, s));
   WF_CUDA(cudaStreamSynchronize(s));

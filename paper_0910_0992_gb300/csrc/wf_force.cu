@@ -24,14 +24,11 @@ __device__ __forceinline__ Vec3<double> fvec(const Cx<double>* f, size_t line_ba
 }
 
 // acc += x y^dag
-__device__ __forceinline__ void outer_acc(Mat3<double>& Z, const Vec3<double>& x, const Vec3<double>& y, double s) {
+__device__ __forceinline__ void outer_acc(Mat3<double>& Z, const Vec3<double>& x, const Vec3<double>& y) {
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      Cx<double> p = cfmaconj(czero<double>(), y.c[j], x.c[i]);  // x_i conj(y_j)
-      Z.e[3 * i + j] = Z.e[3 * i + j] + s * p;
-    }
+    for (int j = 0; j < 3; ++j) Z.e[3 * i + j] = cfmaconj(Z.e[3 * i + j], y.c[j], x.c[i]);  // x_i conj(y_j)
 }
 
 // F^a = coef Re Tr[i T_a Z] = -coef Im Tr[T_a Z], T_a = lambda_a / 2 (Gell-Mann)
@@ -68,15 +65,9 @@ __device__ __forceinline__ size_t lex_site(const Geom& g, int x, int y, int z, i
   return (size_t)x + g.L * ((size_t)y + g.L * ((size_t)z + (size_t)g.L * t));
 }
 
-__global__ void k_force_temporal(const ForceArgs A) {
+__device__ __forceinline__ Mat3<double> force_temporal(const ForceArgs& A, int l, int t, int sl) {
   const Geom& g = A.g;
-  const size_t total = (size_t)g.Nl * g.T;
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  const int t = (int)(i % g.T);
-  const int l = (int)(i / g.T);
   const int tp = g.tp;
-  const int sl = slot_of(g, t);
   const int tn = t == g.T - 1 ? 0 : t + 1;
   const int sln = slot_of(g, tn);
   const double sg = t == g.T - 1 ? A.bc : 1.0;
@@ -91,85 +82,81 @@ __global__ void k_force_temporal(const ForceArgs A) {
   } else {
     U = ldmat(A.ut + (size_t)l * 9 * tp, tp, sl);
   }
-  Mat3<double> Z;
+  Mat3<double> Zl, Zr;
 #pragma unroll
-  for (int k = 0; k < 9; ++k) Z.e[k] = czero<double>();
-  // C_L factor: spins 2, 3 (P_-)
-#pragma unroll
-  for (int s = 2; s < 4; ++s) {
-    Vec3<double> bn = fvec(A.b, lb, 3 * s, tp, sln);
-    Vec3<double> ub = unit ? bn : matvec(U, bn);
-    outer_acc(Z, ub, fvec(A.a, lb, 3 * s, tp, sl), sg);
-  }
-  // C_R factor: spins 0, 1 (P_+)
+  for (int k = 0; k < 9; ++k) Zl.e[k] = Zr.e[k] = czero<double>();
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
-    Vec3<double> cn = fvec(A.c, lb, 3 * s, tp, sln);
-    Vec3<double> uc = unit ? cn : matvec(U, cn);
-    outer_acc(Z, fvec(A.e, lb, 3 * s, tp, sl), uc, -sg);
+    // C_L factor: spins 2, 3 (P_-)
+    const Vec3<double> bn = fvec(A.b, lb, 6 + 3 * s, tp, sln);
+    outer_acc(Zl, unit ? bn : matvec(U, bn), fvec(A.a, lb, 6 + 3 * s, tp, sl));
+    // C_R factor: spins 0, 1 (P_+)
+    const Vec3<double> cn = fvec(A.c, lb, 3 * s, tp, sln);
+    outer_acc(Zr, fvec(A.e, lb, 3 * s, tp, sl), unit ? cn : matvec(U, cn));
   }
-  Z = to_caller_gauge(Z, A, l, sl);
-  int x, y, z;
-  line_coords(g, A.parity, l, x, y, z);
-  project(Z, A.coef, A.F + (lex_site(g, x, y, z, t) * 4 + 3) * 8);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Zl.e[k] = sg * (Zl.e[k] - Zr.e[k]);
+  return Zl;
 }
 
-__global__ void k_force_spatial(const ForceArgs A) {
+// upper components of u +- i sigma_k d (sg = 1, -1), the rest of (1 -+ gamma_k) psi following from them
+__device__ __forceinline__ void half_of(const Cx<double>* f, size_t lb, int tp, int sl, int k, double sg, Vec3<double> (&h)[2]) {
+  isigma(k, fvec(f, lb, 6, tp, sl), fvec(f, lb, 9, tp, sl), h[0], h[1]);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) h[s] = vaxpy(sg, h[s], fvec(f, lb, 3 * s, tp, sl));
+}
+
+// sum_spins x (P y)^dag = 1/2 sum_{two spins} h_x h_y^dag for a projector P = (1 -+ gamma_k) / 2 (the lower
+// spins are a unitary matrix times the upper ones)
+__device__ __forceinline__ Mat3<double> force_spatial(const ForceArgs& A, int l, int sl, int k) {
   const Geom& g = A.g;
-  const size_t total = (size_t)g.Nl * g.T;
-  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  const int t = (int)(i % g.T);
-  const int l = (int)(i / g.T);
   const int tp = g.tp;
-  const int sl = slot_of(g, t);
   int nb[6];
   neighbour_lines(g, A.parity, l, nb);
-  int x, y, z;
-  line_coords(g, A.parity, l, x, y, z);
-  const size_t lb = (size_t)l * NSPIN_C * tp;
-  for (int k = 0; k < 3; ++k) {
-    const size_t nbb = (size_t)nb[2 * k] * NSPIN_C * tp;
-    const Mat3<double> U = ldmat(A.us_p + ((size_t)k * g.Nl + l) * NLINK_C * tp, tp, sl);
-    // spinors: w(x), v(x+k), vr(x), wr(x+k)
-    Vec3<double> w[4], v[4], vr[4], wr[4];
+  const size_t lb = (size_t)l * NSPIN_C * tp, nbb = (size_t)nb[2 * k] * NSPIN_C * tp;
+  const Mat3<double> U = ldmat(A.us_p + ((size_t)k * g.Nl + l) * NLINK_C * tp, tp, sl);
+  Mat3<double> Z, Zr;
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      w[s] = fvec(A.w, lb, 3 * s, tp, sl);
-      v[s] = fvec(A.v, nbb, 3 * s, tp, sl);
-      vr[s] = fvec(A.vr, lb, 3 * s, tp, sl);
-      wr[s] = fvec(A.wr, nbb, 3 * s, tp, sl);
-    }
-    // P^-_k w = ((h), -i sigma_k h) / 2 with h = w_up + i sigma_k w_lo; P^+_k wr = ((h'), i sigma_k h') / 2
-    Vec3<double> s0, s1, h0, h1, r0, r1;
-    isigma(k, w[2], w[3], s0, s1);
-    h0 = vscale(0.5, vadd(w[0], s0));
-    h1 = vscale(0.5, vadd(w[1], s1));
-    isigma(k, h0, h1, r0, r1);
-    Vec3<double> pm[4] = {h0, h1, vscale(-1.0, r0), vscale(-1.0, r1)};
-    isigma(k, wr[2], wr[3], s0, s1);
-    h0 = vscale(0.5, vaxpy(-1.0, s0, wr[0]));
-    h1 = vscale(0.5, vaxpy(-1.0, s1, wr[1]));
-    isigma(k, h0, h1, r0, r1);
-    Vec3<double> pp[4] = {h0, h1, r0, r1};
-    Mat3<double> Z;
+  for (int e = 0; e < 9; ++e) Z.e[e] = Zr.e[e] = czero<double>();
+  Vec3<double> x[2], y[2];
+  half_of(A.v, nbb, tp, sl, k, 1.0, x);
+  half_of(A.w, lb, tp, sl, k, 1.0, y);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) Z.e[e] = czero<double>();
+  for (int s = 0; s < 2; ++s) outer_acc(Z, matvec(U, x[s]), y[s]);
+  half_of(A.vr, lb, tp, sl, k, -1.0, x);
+  half_of(A.wr, nbb, tp, sl, k, -1.0, y);
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      outer_acc(Z, matvec(U, v[s]), pm[s], 1.0);
-      outer_acc(Z, vr[s], matvec(U, pp[s]), -1.0);
-    }
-    Z = to_caller_gauge(Z, A, l, sl);
-    project(Z, A.coef, A.F + (lex_site(g, x, y, z, t) * 4 + k) * 8);
-  }
+  for (int s = 0; s < 2; ++s) outer_acc(Zr, x[s], matvec(U, y[s]));
+#pragma unroll
+  for (int e = 0; e < 9; ++e) Z.e[e] = 0.5 * (Z.e[e] - Zr.e[e]);
+  return Z;
 }
 
-void launch_force(const ForceArgs& a, cudaStream_t s) {
-  const size_t total = (size_t)a.g.Nl * a.g.T;
-  const int blocks = (int)((total + 127) / 128);
-  k_force_temporal<<<blocks, 128, 0, s>>>(a);
-  k_force_spatial<<<blocks, 128, 0, s>>>(a);
+struct ForcePair {
+  ForceArgs p[2];
+};
+// One thread per link: blockIdx.y its direction (3: temporal), blockIdx.z its base site's parity. Bound by
+// latency and the FP64 pipe (8^3 x 32: 88 us; one thread per site and parity, with all four spins of the
+// projected spinors, took 274 for the two parities)
+__global__ void __launch_bounds__(64) k_force(const ForcePair F) {
+  const ForceArgs& A = F.p[blockIdx.z];
+  const Geom& g = A.g;
+  const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (i >= (size_t)g.Nl * g.T) return;
+  const int t = (int)(i % g.T), l = (int)(i / g.T), mu = blockIdx.y;
+  const int sl = slot_of(g, t);
+  const Mat3<double> Z = to_caller_gauge(mu == 3 ? force_temporal(A, l, t, sl) : force_spatial(A, l, sl, mu), A, l, sl);
+  int x, y, z;
+  line_coords(g, A.parity, l, x, y, z);
+  project(Z, A.coef, A.F + (lex_site(g, x, y, z, t) * 4 + mu) * 8);
+}
+
+void launch_force(const ForceArgs (&a)[2], cudaStream_t s) {
+  ForcePair f;
+  f.p[0] = a[0];
+  f.p[1] = a[1];
+  const unsigned blocks = (unsigned)(((size_t)a[0].g.Nl * a[0].g.T + 63) / 64);
+  k_force<<<dim3(blocks, 4, 2), 64, 0, s>>>(f);
   WF_CUDA(cudaGetLastError());
 }
 

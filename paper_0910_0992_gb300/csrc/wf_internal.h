@@ -270,7 +270,8 @@ struct ForceArgs {
   double bc;
   double* F;                 // [V][4][8], caller's gauge
 };
-void launch_force(const ForceArgs& a, cudaStream_t s);
+// both parities
+void launch_force(const ForceArgs (&a)[2], cudaStream_t s);
 
 // Clover term (wf_clover.cu): build H_a, H_b (half the chiral blocks of A, [Nl][2][36][tp] per
 // parity) from the lexicographic FP64 links, rotated by rot[p] (the axial-frame rotation, or
