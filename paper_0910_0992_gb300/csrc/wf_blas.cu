@@ -157,6 +157,7 @@ template <typename R>
 __global__ void __launch_bounds__(kBT) k_cg_r_check(Cx<R>* __restrict__ r, const Cx<R>* __restrict__ q, size_t n,
                                                     const double* gamma, const double* qq, double* partial, double* rr,
                                                     const size_t* offs, const CgState c) {
+  grid_dep();
   const int rhs = blockIdx.y;
   const bool on = c.active[rhs] != 0;
   const double qn = qq[rhs];
@@ -195,7 +196,7 @@ __global__ void __launch_bounds__(kBT) k_cg_r_check(Cx<R>* __restrict__ r, const
 template <typename R>
 void launch_cg_r_check(Cx<R>* r, const Cx<R>* q, size_t n, int nrhs, const double* gamma, const double* qq,
                        double* partial, double* rr, const CgState& c, cudaStream_t s, const size_t* offs) {
-  k_cg_r_check<R><<<dim3(parts_for(n), nrhs), kBT, 0, s>>>(r, q, n, gamma, qq, partial, rr, offs, c);
+  launch_dep(k_cg_r_check<R>, dim3(parts_for(n), nrhs), kBT, 0, s, r, q, n, gamma, qq, partial, rr, offs, c);
   WF_CUDA(cudaGetLastError());
 }
 template void launch_cg_r_check<float>(Cx<float>*, const Cx<float>*, size_t, int, const double*, const double*, double*,
@@ -214,6 +215,7 @@ __global__ void __launch_bounds__(kBT) k_cg_p(Cx<R>* __restrict__ p, const Cx<R>
                                                const double* gnew, const double* gold, const int* active,
                                                const size_t* offs, Cx<R>* __restrict__ x, const double* qq,
                                                const int* upd, const CgAdvance adv) {
+  grid_dep();
   const int rhs = blockIdx.y;
   const bool on = active[rhs] != 0;
   const bool dox = x && upd[rhs];
@@ -252,7 +254,7 @@ void launch_cg_p(Cx<R>* p, const Cx<R>* sv, size_t n, int nrhs, const double* gn
                  const int* active, cudaStream_t s, const size_t* offs, Cx<R>* x, const double* qq, const int* upd,
                  const CgAdvance& adv) {
   const int parts = parts_for(n) * 2;
-  k_cg_p<R><<<dim3(parts, nrhs), kBT, 0, s>>>(p, sv, n, gnew, gold, active, offs, x, qq, upd, adv);
+  launch_dep(k_cg_p<R>, dim3(parts, nrhs), kBT, 0, s, p, sv, n, gnew, gold, active, offs, x, qq, upd, adv);
   WF_CUDA(cudaGetLastError());
 }
 template void launch_cg_p<float>(Cx<float>*, const Cx<float>*, size_t, int, const double*, const double*,

@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(kBlock) k_clover_apply(const Geom g, const Cx<
 // solve 19.3 -> 18.9 ms, its first pass 22.0 -> 20.9 ms
 template <bool AX, bool ODD>
 __global__ void __launch_bounds__(32, 8) k_abar(const AbarArgs B) {
+  grid_dep();
   using R = float;
   const LineArgs<R>& A = B.line;
   const Geom& g = A.g;
@@ -504,9 +505,9 @@ void launch_abar(const AbarArgs& a, bool axial, bool odd, cudaStream_t s) {
   if (g.n < 1 || g.n > NMAX) throw Error(WF_EINVAL, "Abar kernel: unsupported sites per lane");
   const unsigned blocks = (unsigned)((g.Nl + g.lpw - 1) / g.lpw);
   if (axial)
-    odd ? k_abar<true, true><<<blocks, 32, 0, s>>>(a) : k_abar<true, false><<<blocks, 32, 0, s>>>(a);
+    launch_dep(odd ? k_abar<true, true> : k_abar<true, false>, blocks, 32, 0, s, a);
   else
-    odd ? k_abar<false, true><<<blocks, 32, 0, s>>>(a) : k_abar<false, false><<<blocks, 32, 0, s>>>(a);
+    launch_dep(odd ? k_abar<false, true> : k_abar<false, false>, blocks, 32, 0, s, a);
   WF_CUDA(cudaGetLastError());
 }
 

@@ -233,6 +233,10 @@ __host__ __device__ __forceinline__ void neighbour_lines(const Geom& g, int p, i
   nb[5] = line_of(g, x, y, (z + L - 1) % L);
 }
 
+// Start of a kernel launched by launch_dep (wf_internal.h): waits until the kernel before it in the stream has
+// completed. Precedes every access to memory.
+__device__ __forceinline__ void grid_dep() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Spinor component index: spin * 3 + colour. Dirac-Pauli basis: spins 0, 1 are the
 // P_+ = (1 + gamma_t)/2 ("upper") half, spins 2, 3 the P_- ("lower") half.
 constexpr int NSPIN_C = 12;

@@ -49,6 +49,7 @@ __device__ __forceinline__ void eo_add_norm(double* norm2, int rhs, size_t sline
 
 template <typename R, bool AX>
 __global__ void __launch_bounds__(kEoThreads, WF_EO_MINB) k_dslash4(const EoArgs<R> A) {
+  grid_dep();
   const Geom& g = A.g;
   const int Th = g.T / 2;
   const int L = g.L;
@@ -211,6 +212,7 @@ struct EoDir {
 // k_dslash4. 16^3 x 96, 4 sources: 1.16 ms with every operation in FP64, 0.42 ms so.
 template <bool AX, int S>
 __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_dslash4_fx(const EoArgs<double> A) {
+  grid_dep();
   const Geom& g = A.g;
   const int Th = g.T / 2, L = g.L;
   const size_t V3 = (size_t)L * L * L;
@@ -288,9 +290,9 @@ static void launch_dslash4_impl(const EoArgs<R>& a, bool axial, cudaStream_t s) 
   const size_t total = (size_t)a.nrhs * a.g.L * a.g.L * a.g.L * (a.g.T / 2);
   const int blocks = (int)((total + kEoThreads - 1) / kEoThreads);
   if (axial)
-    k_dslash4<R, true><<<blocks, kEoThreads, 0, s>>>(a);
+    launch_dep(k_dslash4<R, true>, blocks, kEoThreads, 0, s, a);
   else
-    k_dslash4<R, false><<<blocks, kEoThreads, 0, s>>>(a);
+    launch_dep(k_dslash4<R, false>, blocks, kEoThreads, 0, s, a);
   WF_CUDA(cudaGetLastError());
 }
 
@@ -338,7 +340,7 @@ void launch_dslash4(const EoArgs<R>& a, bool axial, cudaStream_t s) {
     fx_launch(total, [&](auto S, unsigned b, int th, size_t smem) {
       auto* k = axial ? k_dslash4_fx<true, S.value> : k_dslash4_fx<false, S.value>;
       fx_allow(k, smem);
-      k<<<b, th, smem, s>>>(a);
+      launch_dep(k, b, th, smem, s, a);
     });
     WF_CUDA(cudaGetLastError());
   } else {

@@ -56,6 +56,7 @@ __device__ __forceinline__ bool site_at(const Geom& g, size_t i, int nrhs, int& 
 template <int S>
 __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks)
     k_hop_fx(const LineArgs<double> A, int post) {
+  grid_dep();
   const Geom& g = A.g;
   int rhs, l, sl, t;
   bool in = site_at(g, fx_site<S>(), A.nrhs, rhs, l, sl, t);
@@ -91,6 +92,7 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks)
 // The Wilson matrix on the output parity (k_apply_M of wf_line_kernels.cuh), one thread per site
 template <bool AX, int S>
 __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_apply_M_fx(const MArgs<double> A) {
+  grid_dep();
   const Geom& g = A.g;
   int rhs, l, sl, t;
   const bool in = site_at(g, fx_site<S>(), A.nrhs, rhs, l, sl, t);
@@ -156,7 +158,7 @@ void launch_hop_fx(const LineArgs<double>& a, bool post, cudaStream_t s) {
   if (!a.fx_out || !a.fx_nbr) throw Error(1, "FP64 hop: no fixed-point links");
   fx_launch((size_t)a.nrhs * a.g.Nl * a.g.tp, [&](auto S, unsigned b, int th, size_t smem) {
     fx_allow(k_hop_fx<S.value>, smem);
-    k_hop_fx<S.value><<<b, th, smem, s>>>(a, post ? 1 : 0);
+    launch_dep(k_hop_fx<S.value>, b, th, smem, s, a, post ? 1 : 0);
   });
   WF_CUDA(cudaGetLastError());
 }
@@ -166,7 +168,7 @@ void launch_apply_M_fx(const MArgs<double>& a, bool axial, cudaStream_t s) {
   fx_launch((size_t)a.nrhs * a.g.Nl * a.g.tp, [&](auto S, unsigned b, int th, size_t smem) {
     auto* k = axial ? k_apply_M_fx<true, S.value> : k_apply_M_fx<false, S.value>;
     fx_allow(k, smem);
-    k<<<b, th, smem, s>>>(a);
+    launch_dep(k, b, th, smem, s, a);
   });
   WF_CUDA(cudaGetLastError());
 }

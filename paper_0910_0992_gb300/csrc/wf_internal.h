@@ -1,6 +1,7 @@
 // Host-side internals of libwf: the handle, device buffers and kernel launchers.
 #pragma once
 
+#include <utility>
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -63,6 +64,27 @@ template <typename R> struct LineArgs;
 // which compiled variant of the line kernel to launch: the three Schur-operator kernels
 // have their source and solve ops fixed at compile time, as has the plain hop (copy on both
 // halves); LK_GENERIC reads them from the arguments
+// kernel<<<grid, block, smem, s>>>(args...) whose launch may overlap the end of the kernel before it in the
+// stream; the kernel starts with grid_dep (wf_common.cuh) and reads nothing through the read-only path before
+// it has branched. Schur apply FP64 4^3 x 16 100 -> 85 us, FP32 16^3 x 128 217 -> 207; in graphs: FP64 solve
+// 8^3 x 32, two sources, 5.00 -> 4.88 ms, force and action 8^3 x 32 3.01 -> 2.88 ms. Triggering the next launch at a
+// kernel's start loses that (5.71, 3.47 ms): its waiting CTAs are resident on the SMs that were free first,
+// and share them when their turn comes.
+template <class... P, class... A>
+inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = at;
+  c.numAttrs = 1;
+  WF_CUDA(cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...));
+}
+
 enum LineKind { LK_GENERIC = 0, LK_SCHUR_A = 1, LK_SCHUR_B = 2, LK_SCHUR_C = 3, LK_HOP = 4 };
 
 template <typename R>

@@ -43,7 +43,7 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
     // FP16 spinor storage (FP32 arithmetic): K-a on this kernel, the hop kernels on the wide one
     if constexpr (std::is_same<R, float>::value) {
       if (axial && kind == LK_SCHUR_A && a.g.n >= 1 && a.g.n <= NMAX) {
-        k_line<float, true, SRC_LOAD, OP_FWD, OP_SKIP, true><<<line_blocks(a), kLineThreads, 0, s>>>(a);
+        launch_dep(k_line<float, true, SRC_LOAD, OP_FWD, OP_SKIP, true>, line_blocks(a), kLineThreads, 0, s, a);
         WF_CUDA(cudaGetLastError());
         return;
       }
@@ -76,14 +76,14 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
         q.opl = OP_SKIP;
       }
       const dim3 grid(line_warps(a.g, a.nrhs), 4);
-      axial ? k_line_spin<true><<<grid, 32, 0, s>>>(q) : k_line_spin<false><<<grid, 32, 0, s>>>(q);
+      launch_dep(axial ? k_line_spin<true> : k_line_spin<false>, grid, 32, 0, s, q);
       WF_CUDA(cudaGetLastError());
       return;
     }
   }
   constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;
   constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
-#define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV><<<b, th, 0, s>>>(a)
+#define WF_KL(AXV, SRCV, OPUV, OPLV) launch_dep(k_line<R, AXV, SRCV, OPUV, OPLV>, b, th, 0, s, a)
   if (axial) {
     switch (kind) {
       case LK_SCHUR_A: WF_KL(true, SRC_LOAD, OP_FWD, OP_SKIP); break;
@@ -232,9 +232,9 @@ void launch_apply_M(const MArgs<R>& a, bool axial, cudaStream_t s) {
     return;
   }
   if (axial)
-    k_apply_M<R, true, NMAX><<<blocks, kLineThreads, 0, s>>>(a);
+    launch_dep(k_apply_M<R, true, NMAX>, blocks, kLineThreads, 0, s, a);
   else
-    k_apply_M<R, false, NMAX><<<blocks, kLineThreads, 0, s>>>(a);
+    launch_dep(k_apply_M<R, false, NMAX>, blocks, kLineThreads, 0, s, a);
   WF_CUDA(cudaGetLastError());
   }
 }

@@ -386,6 +386,7 @@ template <typename R, int SPL, bool EO>
 __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks)
     k_import_spinor(const Geom g, const SpinorTile t, int compact, int par, const Cx<double>* __restrict__ lex, Cx<R>* even,
                     Cx<R>* odd, int nrhs, int g5, const Cx<double>* g_e, const Cx<double>* g_o) {
+  grid_dep();
   __shared__ __align__(16) Cx<double> buf[kTileThreads / SPL * kTileRow];
   const TileAt at(t, compact ? 1 : 2, par, nrhs);
   Cx<R>* dst = at.p ? odd : even;
@@ -449,6 +450,7 @@ template <typename R, int SPL, bool EO>
 __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks)
     k_export_spinor(const Geom g, const SpinorTile t, int compact, int par, const Cx<R>* even, const Cx<R>* odd,
                     Cx<double>* __restrict__ lex, int nrhs, int g5, const Cx<double>* g_e, const Cx<double>* g_o) {
+  grid_dep();
   __shared__ __align__(16) Cx<double> buf[kTileThreads / SPL * kTileRow];
   const TileAt at(t, compact ? 1 : 2, par, nrhs);
   const Cx<R>* src = at.p ? odd : even;  // null: that parity's sites are zero
@@ -749,9 +751,9 @@ static void launch_import_tiles(const Geom& g, int par, const Cx<double>* in, Cx
   const int compact = par >= 0;
   const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, EO, grid, split);
   if (split)
-    k_import_spinor<R, 4, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, in, even, odd, nrhs, g5, g_e, g_o);
+    launch_dep(k_import_spinor<R, 4, EO>, grid, kTileThreads, 0, s, g, t, compact, par, in, even, odd, nrhs, g5, g_e, g_o);
   else
-    k_import_spinor<R, 1, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, in, even, odd, nrhs, g5, g_e, g_o);
+    launch_dep(k_import_spinor<R, 1, EO>, grid, kTileThreads, 0, s, g, t, compact, par, in, even, odd, nrhs, g5, g_e, g_o);
   WF_CUDA(cudaGetLastError());
 }
 template <typename R, bool EO>
@@ -762,9 +764,9 @@ static void launch_export_tiles(const Geom& g, int par, const Cx<R>* even, const
   const int compact = par >= 0;
   const SpinorTile t = tile_of(g, compact ? 1 : 2, nrhs, EO, grid, split);
   if (split)
-    k_export_spinor<R, 4, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, even, odd, out, nrhs, g5, g_e, g_o);
+    launch_dep(k_export_spinor<R, 4, EO>, grid, kTileThreads, 0, s, g, t, compact, par, even, odd, out, nrhs, g5, g_e, g_o);
   else
-    k_export_spinor<R, 1, EO><<<grid, kTileThreads, 0, s>>>(g, t, compact, par, even, odd, out, nrhs, g5, g_e, g_o);
+    launch_dep(k_export_spinor<R, 1, EO>, grid, kTileThreads, 0, s, g, t, compact, par, even, odd, out, nrhs, g5, g_e, g_o);
   WF_CUDA(cudaGetLastError());
 }
 

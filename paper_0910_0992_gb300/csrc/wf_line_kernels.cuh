@@ -192,6 +192,7 @@ __device__ __forceinline__ void line_body(const LineArgs<R>& A, int blk) {
 
 template <typename R, bool AX, int SRC, int OPU, int OPL, bool H = false, int NM = NMAX>
 __global__ void __launch_bounds__(kLineThreads, LineMinBlocks<R>::value) k_line(const LineArgs<R> A) {
+  grid_dep();
   line_body<R, AX, SRC, OPU, OPL, H, NM>(A, blockIdx.x);
 }
 
@@ -203,6 +204,7 @@ __global__ void __launch_bounds__(kLineThreads, LineMinBlocks<R>::value) k_line(
 template <bool AX>
 __global__ void __launch_bounds__(32) k_line_spin(const LineArgs<double> A) {
   using R = double;
+  grid_dep();
   const Geom& g = A.g;
   const int h = blockIdx.y >> 1, op = h ? A.opl : A.opu;
   if (op == OP_SKIP) return;
@@ -247,6 +249,7 @@ inline int line_threads(const LineArgs<R>& a) {
 // ----------------------------------------------------------------------------
 template <typename R, bool AX, int NM>
 __global__ void __launch_bounds__(kLineThreads) k_apply_M(const MArgs<R> A) {
+  grid_dep();
   const Geom& g = A.g;
   const int lane = threadIdx.x & 31;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

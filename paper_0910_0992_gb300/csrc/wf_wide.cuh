@@ -504,6 +504,7 @@ __device__ __forceinline__ void line_wide_body(const LineArgs<R>& A, int blk) {
 template <typename R, int SRC, int OPU, int OPL, int TPC, bool H = false, bool STG = false>
 __global__ void __launch_bounds__(kWideCta, STG ? 6 : WideMinBlocks<R, SRC == SRC_HOP && OPU == OP_COPY>::value)
     k_line_wide(const LineArgs<R> A) {
+  grid_dep();
 #define WF_WIDE_BLOCK ((int)blockIdx.x)
 #include "wf_wide_body.inc"
 #undef WF_WIDE_BLOCK
@@ -585,14 +586,14 @@ void launch_line_wide(const LineArgs<R>& a, int kind, cudaStream_t s) {
     if (a.h16) {                                                                                  \
       if (!kH) throw Error(1, "wide line kernel: FP16 storage only for the hop kernels");         \
       if (t128)                                                                                   \
-        wide::k_line_wide<R, SRCV, OPUV, OPLV, 128, kH><<<blocks, wide::kWideCta, 0, s>>>(a);     \
+        launch_dep(wide::k_line_wide<R, SRCV, OPUV, OPLV, 128, kH>, blocks, wide::kWideCta, 0, s, a); \
       else                                                                                        \
-        wide::k_line_wide<R, SRCV, OPUV, OPLV, 0, kH><<<blocks, wide::kWideCta, 0, s>>>(a);       \
+        launch_dep(wide::k_line_wide<R, SRCV, OPUV, OPLV, 0, kH>, blocks, wide::kWideCta, 0, s, a); \
     } else if (t128) {                                                                            \
       constexpr bool kS = kF32 && (SRCV) == SRC_HOP; /* staged */                                 \
-      wide::k_line_wide<R, SRCV, OPUV, OPLV, 128, false, kS><<<blocks, wide::kWideCta, 0, s>>>(a); \
+      launch_dep(wide::k_line_wide<R, SRCV, OPUV, OPLV, 128, false, kS>, blocks, wide::kWideCta, 0, s, a); \
     } else {                                                                                      \
-      wide::k_line_wide<R, SRCV, OPUV, OPLV, 0><<<blocks, wide::kWideCta, 0, s>>>(a);             \
+      launch_dep(wide::k_line_wide<R, SRCV, OPUV, OPLV, 0>, blocks, wide::kWideCta, 0, s, a); \
     }                                                                                             \
   } while (0)
   switch (kind) {
