@@ -339,9 +339,8 @@ void launch_hop_config(wf_handle* h, const LineArgs<float>& a0, int kind) {
 }
 
 // Autotuner of the FP32 hop kernels K-b and K-c: the first time a handle applies M-hat to a
-// given number of right-hand sides, every candidate -- the register-fed kernels (one thread per
-// site or n sites per lane) and, for 128-slot lines, the bulk-fed kernels with 1 or 2 sources per
-// unit and 2 to 4 stages, each over traversal tiles of every divisor of L from 2 to 12 rows of y --
+// given number of right-hand sides, every candidate -- one thread per site and, but for 128-slot
+// lines, n sites per lane, each over traversal tiles of every divisor of L from 2 to 12 rows of y --
 // runs K-b and K-c on the call's own buffers, once untimed and three times timed with CUDA
 // events; the fastest is kept for the handle. The timed runs write only the work fields K-b and
 // K-c own (no norms); the call then computes its result as usual. Environment WF_HOP fixes the
@@ -784,7 +783,7 @@ std::vector<int> cgnr(wf_handle* h, const OpFn<R>& A, const OpFn<double>& A64, c
     if (v > 0.0 && v < 1.0) delta = v;
   }
   // Iterations run in blocks without host synchronisation: convergence and the reliable-update
-  // trigger are decided on the device after every x, r update (k_cg_check); the host reads the
+  // trigger are decided on the device after every r update (k_cg_r_check); the host reads the
   // state once per block, performs reliable updates, and sizes the next block from the observed
   // convergence rate (IterationGraph).
   std::vector<double> tgt2(nrhs), ru2(nrhs);
