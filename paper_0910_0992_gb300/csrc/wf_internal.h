@@ -61,9 +61,6 @@ struct DevBuf {
 // ----------------------------------------------------------------------------
 template <typename R> struct LineArgs;
 
-// which compiled variant of the line kernel to launch: the three Schur-operator kernels
-// have their source and solve ops fixed at compile time, as has the plain hop (copy on both
-// halves); LK_GENERIC reads them from the arguments
 // kernel<<<grid, block, smem, s>>>(args...) whose launch may overlap the end of the kernel before it in the
 // stream; the kernel starts with grid_dep (wf_common.cuh) and reads nothing through the read-only path before
 // it has branched. Schur apply FP64 4^3 x 16 100 -> 85 us, FP32 16^3 x 128 217 -> 207; in graphs: FP64 solve
@@ -85,6 +82,9 @@ inline void launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   WF_CUDA(cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...));
 }
 
+// which compiled variant of the line kernel to launch: the three Schur-operator kernels
+// have their source and solve ops fixed at compile time, as has the plain hop (copy on both
+// halves); LK_GENERIC reads them from the arguments
 enum LineKind { LK_GENERIC = 0, LK_SCHUR_A = 1, LK_SCHUR_B = 2, LK_SCHUR_C = 3, LK_HOP = 4 };
 
 template <typename R>
