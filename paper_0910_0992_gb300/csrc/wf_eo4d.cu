@@ -236,7 +236,9 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_dsl
 
   Vec3<double> acc[4];
   const EoDir dir{A, x, y, z, p3, l, sl, h, A.in + (size_t)rhs * V3 * fstride, cu, cl};
-  const double unit = hop_fx<S>(dir, Th, tp, active, acc) * A.inv_gf;
+  double unit[4];
+  hop_fx<S>(dir, Th, tp, active, acc, unit);
+  const double af = A.a * A.inv_gf;
   if (S > 1 && threadIdx.x >= 32) return;
   // temporal hops: P_- U_t(t) psi(t+1) on spins 2-3, P_+ U_t^dag(t-1) psi(t-1) on spins 0-1
   const Cx<double>* own = A.in + ((size_t)rhs * V3 + s3) * fstride;
@@ -272,7 +274,7 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_dsl
     for (int s = 0; s < 4; ++s) {
       const int so = A.swap_out ? (s + 2) % 4 : s;
       Vec3<double> val = vscale(s < 2 ? A.a * sb : A.a * sf, s < 2 ? b[s] : f[s - 2]);
-      val = vaxpy(A.a * unit, acc[s], val);
+      val = vaxpy(af * unit[s], acc[s], val);
       if (A.x1) val = vaxpy(A.b1, ldvec_stream(A.x1 + at + so * 3 * Th, Th, 0), val);
       if (A.x2) val = vaxpy(A.b2, ldvec_stream(A.x2 + at + so * 3 * Th, Th, 0), val);
       if (A.stream_out)

@@ -64,9 +64,10 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks)
   const int tp = g.tp;
   const size_t base = ((size_t)rhs * g.Nl + l) * NSPIN_C * tp;
   Vec3<double> h[4];
+  double unit[4] = {0.0, 0.0, 0.0, 0.0};
   const bool site = in && t < g.T;
-  double unit = hop_fx<S>(
-      LineDir(g, A.parity, rhs, l, sl, A.src_up, A.src_lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site, h);
+  hop_fx<S>(LineDir(g, A.parity, rhs, l, sl, A.src_up, A.src_lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site,
+            h, unit);
   if (!in || (S > 1 && threadIdx.x >= 32)) return;
   if (!site) {
 #pragma unroll
@@ -74,17 +75,19 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks)
   }
   if (A.xpre && t < g.T) {
 #pragma unroll
-    for (int s = 0; s < 4; ++s) h[s] = vaxpy(A.apre * unit, h[s], ldvec(A.xpre + base + 3 * s * tp, tp, sl));
-    unit = 1.0;
+    for (int s = 0; s < 4; ++s) {
+      h[s] = vaxpy(A.apre * unit[s], h[s], ldvec(A.xpre + base + 3 * s * tp, tp, sl));
+      unit[s] = 1.0;
+    }
   }
 #pragma unroll
   for (int s = 0; s < 4; ++s) {
     const int so = A.swap_out ? (s + 2) % 4 : s;
     Vec3<double> v;
     if (post && A.xpost)
-      v = vaxpy(A.apost * unit, h[s], ldvec(A.xpost + base + 3 * so * tp, tp, sl));
+      v = vaxpy(A.apost * unit[s], h[s], ldvec(A.xpost + base + 3 * so * tp, tp, sl));
     else
-      v = vscale(unit, h[s]);
+      v = vscale(unit[s], h[s]);
     stvec(A.out + base + 3 * so * tp, tp, sl, v);
   }
 }
@@ -103,8 +106,8 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_app
   Vec3<double> h[4];
   const Cx<double>* up = A.psi_q + (A.swap ? 6 * tp : 0);
   const Cx<double>* lo = A.psi_q + (A.swap ? 0 : 6 * tp);
-  const double unit =
-      hop_fx<S>(LineDir(g, A.parity, rhs, l, sl, up, lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site, h);
+  double unit[4];
+  hop_fx<S>(LineDir(g, A.parity, rhs, l, sl, up, lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site, h, unit);
   if (S > 1 && threadIdx.x >= 32) return;
   // axial frame: spins 0-1 at t = 0 need P^dag psi(T - 1), spins 2-3 at t = T - 1 P psi(0)
   Vec3<double> wr[2];
@@ -132,7 +135,7 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_app
       }
       val = vscale(A.mu, ldvec(pp + 3 * sr * tp, tp, sl));
       val = vaxpy(s < 2 ? -sb : -sf, dt, val);
-      val = vaxpy(-A.inv_gf * unit, h[s], val);
+      val = vaxpy(-A.inv_gf * unit[s], h[s], val);
     }
     if (A.x) val = vaxpy(A.a, val, ldvec(A.x + base + 3 * sr * tp, tp, sl));
     stvec(A.out + base + 3 * sr * tp, tp, sl, val);

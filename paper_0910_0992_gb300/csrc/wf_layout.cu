@@ -117,8 +117,8 @@ __device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl,
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const Cx<double> e = gl[(size_t)k * tp + sl];
-    G.re[k] = fx_limbs(fx_from(e.re, 1023));  // |g| <= 1 + 1e-9: exponents up to 1023
-    G.im[k] = fx_limbs(fx_from(e.im, 1023));
+    G.re[k] = fx_limbs(fx_from<3>(e.re, 1023));  // |g| <= 1 + 1e-9: exponents up to 1023
+    G.im[k] = fx_limbs(fx_from<3>(e.im, 1023));
   }
 }
 // w = g v (DAG: g^dag v), the six numbers of v sharing one exponent; false (w unset) outside the
@@ -134,7 +134,7 @@ __device__ __forceinline__ bool rotate3_fx(const FxMat& G, const double (&v)[6],
   int2 h[6], n[6];  // limbs of v and of -v
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    h[i] = fx_limbs(fx_from(v[i], E));
+    h[i] = fx_limbs(fx_from<3>(v[i], E));
     n[i] = make_int2(-h[i].x, -h[i].y);
   }
 #pragma unroll
