@@ -6,32 +6,32 @@
 // us). The direction d of a site's stencil is a half-spinor of 12 real numbers times one SU(3) link, and
 //   * a direction makes two result spins of each pair of the neighbour's spins (axes x, y: 0 and 3 of
 //     spins 0 and 3, 1 and 2 of 1 and 2; z: 0 and 2, 1 and 3). Every result spin r has an exponent E_r,
-//     the largest of the numbers that made it so far; a pair is taken as v = x 2^(56 - F), F the smaller
-//     exponent of its two results, |v| < 2^57: an exact shift of the 53-bit mantissa but for bits below
-//     2^(F - 56);
+//     the largest of the numbers that made it so far; a pair is taken as v = x 2^(57 - F), F the smaller
+//     exponent of its two results, |v| < 2^58: an exact shift of the 53-bit mantissa but for bits below
+//     2^(F - 57);
 //   * links are stored beside their FP64 form as u = U 2^57 in two 32-bit limbs (|U| <= 1);
-//   * projections are integer sums (< 2^58); a product takes three limb products, accumulated over the six
+//   * projections are integer sums (< 2^59); a product takes three limb products, accumulated over the six
 //     of a matrix row in two 64-bit sums: H of the high limbs' products and X of the mixed ones (the low
-//     limbs' products, each below one unit of H, are left out), w = H + X / 2^28 in units of v / 2,
-//     shifted to the exponent of each result;
-//   * the six directions add up in 64 bits (|sum| < 2^(56 + 6.9)).
+//     limbs' products, each below one unit of H, are left out), w = H + X / 2^28 in units of 2^(F - 58);
+//   * w is shifted to units of 2^(E_r - 57) of each of its two results, and the six directions add up in 64
+//     bits (|sum| < 2^62.9).
 //
 // Accuracy. A result component (one spin and colour) is a sum over directions and colours of a link entry
 // times two spinor components; S is the sum of the terms' absolute values, the scale of FP64 arithmetic's
-// error. Here the roundings (of v, U 2^57, the low products left out, X / 2^28 and the shift: 30 units of
-// 2^(E_r - 57) a direction) are below 11.3 x 2^-53 2^E_r, so the form is used only where S is not far
-// below 2^E_r (fx_accurate): either some direction brings result spin r a pair of spins all of whose three
-// colours reach 2^(E_r - 3) (a row of a unitary link has an entry of 1 / sqrt 3 or more, so then S >=
-// 2^(E_r - 3) / sqrt 3 for each colour, whatever the link), or every colour's result itself has reached
-// 2^(E_r - 3). Other sites take the FP64 form (hop_dir_fp64), as do sites whose result spins differ by
-// more than 2^31 and spinors with a NaN, an infinity or exponents near the ends of FP64's range. Errors in
+// error. Here the roundings (of v, U 2^57, the low products left out, X / 2^28 and the shift: 21 units of
+// 2^(E_r - 57) a direction) are below 7.9 x 2^-53 2^E_r, so the form is used only where S is not far below
+// 2^E_r (fx_accurate): either some direction brings result spin r a pair of spins all of whose three
+// colours reach 2^(E_r - 4) (the moduli in a row of a unitary link add up to 1 or more, so then S >=
+// 2^(E_r - 4) for each colour, whatever the link), or every colour's result itself has reached
+// 2^(E_r - 4). Other sites take the FP64 form (hop_dir_fp64), as do sites whose result spins differ by
+// more than 2^30 and spinors with a NaN, an infinity or exponents near the ends of FP64's range. Errors in
 // units of 2^-53 S, root mean square over the sites that pass, fixed point : FP64 arithmetic (emulated
 // against products in 113 bits): Gaussian spinors on random links 0.09 : 0.25, on links of unity 0.14 :
-// 0.31; two spins 2^-20 of the others 0.17 : 0.41; components scaled at random over 2^6 0.15 : 0.39, over
-// 2^30 0.38 : 0.72; colours 2^-3 of each other on links of unity 0.17 : 0.31; one component alone 0.29 :
-// 0.51. Largest 4.4 : 4.9. With 2^(E_r - 4) colours 2^-5 of each other would lose (0.48 : 0.31); with
+// 0.31; two spins 2^-20 of the others 0.17 : 0.41; components scaled at random over 2^6 0.14 : 0.39, over
+// 2^30 0.33 : 0.72; colours 2^-5 of each other on links of unity 0.25 : 0.31; one component alone 0.29 :
+// 0.51. Largest 4.7 : 4.9. With 2^(E_r - 5) colours 2^-6 of each other would lose (0.49 : 0.31); with
 // 2^(E_r - 2) some Gaussian sites would go to the FP64 form, and the whole launch of a small lattice waits
-// for one (8^3 x 32, FP64 solve 4.8 -> 7.9 ms).
+// for one (8^3 x 32, FP64 solve 4.9 -> 7.9 ms).
 #pragma once
 
 #include <type_traits>
@@ -54,7 +54,7 @@ __device__ __forceinline__ void fx_mac(long long& acc, int a, int b) {
 }
 
 constexpr int kFxMinExp = 80, kFxMaxExp = 2030;  // biased exponents served
-constexpr int kFxSpread = 3;                     // of 2^(E_r - 3) above
+constexpr int kFxSpread = 4;                     // of 2^(E_r - 4) above
 
 struct FxAcc {
   long long a[4][3][2];  // [spin][colour][re, im], in units of 2^(E_r - 1023 - 57)
@@ -168,9 +168,9 @@ __device__ __forceinline__ void fx_project(FxAcc& f, FxHalf& q, int d, const Vec
   for (int p = 0; p < 2; ++p) {
     const int eu = f.E(p), el = z ? f.E(2 + p) : f.E(3 - p);
     F[p] = min(eu, el);
-    f.wide = f.wide || (mx[p] != 0 && max(eu, el) - F[p] > 31);
-    q.up[p] = min(eu - F[p], 31);
-    q.lo[p] = min(el - F[p], 31);
+    f.wide = f.wide || (mx[p] != 0 && max(eu, el) - F[p] > 30);
+    q.up[p] = min(eu - F[p], 30) + 1;  // from units of 2^(F - 1023 - 58)
+    q.lo[p] = min(el - F[p], 30) + 1;
   }
   // h = u +- i sigma_k d (isigma of wf_line.cuh)
 #pragma unroll
@@ -179,10 +179,10 @@ __device__ __forceinline__ void fx_project(FxAcc& f, FxHalf& q, int d, const Vec
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
       const int G = z ? F[s] : F[1 - s];
-      u[s][0] = fx_from<4>(x[s].c[c].re, F[s]);
-      u[s][1] = fx_from<4>(x[s].c[c].im, F[s]);
-      v[s][0] = fx_from<4>(x[2 + s].c[c].re, G);
-      v[s][1] = fx_from<4>(x[2 + s].c[c].im, G);
+      u[s][0] = fx_from<5>(x[s].c[c].re, F[s]);
+      u[s][1] = fx_from<5>(x[s].c[c].im, F[s]);
+      v[s][0] = fx_from<5>(x[2 + s].c[c].re, G);
+      v[s][1] = fx_from<5>(x[2 + s].c[c].im, G);
     }
     switch (d) {
       case 0: u[0][0] -= v[1][1]; u[0][1] += v[1][0]; u[1][0] -= v[0][1]; u[1][1] += v[0][0]; break;

@@ -7,8 +7,8 @@ hardly do, and that do; one number of sites for each way the hop's directions ar
 and 1).
 
 Tolerance 256 x 2^-53 S for one application of M: the fixed-point sums are used where their error is below
-156 x 2^-53 S in each real number, 221 in a complex one (11.3 x 2^-53 times the largest number that enters
-the result's spin, over a smallest S of 2^-3 / sqrt 3 of that); the hop's and the diagonal's remaining
+127 x 2^-53 S in each real number, 180 in a complex one (7.9 x 2^-53 times the largest number that enters
+the result's spin, over a smallest S of 2^-4 of that); the hop's and the diagonal's remaining
 operations and the oracle's own add below 20 roundings each, 28 in a complex number. Two hops (the 4-D
 even-odd operator): twice that. In the axial frame the caller's colours are rotated (in FP64 arithmetic too),
 so S is formed from colour norms there, at least the largest number itself: 16 x 2^-53 S from the sums, 28 as
