@@ -108,65 +108,101 @@ __device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl,
     split_unit(e.im, G.h[k].im, G.l[k].im);
   }
 }
-// A rotation matrix in fixed point (wf_fixed.cuh): limbs of g 2^55
+// A rotation matrix in fixed point (wf_fixed.cuh): limbs of g 2^58
 struct FxMat {
   int2 re[9], im[9];
+  bool one;  // the unit matrix (t = 0 of every line): vectors pass unchanged
 };
 __device__ __forceinline__ int2 fx_limbs(long long v) { return make_int2((int)(v >> 28), (int)v & 0xfffffff); }
 __device__ __forceinline__ void load_rotation(const Cx<double>* __restrict__ gl, int tp, int sl, FxMat& G) {
+  G.one = true;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const Cx<double> e = gl[(size_t)k * tp + sl];
-    G.re[k] = fx_limbs(fx_from<3>(e.re, 1023));  // |g| <= 1 + 1e-9: exponents up to 1023
-    G.im[k] = fx_limbs(fx_from<3>(e.im, 1023));
+    G.re[k] = fx_limbs(fx_from<6>(e.re, 1023));  // |g| <= 1 + 1e-6: exponents up to 1023
+    G.im[k] = fx_limbs(fx_from<6>(e.im, 1023));
+    G.one = G.one && e.re == (k % 4 ? 0.0 : 1.0) && e.im == 0.0;
   }
 }
-// w = g v (DAG: g^dag v), the six numbers of v sharing one exponent; false (w unset) outside the
-// fixed-point range. Four spins of a site: about 1100 integer instructions and 24 conversions against 144
-// FP64 multiply-adds, i.e. some 20 clocks per site and SM against 72.
+// w = g v (DAG: g^dag v), the six numbers of v sharing one exponent E. Four spins of a site: about 1100
+// integer instructions and 24 conversions against 144 FP64 multiply-adds, i.e. some 20 clocks per site
+// and SM against 72. The roundings (v to 2^(E - 57), g to 2^-58, the low limbs' products left out,
+// X / 2^28) are below 0.63 x 2^-53 2^E; a component whose terms add up to S in absolute value therefore needs
+// S not far below 2^E, as in the hops: all three colours of v reach 2^(E - 4) (then S does, whatever g
+// is), or all of w's have. False (w unset) otherwise and outside the fixed-point range. Emulated, errors
+// in units of 2^-53 S, root mean square, fixed point : FP64 arithmetic: Gaussian vectors 0.28 : 0.53
+// (with v to 2^(E - 55), g to 2^-55 and X / 2^28 rounded down 0.81, half an ulp of it one-sided); colours
+// scattered over 2^20, g random 0.39 : 0.72, g near 1 0.48 : 0.75; 2^-4 of each other, g diagonal
+// 0.46 : 0.52. With 2^(E - 5) the last would lose (0.59 : 0.53).
+constexpr int kRotSpread = 4;
+// the larger of two magnitudes' high words
+__device__ __forceinline__ unsigned fx_word(double a, double b) {
+  return max((unsigned)__double2hiint(a) & 0x7fffffffu, (unsigned)__double2hiint(b) & 0x7fffffffu);
+}
 template <bool DAG>
 __device__ __forceinline__ bool rotate3_fx(const FxMat& G, const double (&v)[6], double (&w)[6]) {
-  unsigned mx = 0;
+  if (G.one) {
 #pragma unroll
-  for (int i = 0; i < 6; ++i) mx = max(mx, (unsigned)__double2hiint(v[i]) & 0x7fffffffu);
-  const int e = (int)(mx >> 20), E = max(e, kFxMinExp);
-  if (mx != 0 && (e < kFxMinExp || e >= kFxMaxExp)) return false;
-  int2 h[6], n[6];  // limbs of v and of -v
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    h[i] = fx_limbs(fx_from<3>(v[i], E));
-    n[i] = make_int2(-h[i].x, -h[i].y);
+    for (int i = 0; i < 6; ++i) w[i] = v[i];
+    return true;
   }
+  unsigned mx = 0, mn = ~0u;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const unsigned m = fx_word(v[2 * c], v[2 * c + 1]);
+    mx = max(mx, m);
+    mn = min(mn, m);
+  }
+  const int E = (int)(mx >> 20);
+  if (mx == 0) {  // zeros, or numbers below 2^-1042
+    unsigned low = 0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      low |= (unsigned)__double2loint(v[i]);
+      w[i] = 0.0;
+    }
+    return low == 0;
+  }
+  if (E < kFxMinExp || E >= kFxMaxExp) return false;
+  int2 h[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) h[i] = fx_limbs(fx_from<5>(v[i], E));
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    long long H[2] = {}, X[2] = {};
+    constexpr long long half = 1LL << 27;  // of X / 2^28, whose shift rounds down
+    long long H[2] = {}, X[2] = {half, half};
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
       const int2 r = G.re[DAG ? 3 * b + a : 3 * a + b], i = G.im[DAG ? 3 * b + a : 3 * a + b];
       // re: gr vr -+ gi vi, im: gr vi +- gi vr
-      const int2 vr = h[2 * b], vi = h[2 * b + 1], xi = DAG ? vi : n[2 * b + 1], xr = DAG ? n[2 * b] : vr;
+      const int2 vr = h[2 * b], vi = h[2 * b + 1], m = make_int2(-i.x, -i.y), ir = DAG ? i : m, ii = DAG ? m : i;
       fx_mac(H[0], r.x, vr.x);
       fx_mac(X[0], r.x, vr.y);
       fx_mac(X[0], r.y, vr.x);
-      fx_mac(H[0], i.x, xi.x);
-      fx_mac(X[0], i.x, xi.y);
-      fx_mac(X[0], i.y, xi.x);
+      fx_mac(H[0], ir.x, vi.x);
+      fx_mac(X[0], ir.x, vi.y);
+      fx_mac(X[0], ir.y, vi.x);
       fx_mac(H[1], r.x, vi.x);
       fx_mac(X[1], r.x, vi.y);
       fx_mac(X[1], r.y, vi.x);
-      fx_mac(H[1], i.x, xr.x);
-      fx_mac(X[1], i.x, xr.y);
-      fx_mac(X[1], i.y, xr.x);
+      fx_mac(H[1], ii.x, vr.x);
+      fx_mac(X[1], ii.x, vr.y);
+      fx_mac(X[1], ii.y, vr.x);
     }
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-      // g v = (H 2^56 + X 2^28) 2^-55 in units of 2^(E - 1023 - 55): H + X / 2^28 in units of 2^(E - 1077)
+      // g v = (H 2^56 + X 2^28) 2^-58 in units of 2^(E - 1023 - 57): H + X / 2^28 in units of 2^(E - 1082)
       const double x = (double)(H[q] + (X[q] >> 28));
       const int hi = __double2hiint(x);
-      w[2 * a + q] = __hiloint2double(hi ? hi + ((E - 1077) << 20) : 0, __double2loint(x));
+      w[2 * a + q] = __hiloint2double(hi ? hi + ((E - 1082) << 20) : 0, __double2loint(x));
     }
   }
-  return true;
+  const int least = E - kRotSpread;
+  if ((int)(mn >> 20) >= least) return true;
+  bool large = true;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) large = large && (int)(fx_word(w[2 * c], w[2 * c + 1]) >> 20) >= least;
+  return large;
 }
 
 // s + c = g v (DAG: g^dag v) for a vector v = f + lo (lo of relative size 2^-20 at most, or zero):
@@ -261,43 +297,49 @@ __device__ __forceinline__ void import_spin(const SplitMat& G, const Cx<double>*
 #pragma unroll
   for (int k = 0; k < 3; ++k) out[(size_t)k * os] = mk<float>(s[2 * k] + c[2 * k], s[2 * k + 1] + c[2 * k + 1]);
 }
-// One spin of a site on export: v rotated by G^dag into out (shared memory, 3 FP64 elements)
+// One spin of a site on export: v = in (components os elements apart) rotated by G^dag into out (shared
+// memory, 3 FP64 elements)
 template <typename R>
-__device__ __noinline__ void export_spin_wide(const Cx<double>* gl, int tp, Vec3<R> v, bool neg, Cx<double>* out) {
+__device__ __noinline__ void export_spin_wide(const Cx<double>* gl, int tp, const Cx<R>* in, int os, bool neg,
+                                              Cx<double>* out) {
   for (int a = 0; a < 3; ++a) {
     Cx<double> w = czero<double>();
-    for (int b = 0; b < 3; ++b)
-      w = cfmaconj(w, gl[(size_t)(3 * b + a) * tp], mk<double>((double)v.c[b].re, (double)v.c[b].im));
+    for (int b = 0; b < 3; ++b) {
+      const Cx<R> v = in[(size_t)b * os];
+      w = cfmaconj(w, gl[(size_t)(3 * b + a) * tp], mk<double>((double)v.re, (double)v.im));
+    }
     out[a] = neg ? mk<double>(-w.re, -w.im) : w;
   }
 }
-__device__ __forceinline__ void export_spin(const FxMat& G, const Cx<double>* gl, int tp, int sl, const Vec3<double>& v,
-                                            bool neg, Cx<double>* out) {
+__device__ __forceinline__ void export_spin(const FxMat& G, const Cx<double>* gl, int tp, int sl, const Cx<double>* in,
+                                            int os, bool neg, Cx<double>* out) {
   double x[6], w[6];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    x[2 * c] = neg ? -v.c[c].re : v.c[c].re;
-    x[2 * c + 1] = neg ? -v.c[c].im : v.c[c].im;
+    const Cx<double> v = in[(size_t)c * os];
+    x[2 * c] = neg ? -v.re : v.re;
+    x[2 * c + 1] = neg ? -v.im : v.im;
   }
   if (!rotate3_fx<true>(G, x, w)) {
-    export_spin_wide<double>(gl + sl, tp, v, neg, out);
+    export_spin_wide<double>(gl + sl, tp, in, os, neg, out);
     return;
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) out[c] = mk<double>(w[2 * c], w[2 * c + 1]);
 }
 __device__ __forceinline__ void export_spin(const SplitMat& G, const Cx<double>* gl, int tp, int sl,
-                                            const Vec3<float>& v, bool neg, Cx<double>* out) {
+                                            const Cx<float>* in, int os, bool neg, Cx<double>* out) {
   float f[6];
   bool ok = true;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    f[k] = k & 1 ? v.c[k >> 1].im : v.c[k >> 1].re;
+    const Cx<float> v = in[(size_t)(k >> 1) * os];
+    f[k] = k & 1 ? v.im : v.re;
     const unsigned a = __float_as_uint(f[k]) & 0x7fffffffu;
     ok &= a == 0 || (a >= (47u << 23) && a < (227u << 23));  // [2^-80, 2^100)
   }
   if (!ok) {
-    export_spin_wide<float>(gl + sl, tp, v, neg, out);
+    export_spin_wide<float>(gl + sl, tp, in, os, neg, out);
     return;
   }
   const float lo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -478,17 +520,14 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks)
       for (int i = 0; i < 4 / SPL; ++i) {
         const int sp = sp0 + i * SPL, ss = g5 ? (sp + 2) % 4 : sp;
         Cx<double>* out = buf + row * kTileRow + sp * 3;
-        Vec3<R> v = {};
-        if (src) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) v.c[c] = in[(size_t)(ss * 3 + c) * os];
-        }
+        const Cx<R>* from = in + (size_t)ss * 3 * os;
         if (src && gr) {
-          export_spin(G, gl, g.tp, gsl, v, g5 != 0, out);
+          export_spin(G, gl, g.tp, gsl, from, os, g5 != 0, out);
         } else {
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            const Cx<double> w = mk<double>((double)v.c[c].re, (double)v.c[c].im);
+            const Cx<R> v = src ? from[(size_t)c * os] : czero<R>();
+            const Cx<double> w = mk<double>((double)v.re, (double)v.im);
             out[c] = g5 ? mk<double>(-w.re, -w.im) : w;
           }
         }
