@@ -849,7 +849,8 @@ void qinv(wf_handle* h, const QFactors<R>& F, int p, const Cx<R>* in, Cx<R>* out
   const unsigned blocks = (unsigned)((size_t)h->g.Nl * ngrp);
   Prof P(h, tag<R>("qinv_apply_f64", "qinv_apply_f32"));
   auto run = [&](auto kernel) {
-    WF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit belongs to the kernel, not to the handle: always the longest line's, which any thread's launch fits
+    WF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)qinv_smem<R>(kTMax, G)));
     kernel<<<blocks, 32 * G, smem, h->stream>>>(a, ngrp);
     WF_CUDA(cudaGetLastError());
   };
