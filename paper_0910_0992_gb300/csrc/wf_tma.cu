@@ -267,7 +267,10 @@ __global__ void __launch_bounds__(32) k_line_tma(const LineArgs<float> A, int* e
 
 template <int OPU, int OPL>
 static void launch_tma_variant(const LineArgs<float>& a, int* err, cudaStream_t s) {
-  const size_t smem = (size_t)kStages * 18 * a.g.tp * sizeof(Cx<float>) + kStages * sizeof(uint64_t);
+  auto bytes = [](int tp) { return (size_t)kStages * 18 * tp * sizeof(Cx<float>) + kStages * sizeof(uint64_t); };
+  const size_t smem = bytes(a.g.tp);
+  // the limit belongs to the kernel: always the longest line's, which any thread's launch fits
+  WF_CUDA(cudaFuncSetAttribute(k_line_tma<OPU, OPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(32 * NMAX)));
   // resident CTAs per SM for this shared-memory size, looked up once (shared by threads)
   static std::mutex mu;
   static std::map<size_t, int> occ;
@@ -278,7 +281,6 @@ static void launch_tma_variant(const LineArgs<float>& a, int* err, cudaStream_t 
     std::lock_guard<std::mutex> lock(mu);
     auto it = occ.find(smem);
     if (it == occ.end()) {
-      WF_CUDA(cudaFuncSetAttribute(k_line_tma<OPU, OPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       WF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_per_sm, k_line_tma<OPU, OPL>, 32, smem));
       if (ctas_per_sm < 1) ctas_per_sm = 1;
       occ[smem] = ctas_per_sm;
@@ -286,7 +288,6 @@ static void launch_tma_variant(const LineArgs<float>& a, int* err, cudaStream_t 
       ctas_per_sm = it->second;
     }
   }
-  WF_CUDA(cudaFuncSetAttribute(k_line_tma<OPU, OPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int lines = a.nrhs * a.g.Nl;
   const int grid = lines < sms * ctas_per_sm ? lines : sms * ctas_per_sm;
   k_line_tma<OPU, OPL><<<grid, 32, smem, s>>>(a, err);
