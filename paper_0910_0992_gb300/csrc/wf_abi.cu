@@ -37,7 +37,7 @@ int guarded(wf_handle* h, F&& f) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev != h->device) WF_CUDA(cudaSetDevice(h->device));
-    return f();
+    return with_memory(h, f);
   } catch (const Error& e) {
     return fail(h, e.code, e.what());
   } catch (const std::bad_alloc&) {
@@ -140,8 +140,11 @@ LineArgs<R> line_args(wf_handle* h, int parity, int nrhs) {
   a.opl = OP_COPY;
   a.drop_job = -1;
   a.df = (sizeof(R) == 8 && h->df_ops) ? 1 : 0;
-  a.fx_out = h->usfx[parity].as<int4>();
-  a.fx_nbr = h->usfx[1 - parity].as<int4>();
+  if constexpr (sizeof(R) == 8) {
+    fx_links(h);
+    a.fx_out = h->fx(parity);
+    a.fx_nbr = h->fx(1 - parity);
+  }
   return a;
 }
 
@@ -278,6 +281,33 @@ std::vector<int2> build_unit_table(const Geom& g, int nrhs, int gsrc) {
 }  // namespace
 
 namespace wf {
+// Memory for the fixed-point links; without it, or with WF_FX=0, they are not tried again for this field
+static bool fx_room(wf_handle* h) {
+  const char* e = std::getenv("WF_FX");
+  const size_t bytes = (size_t)27 * h->g.Nl * h->g.tp * sizeof(int4);
+  try {
+    if (e && e[0] == '0') throw Error(WF_ENOMEM, "WF_FX=0");
+    for (int p = 0; p < 2; ++p) h->usfx[p].ensure(bytes, h->stream);
+  } catch (const Error& err) {
+    if (err.code != WF_ENOMEM) throw;
+    fx_drop(h);
+    return false;
+  }
+  return true;
+}
+void fx_drop(wf_handle* h) {
+  WF_CUDA(cudaStreamSynchronize(h->stream));
+  for (int p = 0; p < 2; ++p) h->usfx[p].release();
+  h->fx_state = wf_handle::FX_NONE;
+}
+void fx_links(wf_handle* h) {
+  if (h->fx_state != wf_handle::FX_NOT_YET || !fx_room(h)) return;
+  Prof P(h, "links_fx", 2);
+  for (int p = 0; p < 2; ++p)
+    launch_links_fx(h->us64[p].as<Cx<double>>(), h->usfx[p].as<int4>(), (size_t)27 * h->g.Nl * h->g.tp, h->stream);
+  h->fx_state = wf_handle::FX_FORMED;
+}
+
 // index tables for the wide kernels (built once per handle and per nrhs, on the handle's stream)
 void attach_tables(wf_handle* h, LineArgs<float>& a) {
   const Geom& g = h->g;
@@ -517,6 +547,7 @@ template <typename R>
 void m_apply(wf_handle* h, const Cx<R>* in_e, const Cx<R>* in_o, Cx<R>* out_e, Cx<R>* out_o, const Cx<R>* x_e,
              const Cx<R>* x_o, double a, int nrhs) {
   Gauge<R> G = gauge_of<R>(h);
+  if (sizeof(R) == 8) fx_links(h);
   for (int p = 0; p < 2; ++p) {
     MArgs<R> m;
     std::memset(&m, 0, sizeof(m));
@@ -529,8 +560,8 @@ void m_apply(wf_handle* h, const Cx<R>* in_e, const Cx<R>* in_o, Cx<R>* out_e, C
     m.pl = G.pl[p];
     m.us_out = G.us[p];
     m.us_nbr = G.us[1 - p];
-    m.fx_out = h->usfx[p].as<int4>();
-    m.fx_nbr = h->usfx[1 - p].as<int4>();
+    m.fx_out = h->fx(p);
+    m.fx_nbr = h->fx(1 - p);
     m.x = p ? x_o : x_e;
     m.a = (R)a;
     m.out = p ? out_o : out_e;
@@ -1838,11 +1869,12 @@ EoArgs<R> eo_args(wf_handle* h, int par, int nrhs) {
   a.g = h->g;
   a.par = par;
   a.nrhs = nrhs;
+  if (sizeof(R) == 8) fx_links(h);
   for (int p = 0; p < 2; ++p) {
     a.ut[p] = G.ut[p];
     a.pl[p] = G.pl[p];
     a.us[p] = G.us[p];
-    a.fx[p] = h->usfx[p].as<int4>();
+    a.fx[p] = h->fx(p);
   }
   a.inv_gf = (R)(1.0 / h->g.gamma_f);
   a.bc = (R)h->g.bc;
@@ -2064,6 +2096,7 @@ OpFn<R> full_op(wf_handle* h, bool temporal) {
     const int tp = h->g.tp;
     auto mrun = [&](const Cx<R>* in, Cx<R>* out, int swap) {
       Gauge<R> G = gauge_of<R>(h);
+      if (sizeof(R) == 8) fx_links(h);
       for (int p = 0; p < 2; ++p) {
         MArgs<R> m;
         std::memset(&m, 0, sizeof(m));
@@ -2076,8 +2109,8 @@ OpFn<R> full_op(wf_handle* h, bool temporal) {
         m.pl = G.pl[p];
         m.us_out = G.us[p];
         m.us_nbr = G.us[1 - p];
-        m.fx_out = h->usfx[p].as<int4>();
-        m.fx_nbr = h->usfx[1 - p].as<int4>();
+        m.fx_out = h->fx(p);
+        m.fx_nbr = h->fx(1 - p);
         m.swap = swap;
         m.out = out + p * hn;
         m.mu = (R)h->g.mu;
@@ -2918,7 +2951,6 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
       h->lamf64[p].ensure(nlam * sizeof(Cx<double>), s);
       if (!h->axial) h->ut32[p].ensure(nut * sizeof(Cx<float>), s);
       h->us32[p].ensure(nus32 * sizeof(Cx<float>), s);
-      h->usfx[p].ensure(nus * sizeof(int4), s);
       h->lamb32[p].ensure(nlam * sizeof(Cx<float>), s);
       h->lamf32[p].ensure(nlam * sizeof(Cx<float>), s);
     }
@@ -2926,6 +2958,11 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
     WF_CUDA(cudaMemsetAsync(h->iflag.p, 0, sizeof(int), s));
     Cx<double>* ut[2] = {h->ut64[0].as<Cx<double>>(), h->ut64[1].as<Cx<double>>()};
     Cx<double>* us[2] = {h->us64[0].as<Cx<double>>(), h->us64[1].as<Cx<double>>()};
+    // the fixed-point links with the others where the handle has used them before, and on lattices that
+    // wf_apply_schur_noalloc can serve, which may not form them itself; else by the first FP64 operator (they take
+    // as much memory as the FP64 links, 764 MB on 24^3 x 128, which FP32 operators never need)
+    h->fx_state = wf_handle::FX_NOT_YET;
+    const bool fx_now = (h->usfx[0].p || 4 * h->half_int() * sizeof(Cx<double>) <= WF_NOALLOC_SCRATCH_BYTES) && fx_room(h);
     if (h->axial) {  // ut becomes the rotation g, lamf the wrap matrix P Lambda
       AxialOut o;
       for (int p = 0; p < 2; ++p) {
@@ -2940,12 +2977,12 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
         o.lamb32[p] = h->lamb32[p].as<Cx<float>>();
         o.wrap32[p] = h->lamf32[p].as<Cx<float>>();
         o.us32[p] = h->us32[p].as<Cx<float>>();
-        o.usfx[p] = h->usfx[p].as<int4>();
+        o.usfx[p] = fx_now ? h->usfx[p].as<int4>() : nullptr;
       }
       Prof P(h, "gauge_ingest", 2);
       launch_axial_frame(g, dU, o, h->iflag.as<int>(), s);
     } else {
-      Prof P(h, "gauge_ingest", 1 + 2 * 6);
+      Prof P(h, "gauge_ingest", 1 + 2 * (5 + fx_now));
       launch_import_gauge(g, dU, ut, us, s);
       for (int p = 0; p < 2; ++p) {
         launch_tline_init(g, ut[p], h->lamb64[p].as<Cx<double>>(), h->lamf64[p].as<Cx<double>>(), h->iflag.as<int>(), s);
@@ -2953,13 +2990,14 @@ int wf_load_gauge(wf_handle_t* h, const double* U) {
         launch_d2f_links(us[p], h->us32[p].as<Cx<float>>(), (size_t)3 * g.Nl, g.tp, s);
         launch_d2f(h->lamb64[p].as<Cx<double>>(), h->lamb32[p].as<Cx<float>>(), nlam, s);
         launch_d2f(h->lamf64[p].as<Cx<double>>(), h->lamf32[p].as<Cx<float>>(), nlam, s);
-        launch_links_fx(us[p], h->usfx[p].as<int4>(), nus, s);
+        if (fx_now) launch_links_fx(us[p], h->usfx[p].as<int4>(), nus, s);
       }
     }
     int flag = 0;
     WF_CUDA(cudaMemcpyAsync(&flag, h->iflag.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     WF_CUDA(cudaStreamSynchronize(s));
     h->gauge = true;
+    if (fx_now) h->fx_state = wf_handle::FX_FORMED;
     if (flag) {
       h->gauge = false;
       throw Error(WF_ESINGULAR, "temporal preconditioner singular: |det(1 - bc mu^-T P)| < 1e-12 on some line");

@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_dsl
   Vec3<double> acc[4];
   const EoDir dir{A, x, y, z, p3, l, sl, h, A.in + (size_t)rhs * V3 * fstride, cu, cl};
   double unit[4];
-  hop_fx<S>(dir, Th, tp, active, acc, unit);
+  hop_fx<S>(dir, Th, tp, active, A.fx[0] != nullptr, acc, unit);
   const double af = A.a * A.inv_gf;
   if (S > 1 && threadIdx.x >= 32) return;
   // temporal hops: P_- U_t(t) psi(t+1) on spins 2-3, P_+ U_t^dag(t-1) psi(t-1) on spins 0-1
@@ -337,7 +337,6 @@ void launch_dslash4(const EoArgs<R>& a, bool axial, cudaStream_t s) {
     }
   }
   if constexpr (std::is_same<R, double>::value) {
-    if (!a.fx[0] || !a.fx[1]) throw Error(1, "FP64 dslash: no fixed-point links");
     const size_t total = (size_t)a.nrhs * a.g.L * a.g.L * a.g.L * (a.g.T / 2);
     fx_launch(total, [&](auto S, unsigned b, int th, size_t smem) {
       auto* k = axial ? k_dslash4_fx<true, S.value> : k_dslash4_fx<false, S.value>;

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks)
   double unit[4] = {0.0, 0.0, 0.0, 0.0};
   const bool site = in && t < g.T;
   hop_fx<S>(LineDir(g, A.parity, rhs, l, sl, A.src_up, A.src_lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site,
-            h, unit);
+            A.fx_out != nullptr, h, unit);
   if (!in || (S > 1 && threadIdx.x >= 32)) return;
   if (!site) {
 #pragma unroll
@@ -107,7 +107,8 @@ __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_app
   const Cx<double>* up = A.psi_q + (A.swap ? 6 * tp : 0);
   const Cx<double>* lo = A.psi_q + (A.swap ? 0 : 6 * tp);
   double unit[4];
-  hop_fx<S>(LineDir(g, A.parity, rhs, l, sl, up, lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site, h, unit);
+  hop_fx<S>(LineDir(g, A.parity, rhs, l, sl, up, lo, A.fx_out, A.fx_nbr, A.us_out, A.us_nbr), tp, tp, site,
+            A.fx_out != nullptr, h, unit);
   if (S > 1 && threadIdx.x >= 32) return;
   // axial frame: spins 0-1 at t = 0 need P^dag psi(T - 1), spins 2-3 at t = T - 1 P psi(0)
   Vec3<double> wr[2];
@@ -158,7 +159,6 @@ void launch_links_fx(const Cx<double>* in, int4* out, size_t n, cudaStream_t s) 
 }
 
 void launch_hop_fx(const LineArgs<double>& a, bool post, cudaStream_t s) {
-  if (!a.fx_out || !a.fx_nbr) throw Error(1, "FP64 hop: no fixed-point links");
   fx_launch((size_t)a.nrhs * a.g.Nl * a.g.tp, [&](auto S, unsigned b, int th, size_t smem) {
     fx_allow(k_hop_fx<S.value>, smem);
     launch_dep(k_hop_fx<S.value>, b, th, smem, s, a, post ? 1 : 0);
@@ -167,7 +167,6 @@ void launch_hop_fx(const LineArgs<double>& a, bool post, cudaStream_t s) {
 }
 
 void launch_apply_M_fx(const MArgs<double>& a, bool axial, cudaStream_t s) {
-  if (!a.fx_out || !a.fx_nbr) throw Error(1, "FP64 Wilson matrix: no fixed-point links");
   fx_launch((size_t)a.nrhs * a.g.Nl * a.g.tp, [&](auto S, unsigned b, int th, size_t smem) {
     auto* k = axial ? k_apply_M_fx<true, S.value> : k_apply_M_fx<false, S.value>;
     fx_allow(k, smem);

@@ -264,7 +264,7 @@ __device__ __forceinline__ double fx_unit(const FxAcc& f, int r) { return __hilo
 struct HopDir {
   const Cx<double>* up;  // the neighbour's components that supply spins 0-1, and
   const Cx<double>* lo;  // spins 2-3, cs elements apart
-  const int4* fx;        // the link in fixed point and in FP64, entries ls elements apart
+  const int4* fx;        // the link in fixed point (if there) and in FP64, entries ls elements apart
   const Cx<double>* u;
 };
 
@@ -312,9 +312,11 @@ __device__ __forceinline__ size_t fx_site() {
 // D_s = unit[s] h[s] for spin s (so that the scale joins the next multiply-add). With S > 1 the S warps
 // of a CTA take 6 / S directions each of the same 32 sites and warp 0 adds them up (integers: exactly,
 // but for the shift to a common exponent that the six directions of one thread see as well); the others
-// have no result. Called by every thread of the CTA; site: whether the thread has one.
+// have no result. Called by every thread of the CTA; site: whether the thread has one; fixed: whether there are
+// fixed-point links (else FP64 arithmetic).
 template <int S, class Dir>
-__device__ __forceinline__ void hop_fx(const Dir& dir, int cs, int ls, bool site, Vec3<double> (&h)[4], double (&unit)[4]) {
+__device__ __forceinline__ void hop_fx(const Dir& dir, int cs, int ls, bool site, bool fixed, Vec3<double> (&h)[4],
+                                       double (&unit)[4]) {
   extern __shared__ int4 fx_shared[];
   int4* stage = fx_shared + (threadIdx.x >> 5) * kFxStage + (threadIdx.x & 31);
   constexpr int N = 6 / S;
@@ -334,7 +336,8 @@ __device__ __forceinline__ void hop_fx(const Dir& dir, int cs, int ls, bool site
     for (int e = 0; e < 9; ++e) fx_copy(stage + 32 * (12 + e), q.fx + (size_t)e * ls);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if (site) {
+  f.wide = !fixed;
+  if (site && fixed) {
     HopDir next = dir(d0);
     fetch_spinor(next);
     fetch_link(next);

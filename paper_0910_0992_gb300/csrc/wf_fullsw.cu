@@ -880,8 +880,11 @@ void hop(wf_handle* h, int p, const Cx<R>* in, Cx<R>* out, int nrhs, const Cx<R>
   a.pl = gauge_pl<R>(h, p);
   a.us_out = gauge_us<R>(h, p);
   a.us_nbr = gauge_us<R>(h, 1 - p);
-  a.fx_out = h->usfx[p].as<int4>();
-  a.fx_nbr = h->usfx[1 - p].as<int4>();
+  if constexpr (sizeof(R) == 8) {
+    fx_links(h);
+    a.fx_out = h->fx(p);
+    a.fx_nbr = h->fx(1 - p);
+  }
   a.inv_mu = (R)(1.0 / h->g.mu);
   a.bc = (R)h->g.bc;
   a.xpost = xpost;
@@ -1008,8 +1011,9 @@ void msw_residual(wf_handle* h, int p, const Cx<double>* psi_e, const Cx<double>
   a.pl = h->pl64[p].as<Cx<double>>();
   a.us_out = h->us64[p].as<Cx<double>>();
   a.us_nbr = h->us64[1 - p].as<Cx<double>>();
-  a.fx_out = h->usfx[p].as<int4>();
-  a.fx_nbr = h->usfx[1 - p].as<int4>();
+  fx_links(h);
+  a.fx_out = h->fx(p);
+  a.fx_nbr = h->fx(1 - p);
   a.x = eta;
   a.a = -1.0;
   a.out = r;
@@ -1233,7 +1237,7 @@ int guard(wf_handle* h, F&& f) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev != h->device) WF_CUDA(cudaSetDevice(h->device));
-    return f();
+    return with_memory(h, f);
   } catch (const Error& e) {
     h->err = e.what();
     return e.code;

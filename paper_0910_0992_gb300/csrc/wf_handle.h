@@ -37,7 +37,11 @@ struct wf_handle {
   // gauge, per parity: U_t [Nl][9][tp], spatial [3][Nl][9][tp], Lambda [Nl][9]
   wf::DevBuf ut64[2], us64[2], lamb64[2], lamf64[2];
   wf::DevBuf ut32[2], us32[2], lamb32[2], lamf32[2];
-  wf::DevBuf usfx[2];  // spatial links in fixed point (wf_fixed.cuh), [3][Nl][9][tp]
+  // spatial links in fixed point (wf_fixed.cuh), [3][Nl][9][tp], of the loaded field where fx_state is FX_FORMED
+  enum FxState { FX_NOT_YET, FX_FORMED, FX_NONE };
+  FxState fx_state = FX_NOT_YET;
+  wf::DevBuf usfx[2];
+  const int4* fx(int p) const { return fx_state == FX_FORMED ? usfx[p].as<int4>() : nullptr; }
   // axial frame: ut64 holds the rotation g(x) instead of U_t; P per line
   wf::DevBuf pl64[2], pl32[2];
   // clover term of the SW operator (wf_load_gauge_clover): half its chiral blocks per parity,
@@ -155,6 +159,24 @@ struct Prof {
     }
   }
 };
+
+// Forms the fixed-point links of the loaded field if that has not been tried yet. Without memory for them, and with
+// environment WF_FX=0, fx() stays null: FP64 hops then run in FP64 arithmetic at every site.
+void fx_links(wf_handle* h);
+// gives the fixed-point links' memory back: fx() is null until the next field
+void fx_drop(wf_handle* h);
+// f(), and once more without the fixed-point links if an allocation failed while they were held (a call writes its
+// outputs last, after its allocations)
+template <class F>
+int with_memory(wf_handle* h, F&& f) {
+  try {
+    return f();
+  } catch (const Error& e) {
+    if (e.code != WF_ENOMEM || h->fx_state != wf_handle::FX_FORMED) throw;
+  }
+  fx_drop(h);
+  return f();
+}
 
 // index tables of the one-thread-per-site kernels (neighbour lines, traversal order) for a.nrhs
 // sources, built on first use

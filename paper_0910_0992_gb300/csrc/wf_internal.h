@@ -47,6 +47,7 @@ struct DevBuf {
     cudaError_t e = cudaMalloc(&p, nbytes);
     if (e != cudaSuccess) {
       p = nullptr;
+      (void)cudaGetLastError();  // or the next launch's check would report it
       throw Error(2 /*WF_ENOMEM*/, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     }
     bytes = nbytes;
@@ -125,7 +126,7 @@ struct MArgs {
   const Cx<R>* pl;     // per-line boundary link P (axial frame)
   const Cx<R>* us_out; // forward spatial links, own parity
   const Cx<R>* us_nbr; // forward spatial links, other parity
-  const int4* fx_out;  // R = double: both in fixed point (wf_fixed.cuh)
+  const int4* fx_out;  // R = double: both in fixed point (wf_fixed.cuh), or null
   const int4* fx_nbr;
   const Cx<R>* x;      // out = x + a * (M psi) if x != nullptr
   R a;
@@ -166,7 +167,7 @@ void launch_tline_init(const Geom& g, const Cx<double>* ut, Cx<double>* lamb, Cx
                        cudaStream_t s);
 // the axial frame from the lexicographic links, per parity: the rotation g [Nl][9][tp], P, Lambda and
 // the wrap matrix P Lambda [Nl][9] in FP64 and FP32, the rotated spatial links [3][Nl][9][tp] in FP64 and
-// fixed point and [3][Nl][6][tp] in FP32
+// fixed point (null: not) and [3][Nl][6][tp] in FP32
 struct AxialOut {
   Cx<double>*g[2], *pl[2], *lamb[2], *wrap[2], *us[2];
   Cx<float>*pl32[2], *lamb32[2], *wrap32[2], *us32[2];
@@ -256,7 +257,7 @@ struct EoArgs {
   const Cx<R>* ut[2];     // general frame: U_t per 3-D parity, line layout
   const Cx<R>* pl[2];     // axial frame: boundary link P per line
   const Cx<R>* us[2];     // spatial forward links per 3-D parity, line layout
-  const int4* fx[2];      // R = double: the same in fixed point (wf_fixed.cuh)
+  const int4* fx[2];      // R = double: the same in fixed point (wf_fixed.cuh), or null
   R inv_gf, bc;
 };
 template <typename R>

@@ -743,8 +743,10 @@ __global__ void __launch_bounds__(128) k_axial_links(const Geom g, const Cx<doub
 #pragma unroll
   for (int e = 0; e < 9; ++e) {
     o.us[p][(lk * 9 + e) * g.tp + sl] = r.e[e];
-    const int2 re = link_limbs(r.e[e].re), im = link_limbs(r.e[e].im);
-    o.usfx[p][(lk * 9 + e) * g.tp + sl] = make_int4(re.x, re.y, im.x, im.y);
+    if (o.usfx[p]) {
+      const int2 re = link_limbs(r.e[e].re), im = link_limbs(r.e[e].im);
+      o.usfx[p][(lk * 9 + e) * g.tp + sl] = make_int4(re.x, re.y, im.x, im.y);
+    }
     if (e < NC) o.us32[p][(lk * NC + e) * g.tp + sl] = mk<float>((float)r.e[e].re, (float)r.e[e].im);
   }
 }

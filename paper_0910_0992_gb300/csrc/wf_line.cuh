@@ -55,7 +55,7 @@ struct LineArgs {
   const Cx<R>* pl;
   const Cx<R>* us_out;
   const Cx<R>* us_nbr;
-  const int4* fx_out;  // R = double: the spatial links in fixed point (wf_fixed.cuh), [3][Nl][9][tp]
+  const int4* fx_out;  // R = double: the spatial links in fixed point (wf_fixed.cuh), [3][Nl][9][tp], or null
   const int4* fx_nbr;
   const Cx<R>* lamb;  // Lambda for T^-1, [Nl][9]
   const Cx<R>* lamf;  // general frame: Lambda for T^-dag, [Nl][9]; axial frame: the wrap matrix
