@@ -85,27 +85,21 @@ template void launch_norm2<double>(const Cx<double>*, size_t, int, double*, doub
 template <typename R>
 __global__ void __launch_bounds__(kBT) k_cg_xr(Cx<R>* __restrict__ x, Cx<R>* __restrict__ r, const Cx<R>* __restrict__ p,
                                                 const Cx<R>* __restrict__ q, size_t n, const double* gamma,
-                                                const double* qq, const int* active, double* partial,
-                                                const size_t* offs, int* upd) {
+                                                const double* qq, const int* active, double* partial) {
   const int rhs = blockIdx.y;
   const bool on = active[rhs] != 0;
   const double qn = qq[rhs];
   const R alpha = (on && qn > 0.0) ? (R)(gamma[rhs] / qn) : R(0);
-  if (upd && blockIdx.x == 0 && threadIdx.x == 0) upd[rhs] = on ? 1 : 0;
-  size_t off, len;
-  rhs_range(rhs, n, offs, off, len);
-  n = len;
+  const size_t off = rhs * n;
   R part = R(0);  // per-thread partial |r|^2 in the field's precision; FP64 across threads
   for (size_t i = blockIdx.x * (size_t)kBT + threadIdx.x; i < n; i += (size_t)gridDim.x * kBT) {
     const Cx<R> qv = q[off + i];
     Cx<R> rv = r[off + i];
-    if (x) {
-      const Cx<R> pv = p[off + i];
-      Cx<R> xv = x[off + i];
-      xv.re = fma(alpha, pv.re, xv.re);
-      xv.im = fma(alpha, pv.im, xv.im);
-      x[off + i] = xv;
-    }
+    const Cx<R> pv = p[off + i];
+    Cx<R> xv = x[off + i];
+    xv.re = fma(alpha, pv.re, xv.re);
+    xv.im = fma(alpha, pv.im, xv.im);
+    x[off + i] = xv;
     rv.re = fma(-alpha, qv.re, rv.re);
     rv.im = fma(-alpha, qv.im, rv.im);
     r[off + i] = rv;
@@ -117,19 +111,16 @@ __global__ void __launch_bounds__(kBT) k_cg_xr(Cx<R>* __restrict__ x, Cx<R>* __r
 
 template <typename R>
 void launch_cg_xr(Cx<R>* x, Cx<R>* r, const Cx<R>* p, const Cx<R>* q, size_t n, int nrhs, const double* gamma,
-                  const double* qq, const int* active, double* partial, double* rr_out, cudaStream_t s,
-                  const size_t* offs, int* upd) {
+                  const double* qq, const int* active, double* partial, double* rr_out, cudaStream_t s) {
   const int parts = parts_for(n);
-  k_cg_xr<R><<<dim3(parts, nrhs), kBT, 0, s>>>(x, r, p, q, n, gamma, qq, active, partial, offs, upd);
+  k_cg_xr<R><<<dim3(parts, nrhs), kBT, 0, s>>>(x, r, p, q, n, gamma, qq, active, partial);
   k_final_sum<<<nrhs, kBT, 0, s>>>(partial, parts, rr_out);
   WF_CUDA(cudaGetLastError());
 }
 template void launch_cg_xr<float>(Cx<float>*, Cx<float>*, const Cx<float>*, const Cx<float>*, size_t, int,
-                                  const double*, const double*, const int*, double*, double*, cudaStream_t,
-                                  const size_t*, int*);
+                                  const double*, const double*, const int*, double*, double*, cudaStream_t);
 template void launch_cg_xr<double>(Cx<double>*, Cx<double>*, const Cx<double>*, const Cx<double>*, size_t, int,
-                                   const double*, const double*, const int*, double*, double*, cudaStream_t,
-                                   const size_t*, int*);
+                                   const double*, const double*, const int*, double*, double*, cudaStream_t);
 
 // True on every thread of the last block of right-hand side rhs to get here (then its counter is zero
 // again and the other blocks' writes before the call are visible)

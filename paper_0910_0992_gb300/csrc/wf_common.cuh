@@ -233,9 +233,20 @@ __host__ __device__ __forceinline__ void neighbour_lines(const Geom& g, int p, i
   nb[5] = line_of(g, x, y, (z + L - 1) % L);
 }
 
+// SMs of a GB300: launch shapes are sized for them (any number runs)
+constexpr int kSMs = 152;
+
 // Start of a kernel launched by launch_dep (wf_internal.h): waits until the kernel before it in the stream has
 // completed. Precedes every access to memory.
 __device__ __forceinline__ void grid_dep() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// 16 bytes from device to shared memory, asynchronously (both addresses 16-byte aligned; completion tracked
+// per thread in commit groups)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
+               "l"(__cvta_generic_to_global(src))
+               : "memory");
+}
 
 // Spinor component index: spin * 3 + colour. Dirac-Pauli basis: spins 0, 1 are the
 // P_+ = (1 + gamma_t)/2 ("upper") half, spins 2, 3 the P_- ("lower") half.

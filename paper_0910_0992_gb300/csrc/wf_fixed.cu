@@ -153,7 +153,7 @@ __global__ void k_links_fx(const Cx<double>* __restrict__ in, int4* __restrict__
 }  // namespace
 
 void launch_links_fx(const Cx<double>* in, int4* out, size_t n, cudaStream_t s) {
-  const unsigned b = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 152 * 16));
+  const unsigned b = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, kSMs * 16));
   k_links_fx<<<b, 256, 0, s>>>(in, out, n);
   WF_CUDA(cudaGetLastError());
 }

@@ -286,12 +286,6 @@ static __device__ __noinline__ void hop_dir_fp64(int d, HopDir q, int cs, int ls
     }
 }
 
-// 16 bytes of device memory into shared memory, asynchronously
-__device__ __forceinline__ void fx_copy(int4* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
-               "l"(__cvta_generic_to_global(src))
-               : "memory");
-}
 // dynamic shared memory of a warp: 12 spinor and 9 link entries per lane. A lane reads only what it
 // copied, so the copies need no barrier: a direction's spinor arrives while the one before multiplies its
 // link, its link while it is projected.
@@ -326,14 +320,14 @@ __device__ __forceinline__ void hop_fx(const Dir& dir, int cs, int ls, bool site
   auto fetch_spinor = [&](const HopDir& q) {
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      fx_copy(stage + 32 * c, q.up + (size_t)c * cs);
-      fx_copy(stage + 32 * (6 + c), q.lo + (size_t)c * cs);
+      cp_async16(stage + 32 * c, q.up + (size_t)c * cs);
+      cp_async16(stage + 32 * (6 + c), q.lo + (size_t)c * cs);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   auto fetch_link = [&](const HopDir& q) {
 #pragma unroll
-    for (int e = 0; e < 9; ++e) fx_copy(stage + 32 * (12 + e), q.fx + (size_t)e * ls);
+    for (int e = 0; e < 9; ++e) cp_async16(stage + 32 * (12 + e), q.fx + (size_t)e * ls);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   f.wide = !fixed;
@@ -436,11 +430,11 @@ inline void fx_launch(size_t sites, Run&& run) {
     constexpr int th = FxShape<S.value>::threads, per = S.value == 1 ? th : 32;
     run(S, (unsigned)((sites + per - 1) / per), th, fx_smem(th));
   };
-  if (warps <= 152 * FxShape<6>::blocks)
+  if (warps <= kSMs * FxShape<6>::blocks)
     go(std::integral_constant<int, 6>{});
-  else if (warps <= 152 * FxShape<3>::blocks)
+  else if (warps <= kSMs * FxShape<3>::blocks)
     go(std::integral_constant<int, 3>{});
-  else if (warps <= 152 * FxShape<2>::blocks)
+  else if (warps <= kSMs * FxShape<2>::blocks)
     go(std::integral_constant<int, 2>{});
   else
     go(std::integral_constant<int, 1>{});

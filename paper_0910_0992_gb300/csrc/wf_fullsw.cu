@@ -320,13 +320,7 @@ struct QinvArgs {
   R s;                 // boundary sign
 };
 
-// 16- and 8-byte asynchronous global -> shared copies (addresses aligned to their size; completion
-// tracked per thread in commit groups)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
-               "l"(__cvta_generic_to_global(src))
-               : "memory");
-}
+// 8 bytes from device to shared memory, as cp_async16
 __device__ __forceinline__ void cp_async8(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
                "l"(__cvta_generic_to_global(src))
@@ -734,7 +728,7 @@ bool qinv_current(wf_handle* h, unsigned long long* key) {
   WF_CUDA(cudaMemsetAsync(kb, 0, sizeof(unsigned long long), s));
   auto add = [&](const void* p, size_t bytes, unsigned long long salt) {
     const size_t n = bytes / sizeof(unsigned long long);
-    const unsigned blocks = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 152 * 8));
+    const unsigned blocks = (unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, kSMs * 8));
     Prof P(h, "fsw_fingerprint");
     k_fingerprint<<<blocks, 256, 0, s>>>(static_cast<const unsigned long long*>(p), n, salt, kb);
     WF_CUDA(cudaGetLastError());

@@ -63,8 +63,7 @@ struct DevBuf {
 template <typename R> struct LineArgs;
 
 // kernel<<<grid, block, smem, s>>>(args...) whose launch may overlap the end of the kernel before it in the
-// stream; the kernel starts with grid_dep (wf_common.cuh) and reads nothing through the read-only path before
-// it has branched. Schur apply FP64 4^3 x 16 100 -> 85 us, FP32 16^3 x 128 217 -> 207; in graphs: FP64 solve
+// stream; the kernel starts with grid_dep (wf_common.cuh), before any access to memory. Schur apply FP64 4^3 x 16 100 -> 85 us, FP32 16^3 x 128 217 -> 207; in graphs: FP64 solve
 // 8^3 x 32, two sources, 5.00 -> 4.88 ms, force and action 8^3 x 32 3.01 -> 2.88 ms. Triggering the next launch at a
 // kernel's start loses that (5.71, 3.47 ms): its waiting CTAs are resident on the SMs that were free first,
 // and share them when their turn comes.
@@ -180,7 +179,6 @@ void launch_check_links(const Cx<double>* U, size_t nlinks, double tol, int* fla
 void launch_d2f(const Cx<double>* in, Cx<float>* out, size_t n, cudaStream_t s);
 // FP32 copy of spatial links in their two-row storage (nlinks = 3 Nl per parity)
 void launch_d2f_links(const Cx<double>* in, Cx<float>* out, size_t nlinks, int tp, cudaStream_t s);
-void launch_f2d(const Cx<float>* in, Cx<double>* out, size_t n, cudaStream_t s);
 
 // BLAS-1 on flat [nrhs][n] arrays; scalars live in device memory. offs (ragged batches of several
 // lattices): device prefix table [nrhs + 1] of each rhs's first element in the packed vectors, n
@@ -205,14 +203,12 @@ struct CgAdvance {
 template <typename R>
 void launch_cg_r_check(Cx<R>* r, const Cx<R>* q, size_t n, int nrhs, const double* gamma, const double* qq,
                        double* partial, double* rr, const CgState& c, cudaStream_t s, const size_t* offs = nullptr);
-// CG updates: launch_cg_xr does r -= alpha q (alpha = gamma / qq) with |r|^2 into rr_out, and
-// x += alpha p unless x is null; then upd (if given) records the right-hand sides that took the
-// update. launch_cg_p does p = s + beta p (beta = gamma_new / gamma_old) for the active ones and,
+// CG updates: launch_cg_xr does x += alpha p and r -= alpha q (alpha = gamma / qq) with |r|^2 into rr_out.
+// launch_cg_p does p = s + beta p (beta = gamma_new / gamma_old) for the active ones and,
 // with x given, first the deferred x += alpha p (alpha = gamma_old / qq) for those flagged in upd.
 template <typename R>
 void launch_cg_xr(Cx<R>* x, Cx<R>* r, const Cx<R>* p, const Cx<R>* q, size_t n, int nrhs, const double* gamma,
-                  const double* qq, const int* active, double* partial, double* rr_out, cudaStream_t s,
-                  const size_t* offs = nullptr, int* upd = nullptr);
+                  const double* qq, const int* active, double* partial, double* rr_out, cudaStream_t s);
 template <typename R>
 void launch_cg_p(Cx<R>* p, const Cx<R>* sv, size_t n, int nrhs, const double* gamma_new, const double* gamma_old,
                  const int* active, cudaStream_t s, const size_t* offs = nullptr, Cx<R>* x = nullptr,

@@ -26,7 +26,8 @@ namespace wf {
 // In the axial frame the FP32 hop kernels of the Schur operator (K-b, K-c) run as the
 // one-thread-per-site kernels of wf_wide.cu: measured on GB300 (24^3 x 128) 1.15-1.3x faster
 // than k_line. The scan-heavy, memory-light K-a stays on k_line, which amortises the scan over
-// n sites per lane; FP64 arithmetic stays on k_line too. Environment WF_WIDE=0 disables the
+// n sites per lane; FP64 line operations stay on k_line or k_line_spin, after their hop has run in k_hop_fx.
+// Environment WF_WIDE=0 disables the
 // wide FP32 kernels, WF_WIDE=2 uses them for every FP32 axial line operation.
 static bool use_wide(const Geom& g, int kind, bool fp32) {
   static const int mode = []() {  // read once (thread-safe initialisation)
@@ -82,7 +83,6 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
     }
   }
   constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;
-  constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
 #define WF_KL(AXV, SRCV, OPUV, OPLV) launch_dep(k_line<R, AXV, SRCV, OPUV, OPLV>, b, th, 0, s, a)
   if (axial) {
     switch (kind) {
@@ -93,7 +93,7 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
         if (a.src == SRC_LOAD)
           WF_KL(true, SRC_LOAD, -1, -1);
         else
-          WF_KL(true, ANY, -1, -1);
+          WF_KL(true, HOP, -1, -1);
         break;
     }
   } else {
@@ -105,7 +105,7 @@ static void launch_line_impl(const LineArgs<R>& a, int kind, bool axial, cudaStr
         if (a.src == SRC_LOAD)
           WF_KL(false, SRC_LOAD, -1, -1);
         else
-          WF_KL(false, ANY, -1, -1);
+          WF_KL(false, HOP, -1, -1);
         break;
     }
   }
@@ -217,28 +217,25 @@ template void launch_line_multi<float>(const std::vector<LineArgs<float>>&, int,
 template void launch_line<float>(const LineArgs<float>&, int, bool, cudaStream_t);
 template void launch_line<double>(const LineArgs<double>&, int, bool, cudaStream_t);
 
-template <typename R>
-void launch_apply_M(const MArgs<R>& a, bool axial, cudaStream_t s) {
-  if constexpr (std::is_same<R, double>::value) {
-    launch_apply_M_fx(a, axial, s);
-    return;
-  } else {
+template <>
+void launch_apply_M<float>(const MArgs<float>& a, bool axial, cudaStream_t s) {
   if (a.g.n < 1 || a.g.n > NMAX_LONG) throw Error(1, "unsupported sites per lane");
   const int lines = a.nrhs * a.g.Nl;
   const int warps = (lines + a.g.lpw - 1) / a.g.lpw;
   const int blocks = (warps * 32 + kLineThreads - 1) / kLineThreads;
   if (a.g.n > NMAX) {  // lines longer than 128 slots (wf_kernels_long_*.cu)
-    launch_apply_M_long<R>(a, axial, s);
+    launch_apply_M_long<float>(a, axial, s);
     return;
   }
   if (axial)
-    launch_dep(k_apply_M<R, true, NMAX>, blocks, kLineThreads, 0, s, a);
+    launch_dep(k_apply_M<float, true, NMAX>, blocks, kLineThreads, 0, s, a);
   else
-    launch_dep(k_apply_M<R, false, NMAX>, blocks, kLineThreads, 0, s, a);
+    launch_dep(k_apply_M<float, false, NMAX>, blocks, kLineThreads, 0, s, a);
   WF_CUDA(cudaGetLastError());
-  }
 }
-template void launch_apply_M<float>(const MArgs<float>&, bool, cudaStream_t);
-template void launch_apply_M<double>(const MArgs<double>&, bool, cudaStream_t);
+template <>
+void launch_apply_M<double>(const MArgs<double>& a, bool axial, cudaStream_t s) {
+  launch_apply_M_fx(a, axial, s);
+}
 
 }  // namespace wf

@@ -62,11 +62,6 @@ struct SpinorTile {
   int rper;   // sources per CTA
 };
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
-               "l"(__cvta_generic_to_global(src))
-               : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---- FP32 rotation with exact products.
@@ -755,14 +750,10 @@ __global__ void k_d2f(const Cx<double>* __restrict__ in, Cx<float>* __restrict__
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     out[i] = mk<float>((float)in[i].re, (float)in[i].im);
 }
-__global__ void k_f2d(const Cx<float>* __restrict__ in, Cx<double>* __restrict__ out, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    out[i] = mk<double>((double)in[i].re, (double)in[i].im);
-}
 
 static int grid_for(size_t n) {
   int b = nblocks(n);
-  return b > 152 * 16 ? 152 * 16 : (b < 1 ? 1 : b);
+  return b > kSMs * 16 ? kSMs * 16 : (b < 1 ? 1 : b);
 }
 
 // Tile of an import / export over npar parities: about 32 times (runs of 4 to 32 slots) of up to 8
@@ -789,9 +780,9 @@ static SpinorTile tile_of(const Geom& g, int npar, int nrhs, bool eo, dim3& grid
     return (long long)npar * t.ntl * t.nch;
   };
   long long blocks = lines(kTileThreads);
-  split = blocks * nrhs < 2 * 152;
+  split = blocks * nrhs < 2 * kSMs;
   if (split) blocks = lines(kTileThreads / 4);
-  long long rgroups = std::min<long long>(nrhs, (8 * 152 + blocks - 1) / blocks);
+  long long rgroups = std::min<long long>(nrhs, (8 * kSMs + blocks - 1) / blocks);
   t.rper = (int)((nrhs + rgroups - 1) / rgroups);
   grid = dim3((unsigned)blocks, (unsigned)((nrhs + t.rper - 1) / t.rper));
   return t;
@@ -958,10 +949,6 @@ void launch_check_links(const Cx<double>* U, size_t nlinks, double tol, int* fla
 
 void launch_d2f(const Cx<double>* in, Cx<float>* out, size_t n, cudaStream_t s) {
   k_d2f<<<grid_for(n), kThreads, 0, s>>>(in, out, n);
-  WF_CUDA(cudaGetLastError());
-}
-void launch_f2d(const Cx<float>* in, Cx<double>* out, size_t n, cudaStream_t s) {
-  k_f2d<<<grid_for(n), kThreads, 0, s>>>(in, out, n);
   WF_CUDA(cudaGetLastError());
 }
 

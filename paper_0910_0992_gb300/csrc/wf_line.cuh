@@ -363,8 +363,6 @@ __device__ __forceinline__ Vec3<R> vadd(const Vec3<R>& x, const Vec3<R>& y) {
   return w;
 }
 
-// |x|^2 in the field's own precision (GB300's FP64 rate is far below its FP32 rate, so FP32
-// kernels keep FP64 for the final cross-thread sums only)
 // Hermitian 6x6 blocks over slots (the clover term): FP64 whole, [36][stride]; FP32 the diagonal in
 // pairs, then the entries below it, (r, c) at plane 3 + r (r - 1) / 2 + c: [18][stride]
 template <typename R>
@@ -386,6 +384,8 @@ __device__ __forceinline__ Cx<R> herm_entry(const Cx<R>* H, int r, int c, size_t
   }
 }
 
+// |x|^2 in the field's own precision (GB300's FP64 rate is far below its FP32 rate, so FP32
+// kernels keep FP64 for the final cross-thread sums only)
 template <typename R>
 __device__ __forceinline__ R vnorm2(const Vec3<R>& x) {
   R s = R(0);

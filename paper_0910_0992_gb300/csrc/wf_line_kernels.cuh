@@ -12,11 +12,8 @@
 namespace wf {
 
 constexpr int kLineThreads = 128;
-#ifndef WF_LINE_MINB
-#define WF_LINE_MINB 3
-#endif
-// resident CTAs per SM the line kernels are compiled for (3: 168 registers; measured best
-// on GB300 against 1 and 4, where 4 spills)
+
+// T^-1 (FWD: T^-dag) on the spins s0, s0 + 1 (W = 1: s0) of a lane's sites
 template <typename R, bool AX, bool FWD, int NM, int W>
 __device__ __forceinline__ void solve_half(Vec3<R> (&v)[NM][W], int s0, const LineArgs<R>& A, int l, int jj) {
   constexpr int NS = sizeof(R) == 4 && W > 1 ? 2 : 1;
@@ -100,7 +97,11 @@ __device__ __forceinline__ void line_norm(const LineArgs<R>& A, R nrm, int rhs, 
   if (active && jj == 0) atomicAdd(A.norm2 + rhs, dn);
 }
 
-// SRC, OPU, OPL < 0: taken from the arguments at run time
+// resident CTAs per SM the line kernels are compiled for (3: 168 registers; measured best
+// on GB300 against 1 and 4, where 4 spills)
+#ifndef WF_LINE_MINB
+#define WF_LINE_MINB 3
+#endif
 #ifndef WF_LINE_MINB_F64
 #define WF_LINE_MINB_F64 3
 #endif
@@ -109,12 +110,12 @@ struct LineMinBlocks {
   static constexpr int value = sizeof(R) == 4 ? WF_LINE_MINB : WF_LINE_MINB_F64;
 };
 
-// The kernel body for block blk of a launch over one lattice (see k_line and k_line_multi).
+// The kernel body for block blk of a launch over one lattice (see k_line and k_line_multi). OPU, OPL < 0:
+// taken from the arguments at run time.
 template <typename R, bool AX, int SRC, int OPU, int OPL, bool H = false, int NM = NMAX>
 __device__ __forceinline__ void line_body(const LineArgs<R>& A, int blk) {
   static_assert(!H || SRC == SRC_LOAD, "FP16 storage: the line kernel loads its own site only");
   const Geom& g = A.g;
-  const int src = SRC >= 0 ? SRC : A.src;
   const int opu = OPU >= 0 ? OPU : A.opu;
   const int opl = OPL >= 0 ? OPL : A.opl;
   const int lane = threadIdx.x & 31;
@@ -145,47 +146,32 @@ __device__ __forceinline__ void line_body(const LineArgs<R>& A, int blk) {
       }
     }
   } else {
-  Vec3<R> v[NM][4];
-  if (src == SRC_HOP) {
+    Vec3<R> v[NM][4];
     hop_spatial<R>(v, A, rhs, l, jj);
-  } else {
+    if (A.xpre) {
 #pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      const int sl = m * g.lpl + jj;
-      const bool ok = m < n;
-      const bool up = ok && opu != OP_SKIP, lo = ok && opl != OP_SKIP;
-      v[m][0] = up ? ldv<R, H>(A.src_up, base, tp, sl) : vzero<R>();
-      v[m][1] = up ? ldv<R, H>(A.src_up, base + 3 * tp, tp, sl) : vzero<R>();
-      v[m][2] = lo ? ldv<R, H>(A.src_lo, base, tp, sl) : vzero<R>();
-      v[m][3] = lo ? ldv<R, H>(A.src_lo, base + 3 * tp, tp, sl) : vzero<R>();
-    }
-  }
-  if (A.xpre) {
+      for (int m = 0; m < NM; ++m) {
+        if (m >= n) continue;
 #pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      if (m >= n) continue;
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-        v[m][s] = vaxpy(A.apre, v[m][s], ldv<R, H>(A.xpre, base + 3 * s * tp, tp, m * g.lpl + jj));
-    }
-  }
-
-  apply_op<R, AX>(opu, v, 0, A, l, jj);
-  apply_op<R, AX>(opl, v, 2, A, l, jj);
-
-  if (active) {
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      if (m >= n) continue;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if ((h ? opl : opu) == OP_SKIP) continue;
-#pragma unroll
-        for (int s = 0; s < 2; ++s)
-          store_spin<R, H>(A, base, h, s, m * g.lpl + jj, jj * n + m < g.T, v[m][2 * h + s], nrm);
+        for (int s = 0; s < 4; ++s)
+          v[m][s] = vaxpy(A.apre, v[m][s], ldv<R, H>(A.xpre, base + 3 * s * tp, tp, m * g.lpl + jj));
       }
     }
-  }
+    apply_op<R, AX>(opu, v, 0, A, l, jj);
+    apply_op<R, AX>(opl, v, 2, A, l, jj);
+    if (active) {
+#pragma unroll
+      for (int m = 0; m < NM; ++m) {
+        if (m >= n) continue;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if ((h ? opl : opu) == OP_SKIP) continue;
+#pragma unroll
+          for (int s = 0; s < 2; ++s)
+            store_spin<R, H>(A, base, h, s, m * g.lpl + jj, jj * n + m < g.T, v[m][2 * h + s], nrm);
+        }
+      }
+    }
   }
   if (want_norm) line_norm(A, nrm, rhs, jj, active);
 }
@@ -235,7 +221,7 @@ inline int line_blocks(const LineArgs<R>& a, int threads = kLineThreads) {
 // CTA size: one warp where the lattice has fewer than four per SM, so that they spread over all SMs
 // (FP64 then also splits a line's spins, k_line_spin: with 1024 warps that is slower, K-a 19 -> 22 us on
 // 8^3 x 32 with four sources)
-inline bool few_lines(const Geom& g, int nrhs) { return line_warps(g, nrhs) < 4 * 152; }
+inline bool few_lines(const Geom& g, int nrhs) { return line_warps(g, nrhs) < 4 * kSMs; }
 template <typename R>
 inline int line_threads(const LineArgs<R>& a) {
   return few_lines(a.g, a.nrhs) ? 32 : kLineThreads;

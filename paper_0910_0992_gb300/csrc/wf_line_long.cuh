@@ -12,7 +12,6 @@ void launch_line_long(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s
   if (a.g.n <= NMAX || a.g.n > NMAX_LONG || a.h16) throw Error(1, "long-line kernel: unsupported line layout");
   const int th = line_threads(a), b = line_blocks(a, th);
   constexpr int HOP = std::is_same<R, double>::value ? SRC_LOAD : SRC_HOP;  // as in launch_line
-  constexpr int ANY = std::is_same<R, double>::value ? SRC_LOAD : -1;
 #define WF_KL(AXV, SRCV, OPUV, OPLV) k_line<R, AXV, SRCV, OPUV, OPLV, false, NMAX_LONG><<<b, th, 0, s>>>(a)
   if (axial) {
     switch (kind) {
@@ -23,7 +22,7 @@ void launch_line_long(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s
         if (a.src == SRC_LOAD)
           WF_KL(true, SRC_LOAD, -1, -1);
         else
-          WF_KL(true, ANY, -1, -1);
+          WF_KL(true, HOP, -1, -1);
         break;
     }
   } else {
@@ -35,7 +34,7 @@ void launch_line_long(const LineArgs<R>& a, int kind, bool axial, cudaStream_t s
         if (a.src == SRC_LOAD)
           WF_KL(false, SRC_LOAD, -1, -1);
         else
-          WF_KL(false, ANY, -1, -1);
+          WF_KL(false, HOP, -1, -1);
         break;
     }
   }

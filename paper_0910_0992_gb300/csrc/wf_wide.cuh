@@ -393,11 +393,6 @@ constexpr int kWarpStage = 2 * kStageElems;  // a warp's shared memory: its stag
                                              // the transpose (384 elements, in the first stage) and
                                              // K-c's post-axpy operand (384, in the second)
 
-__device__ __forceinline__ void stage_copy(Cx<float>* dst, const Cx<float>* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<unsigned>(__cvta_generic_to_shared(dst))),
-               "l"(__cvta_generic_to_global(src))
-               : "memory");
-}
 
 template <class FreeStage>
 __device__ __forceinline__ void hop_site_staged(Vec3<float> (&h)[4], const LineArgs<float>& A, int rhs, int l,
@@ -421,9 +416,9 @@ __device__ __forceinline__ void hop_site_staged(Vec3<float> (&h)[4], const LineA
     Cx<R>* st = stage + (d & 1) * kStageElems + 2 * lane;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      stage_copy(st + 64 * i, u + 2 * i * tp);
-      stage_copy(st + 64 * (3 + i), v + 2 * i * tp);
-      stage_copy(st + 64 * (6 + i), lk + 2 * i * tp);
+      cp_async16(st + 64 * i, u + 2 * i * tp);
+      cp_async16(st + 64 * (3 + i), v + 2 * i * tp);
+      cp_async16(st + 64 * (6 + i), lk + 2 * i * tp);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
