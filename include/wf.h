@@ -30,6 +30,12 @@
  *   in-place apply). The library never keeps a caller pointer after a call returns.
  * Streams: all device work is ordered on the handle's stream (wf_set_stream); every call
  *   returns only when its results are complete (calls are synchronous for status).
+ * Accuracy: FP64 operators keep FP64 arithmetic's accuracy for every spin and colour of their results,
+ *   however far the components of a field are apart. The FP64 hops and frame rotations run as sums of
+ *   64-bit integers where those are as accurate (error of a result component against the sum of the
+ *   absolute values of its own terms), and in FP64 arithmetic elsewhere; environment WF_FX=0, or a device
+ *   without room for the integer copy of the spatial links (432 bytes per site, formed by the first FP64
+ *   operator on a loaded field), selects FP64 arithmetic for all hops.
  * Errors: every int-returning call returns WF_OK or one of the codes below and records a
  *   message readable with wf_last_error. No C++ exception crosses the ABI.
  */

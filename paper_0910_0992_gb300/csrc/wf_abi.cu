@@ -417,10 +417,10 @@ static wf_handle::HopTune tune_hops(wf_handle* h, const LineArgs<float>& ab, con
   for (int b = 2; b <= 12 && b <= h->g.L; ++b)
     if (h->g.L % b == 0) rows.push_back(b);
   if (rows.empty()) rows.push_back(h->g.by);
-  // 128-slot lines: one thread per site with staged operands alone. It was the fastest at every one of 54
-  // sizes (L 4 to 24, T 100 to 128, 1 to 12 sources; K-b + K-c against the next, bulk-fed stages: 16 : 20 us on
-  // 4^3 x 128 with one source, 163 : 178 on 24^3 x 128, 1324 : 1697 with twelve), and timing the
-  // others too took 250 ms of a handle's first solve of the last of these. Other lines: one thread
+  // 128-slot lines: one thread per site with staged operands alone. It was the fastest at every one of 45
+  // sizes (L 4 to 24, T 97 to 128, 1 to 12 sources; K-b + K-c against the next, bulk-fed stages: 17 : 20 us on
+  // 4^3 x 128 with one source, 162 : 179 on 24^3 x 128, 1326 : 1697 with twelve; least 19.4 : 20.1, 8^3 x 97), and
+  // timing the others too took 250 ms of a handle's first solve of the last of these. Other lines: one thread
   // per site, its operands in registers, against n sites per lane.
   const bool staged = wide_supported(h->g) && h->g.tp == 128 && h->g.n == 4;
   std::vector<wf_handle::HopTune> cands;

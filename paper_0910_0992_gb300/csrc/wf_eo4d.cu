@@ -209,7 +209,7 @@ struct EoDir {
 };
 
 // The dslash in FP64, spatial hops in block fixed point (wf_fixed.cuh); sites, arguments and results of
-// k_dslash4. 16^3 x 96, 4 sources: 1.16 ms with every operation in FP64, 0.42 ms so.
+// k_dslash4. 16^3 x 96, 4 sources: 1.16 ms with every operation in FP64, 0.47 ms so.
 template <bool AX, int S>
 __global__ void __launch_bounds__(FxShape<S>::threads, FxShape<S>::blocks) k_dslash4_fx(const EoArgs<double> A) {
   grid_dep();

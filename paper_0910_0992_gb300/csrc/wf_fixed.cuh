@@ -2,7 +2,7 @@
 //
 // GB300 issues two FP64 multiply-adds per clock and SM, but 64 32 x 32 -> 64-bit integer ones: the 648
 // FP64 operations of a spatial hop cost 324 clocks per site and SM, the same hop in 64-bit fixed point
-// about 90 (M, both parities, 24^3 x 128, 12 sources: 30.4 -> 8.9 ms; 12^3 x 48, 4 sources: 548 -> 188
+// about 100 (M, both parities, 24^3 x 128, 12 sources: 30.4 -> 9.7 ms; 12^3 x 48, 4 sources: 548 -> 209
 // us). The direction d of a site's stencil is a half-spinor of 12 real numbers times one SU(3) link, and
 //   * a direction makes two result spins of each pair of the neighbour's spins (axes x, y: 0 and 3 of
 //     spins 0 and 3, 1 and 2 of 1 and 2; z: 0 and 2, 1 and 3). Every result spin r has an exponent E_r,
@@ -421,8 +421,8 @@ __device__ __forceinline__ void hop_fx(const Dir& dir, int cs, int ls, bool site
 // Launch shape of a hop over `sites`: run(S, blocks, threads, dynamic shared memory) with the directions
 // split over as many warps S (std::integral_constant) as still leaves every CTA resident at once; the
 // chain of six spinor and link fetches is what bounds few sites. The Wilson matrix on one parity, us with
-// S = 1, 2, 3, 6 (32-site warps): 16 warps 28, 22, 20, 17; 256 27, 21, 19, 17; 512 27, 23, 23, 29;
-// 768 34, 27, 34, 40; 1024 33, 32, 37, 49; 1536 42, 44, 49, 68.
+// S = 1, 2, 3, 6 (32-site warps): 16 warps 30, 23, 21, 17; 256 28, 22, 21, 18; 512 29, 25, 23, 30;
+// 768 36, 29, 35, 42; 1024 36, 34, 39, 52; 1536 45, 48, 52, 72.
 template <class Run>
 inline void fx_launch(size_t sites, Run&& run) {
   const size_t warps = (sites + 31) / 32;

@@ -380,8 +380,9 @@ __device__ __forceinline__ Cx<R> pair_sum(Cx<R> a) {
 constexpr int kTMax = 256;     // longest time line
 constexpr int kQMaxWarps = 4;  // sources (warps) of a CTA of k_qinv_line
 // Ring of k_qinv_line: CS time slices per chunk, NST chunks (NST - 1 in flight)
-// (16^3 x 128, us with one / twelve sources: FP32 8 x 2 136 / 1013, 4 x 3 145 / 1118, 4 x 4 139 / 1115,
-// 8 x 3 152 / 1184, 4 x 2 166 / 1127; FP64 2 x 2 1408 / 14898, 4 x 2 1320 / 16411, 2 x 3 1361 / 17273)
+// (16^3 x 128, us with one / twelve sources: FP32 8 x 2 131 / 997, 4 x 3 139 / 1103, 4 x 4 134 / 1108,
+// 8 x 3 152 / 1181, 4 x 2 161 / 1113, 16 x 2 169 / 1099; FP64 2 x 2 1238 / 12571, 1 x 2 1033 / 12882, 4 x 2
+// 1151 / 14793, 2 x 3 1186 / 15537: the fastest for many sources, whose solves are the long ones)
 template <typename R>
 struct QRing {
   static constexpr int CS = sizeof(R) == 8 ? 2 : 8;
@@ -415,9 +416,9 @@ __device__ __forceinline__ void copy_pieces(void* dst, const void* src, int n) {
 // publishes a chunk and frees the one before it.
 // FP32 is bound by DRAM (every block entry of the forward sweep and of Z once, the P_- columns again
 // in the backward sweep: 2880 B per site, and 192 B per source), FP64 by the FP64 pipe (78 warp
-// instructions per line and slice). Measured on 16^3 x 128, FP32 136 us with one source
-// (755 MB of block entries: 0.82 of the copy bandwidth) and 1.01 ms with twelve (the sources' reads of
-// the shared blocks bound it), FP64 1.24 and 12.6 ms. The form before (16-lane groups
+// instructions per line and slice). Measured on 16^3 x 128, FP32 131 us with one source
+// (713 MB of DRAM traffic: 0.80 of the copy bandwidth) and 1.00 ms with twelve (the sources' reads of
+// the shared blocks: the L1's data pipe is 85 % busy, DRAM 15 %), FP64 1.24 and 12.6 ms. The form before (16-lane groups
 // copying their own rows, vectors through global memory in 8-byte elements a component apart) was
 // bound by the L1's tag stage: FP32 0.44 ms with one source and 2.33 ms with twelve, FP64 1.47 and
 // 13.8 ms.

@@ -40,12 +40,12 @@ __device__ __forceinline__ void site_coords(const Geom& g, size_t site, int& x, 
 //
 // The rotation's 144 multiply-adds per site would bound these kernels (GB300: two FP64 FMAs per clock
 // and SM): FP64 fields rotate in fixed point (rotate3_fx; full field of 24^3 x 128 x
-// 12 sources, import 5.1 -> 2.3 ms, export 5.1 -> 2.9; 12^3 x 48 x 4 0.10 -> 0.056 and 0.066 ms), FP32 fields with
+// 12 sources, import 5.1 -> 2.5 ms, export 5.1 -> 2.9; 12^3 x 48 x 4 0.10 -> 0.063 and 0.069 ms), FP32 fields with
 // rotate3_split instead, whose products are exact FP32 ones (below). Spins one after another and six
 // CTAs per SM: the loads of one CTA overlap the arithmetic of the others (unrolled, at 4 CTAs per SM,
 // 1.4 times slower). Measured, one odd field of 24^3 x 128 x 12 sources to and from FP32 (3.1 GB,
-// 0.45 ms at the copy bandwidth): import 0.96 ms, export 0.99 ms; 6.39 and 4.34 ms with one thread
-// per spin, its scattered elements and the rotation in FP64. One source of 16^3 x 128: 43 and 37 us,
+// 0.45 ms at the copy bandwidth): import 1.01 ms, export 1.02 ms; 6.39 and 4.34 ms with one thread
+// per spin, its scattered elements and the rotation in FP64. One source of 16^3 x 128: 43 and 38 us,
 // from 88 and 86.
 // ----------------------------------------------------------------------------
 constexpr int kTileThreads = 128;

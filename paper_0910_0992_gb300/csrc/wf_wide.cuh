@@ -385,9 +385,9 @@ __device__ __forceinline__ void spin_solve4_full(Vec3<R> (&w)[4], int j, const C
 // stages leave room for 6 CTAs per SM. Measured on 24^3 x 128, K-b / K-c: 643 / 681 us with 12 sources
 // and 80 / 83 us with one (register-fed, 7 CTAs: 721 / 789 and 87 / 92; one stage emptied into
 // registers before the next copy, 7 CTAs: 705 / 738 and 86 / 86; two stages at 5 CTAs: 712 / 743 with
-// 12). K-c's 3.9 GB of DRAM traffic then run at 0.85 of the copy bandwidth; K-b is bound by issue
-// slots (0.69 busy) beside 0.52 of DRAM. Once the last direction's operands are in registers,
-// free_stage() runs.
+// 12). K-c's 3.9 GB of DRAM traffic then run at 0.85 of the copy bandwidth; K-b keeps the issue slots and
+// the L1's data pipe busiest (0.66 and 0.69 on 16^3 x 128 with 12 sources, beside 0.50 of DRAM). Once the
+// last direction's operands are in registers, free_stage() runs.
 constexpr int kStageElems = 18 * 32;  // elements of one stage of one warp
 constexpr int kWarpStage = 2 * kStageElems;  // a warp's shared memory: its stages, later its part of
                                              // the transpose (384 elements, in the first stage) and
