@@ -328,11 +328,11 @@ int wf_temporal_logdet(wf_handle_t* h, double* logdet, double* F);
 /* Autotuned configuration of the FP32 hop kernels of M-hat (no counterpart in the paper): the
  * first FP32 Schur apply of a handle for a given nrhs times the candidates (on 128-slot lines, T 97 to
  * 128, the tile heights of variant 1, there with its operands staged through shared memory; elsewhere
- * variants 1 and 2 over the tile heights) and keeps the fastest (environment WF_AUTOTUNE=0 at the first apply keeps the built-in choice; WF_HOP fixes one, see
- * the README). variant: 1 one thread per site, 2 n sites per lane, 3 bulk-copy-fed (shared-memory
- * stages filled by cp.async.bulk; 128-slot lines, WF_HOP only: slower than variant 1 at every measured
- * size); tile_rows: rows of y per traversal tile; ms: the chosen
- * candidate's K-b + K-c time over three runs (0 if fixed by WF_HOP). wf_hop_pipe_config gives the
+ * variants 1 and 2 over the tile heights) and keeps the fastest (environment WF_AUTOTUNE=0 at the first
+ * apply keeps the built-in choice; WF_HOP fixes one, see the README). variant: 1 one thread per site, 2 n
+ * sites per lane, 3 bulk-copy-fed (shared-memory stages filled by cp.async.bulk; 128-slot lines, WF_HOP
+ * only: slower than variant 1 at every measured size); tile_rows: rows of y per traversal tile; ms: the
+ * chosen candidate's K-b + K-c time over three runs (0 if fixed by WF_HOP). wf_hop_pipe_config gives the
  * bulk-fed kernels' sources per unit (1 or 2) and stages (2 to 4); both are 0 for variants 1 and 2.
  * Any output pointer may be null. WF_EINVAL if that nrhs has not been tuned (yet). */
 int wf_hop_config(wf_handle_t* h, int nrhs, int* variant, int* tile_rows, float* ms);
